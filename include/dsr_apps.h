@@ -42,7 +42,7 @@ int dsr_gol_workspace_bytes(int W, int H, size_t* out);
  * initial Alive objects inside the heap. */
 int dsr_gol_create(dsr_heap* heap, int W, int H, const void* alive0_dev, void* workspace_dev, void* stream,
                    dsr_gol** out);
-/* The first call captures one generation (its six launches) into a CUDA
+/* The first call captures one generation (its launches) into a CUDA
  * graph on a stream of its own; every generation is then one graph launch
  * on `stream`. Make the first call outside any stream capture. */
 int dsr_gol_step(dsr_gol* g, int n_gen, void* stream);
@@ -120,7 +120,7 @@ int dsr_wator_workspace_bytes(const dsr_heap* heap, int W, int H, size_t* out);
 int dsr_wator_create(dsr_heap* heap, const dsr_wator_params* p, const void* kind0_dev, void* workspace_dev,
                      void* stream, dsr_wator** out);
 /* Advances n_steps steps on `stream` (each step: F1, F2, S0, S1, S2 as
- * do-alls). A step is replayed from a CUDA graph of its 8 launches that the
+ * do-alls). A step is replayed from a CUDA graph of its launches that the
  * handle captures on first use on a private stream (one for untimed steps,
  * one for the current dsr_wator_phase_timing / _phase_select setting, which
  * is captured when that setting is made); while `stream` is itself being

@@ -70,7 +70,7 @@ struct dsr_dev_heap {
     uint32_t* inject;     /* slow-path allocations left to fail (fault injection) */
     uint32_t* R_bid;      /* do-all block list: block ids */
     dsr_u64* R_mask;      /* do-all block list: occupied-slot snapshot */
-    uint32_t* R_count;    /* entries in R (zero between do-alls) */
+    uint32_t* R_count;    /* entries in R (zero between do-alls); R_count[2]: entries at R's back (application steps) */
     uint32_t* R_done;     /* CTAs of the current method kernel that finished */
     dsr_u64* ctr;         /* [DSR_CTR_SLOTS][DSR_CTR_COUNT] event counters, one row per SM */
     uint32_t* slow;       /* [DSR_MAX_TYPES] slow-path block initialisations in flight */
@@ -210,15 +210,15 @@ __device__ __forceinline__ unsigned dsr_hb_shift(const dsr_hbm& b) {
     return SH ? SH : b.shift;
 }
 
-/* Set bit pos of level l. With retry == false this is try_set: it fails if
+/* Set bit pos of level l (l0, 0 for a block's own bit). With retry == false this is try_set: it fails if
  * the bit is already set. With retry == true it is set(pos): it retries until
  * its own atomicOr changed the bit. If the container was empty before, this
  * thread owes the nested bit, which it sets with set() (never try_set). */
 template <unsigned SH>
-__device__ __forceinline__ bool dsr_hb_set_t(const dsr_hbm& b, dsr_u64 pos, bool retry, uint32_t* err) {
+__device__ __forceinline__ bool dsr_hb_set_t(const dsr_hbm& b, dsr_u64 pos, bool retry, uint32_t* err, int l0 = 0) {
     const unsigned sh = dsr_hb_shift<SH>(b);
     const dsr_u64 lo = (1ull << sh) - 1;
-    for (int l = 0; l < b.n_levels; ++l) {
+    for (int l = l0; l < b.n_levels; ++l) {
         dsr_u64* w = b.lvl[l] + (pos >> sh);
         const dsr_u64 m = 1ull << (pos & lo);
         dsr_u64 prev;
@@ -243,10 +243,10 @@ __device__ __forceinline__ bool dsr_hb_set_t(const dsr_hbm& b, dsr_u64 pos, bool
  * otherwise. If this call cleared the last set bit of its container
  * (popc(prev) == 1) it clears the nested bit with clear(). */
 template <unsigned SH>
-__device__ __forceinline__ bool dsr_hb_clear_t(const dsr_hbm& b, dsr_u64 pos, bool retry, uint32_t* err) {
+__device__ __forceinline__ bool dsr_hb_clear_t(const dsr_hbm& b, dsr_u64 pos, bool retry, uint32_t* err, int l0 = 0) {
     const unsigned sh = dsr_hb_shift<SH>(b);
     const dsr_u64 lo = (1ull << sh) - 1;
-    for (int l = 0; l < b.n_levels; ++l) {
+    for (int l = l0; l < b.n_levels; ++l) {
         dsr_u64* w = b.lvl[l] + (pos >> sh);
         const dsr_u64 m = 1ull << (pos & lo);
         dsr_u64 prev;
@@ -525,13 +525,16 @@ __device__ __forceinline__ dsr_u64 dsr_heap_key(const dsr_dev_heap& H) {
  * by shuffle. Returns DSR_NULL (and sets DSR_ERR_OOM or DSR_ERR_RETRY) on
  * failure. The new object's fields are not initialised. `near` (optional):
  * an object of the same heap whose block the leader tries first, before
- * searching the bitmaps (the leader's own hint counts for its group), for
- * example the parent of a newborn or an object just deleted; a hint only,
- * any handle of the heap or DSR_NULL is allowed. */
-__device__ inline dsr_ref dsr_new(const dsr_dev_heap& H, int T, dsr_ref near = DSR_NULL) {
+ * searching the bitmaps, for example the parent of a newborn or an object just
+ * deleted; a hint only, any handle of the heap or DSR_NULL is allowed. Lanes
+ * with hints in different blocks have leaders of their own, which try their
+ * blocks side by side. */
+template <bool HINT>
+__device__ inline dsr_ref dsr_new_t(const dsr_dev_heap& H, int T, dsr_ref near) {
     const unsigned act = __activemask();
-    const unsigned peers = __match_any_sync(act, dsr_heap_key(H) | (dsr_u64)T);
     const unsigned lane = dsr_lane();
+    unsigned peers = __match_any_sync(act, dsr_heap_key(H) | (dsr_u64)T);
+    if (HINT) peers &= __match_any_sync(act, near >> 6);
     const int leader = __ffs(peers) - 1;
     const int rank = __popc(peers & ((1u << lane) - 1));
     const int need = __popc(peers);
@@ -549,8 +552,9 @@ __device__ inline dsr_ref dsr_new(const dsr_dev_heap& H, int T, dsr_ref near = D
             // one. A group still wanting many slots after a round that
             // searched takes a fresh block rather than walking partly
             // filled ones one by one.
-            const long long nb = round == 0 && near != DSR_NULL && (near >> 6) < H.M ? (long long)(near >> 6) : -1;
-            const bool fresh = DSR_FRESH_REST > 0 && served > 0 && round > (near != DSR_NULL ? 1 : 0) &&
+            const bool hinted = HINT && near != DSR_NULL;
+            const long long nb = round == 0 && hinted && (near >> 6) < H.M ? (long long)(near >> 6) : -1;
+            const bool fresh = DSR_FRESH_REST > 0 && served > 0 && round > (hinted ? 1 : 0) &&
                                need - served >= DSR_FRESH_REST;
             const dsr_grab g = dsr_reserve(H, T, need - served, hint + (unsigned)served, fresh, nb);
             bid = g.bid;
@@ -570,7 +574,10 @@ __device__ inline dsr_ref dsr_new(const dsr_dev_heap& H, int T, dsr_ref near = D
     }
     return mine;
 }
-
+__device__ __forceinline__ dsr_ref dsr_new(const dsr_dev_heap& H, int T) { return dsr_new_t<false>(H, T, DSR_NULL); }
+__device__ __forceinline__ dsr_ref dsr_new(const dsr_dev_heap& H, int T, dsr_ref near) {
+    return dsr_new_t<true>(H, T, near);
+}
 /* delete: callable by any subset of a warp's lanes, with any mix of heaps.
  * Lanes deleting objects of the same block of the same heap are combined
  * into one atomicOr by a leader. DSR_NULL is ignored; a handle outside the
@@ -613,7 +620,8 @@ __device__ __forceinline__ F* dsr_field(const dsr_dev_heap& H, int T, dsr_ref r,
     if (!dsr_check((r >> 6) < H.M && (r & 63) < H.cap[T], H.err, H.dbg, 11, r))
         return reinterpret_cast<F*>(H.dbg + 1);
 #endif
-    return reinterpret_cast<F*>(H.data + (r >> 6) * H.block_bytes + H.foff[T][f]) + (r & 63);
+    // block ids are below 2^32: a 32 x 32-bit multiply gives the block's offset
+    return reinterpret_cast<F*>(H.data + (dsr_u64)(uint32_t)(r >> 6) * H.block_bytes + H.foff[T][f]) + (r & 63);
 }
 
 /* ------------------------------------------------------------------------ */

@@ -1,7 +1,7 @@
 // Game of life as an SMMO program (Fig. 6c): three do-alls per generation
 // over Cell and Alive objects. Rules: B3/S23 on a torus, Moore neighbourhood.
 #include "dsr_apps.h"
-#include "dsr_internal.cuh"
+#include "dsr_steps.cuh"
 
 namespace {
 enum { CELL = 0, ALIVE = 1 };
@@ -13,83 +13,156 @@ struct GolArgs {
     int32_t W, H;
 };
 
-// (i) do-all Cell: number of alive cells among the 8 neighbours.
+// (i) Cell: number of alive cells among the 8 neighbours.
+__device__ __forceinline__ void count_cell(const dsr_dev_heap& H, const GolArgs& a, dsr_ref self) {
+    const int idx = *dsr_field<int32_t>(H, CELL, self, C_IDX);
+    const int y = idx / a.W, x = idx - y * a.W;
+    const int xw = x == 0 ? a.W - 1 : x - 1, xe = x == a.W - 1 ? 0 : x + 1;
+    const dsr_ref* mid = a.cell_ref + (idx - x);
+    const dsr_ref* up = a.cell_ref + (dsr_u64)(y == 0 ? a.H - 1 : y - 1) * a.W;
+    const dsr_ref* down = a.cell_ref + (dsr_u64)(y == a.H - 1 ? 0 : y + 1) * a.W;
+    const dsr_ref c[8] = {up[xw], up[x], up[xe], mid[xw], mid[xe], down[xw], down[x], down[xe]};
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (c[k] != DSR_NULL) n += *dsr_field<int32_t>(H, CELL, c[k], C_ALIVE);
+    *dsr_field<int32_t>(H, CELL, self, C_COUNT) = n;
+}
+
+// (ii) Alive: death when the cell's count is not 2 or 3.
+__device__ __forceinline__ void die(const dsr_dev_heap& H, const GolArgs& a, dsr_ref self) {
+    const int x = *dsr_field<int32_t>(H, ALIVE, self, A_X);
+    const int y = *dsr_field<int32_t>(H, ALIVE, self, A_Y);
+    const dsr_ref c = a.cell_ref[y * a.W + x];
+    if (c == DSR_NULL) return;
+    const int n = *dsr_field<int32_t>(H, CELL, c, C_COUNT);
+    if (n != 2 && n != 3) {
+        *dsr_field<int32_t>(H, CELL, c, C_ALIVE) = 0;
+        dsr_delete(H, self);
+    }
+}
+
+// (iii) Cell: birth of a dead cell with exactly 3 alive neighbours: true for
+// one, which is alive from here on and has the grid index *idx.
+__device__ __forceinline__ bool birth(const dsr_dev_heap& H, dsr_ref self, int* idx) {
+    int32_t* alive = dsr_field<int32_t>(H, CELL, self, C_ALIVE);
+    const int was = *alive, n = *dsr_field<int32_t>(H, CELL, self, C_COUNT);
+    if (was || n != 3) return false;
+    *alive = 1;
+    *idx = *dsr_field<int32_t>(H, CELL, self, C_IDX);
+    return true;
+}
+__device__ __forceinline__ void gol_born(const dsr_dev_heap& H, const GolArgs& a, int idx, dsr_ref r) {
+    if (r == DSR_NULL) return;
+    *dsr_field<int32_t>(H, ALIVE, r, A_X) = idx % a.W;
+    *dsr_field<int32_t>(H, ALIVE, r, A_Y) = idx / a.W;
+}
+
+// ---- list do-alls (dsr_parallel_do) ----------------------------------------
 struct MCount {
     typedef GolArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref self) {
-        const int idx = *dsr_field<int32_t>(H, CELL, self, C_IDX);
-        const int x = idx % a.W, y = idx / a.W;
-        int n = 0;
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int ny = y + dy < 0 ? y + dy + a.H : (y + dy >= a.H ? y + dy - a.H : y + dy);
-#pragma unroll
-            for (int dx = -1; dx <= 1; ++dx) {
-                if (dx == 0 && dy == 0) continue;
-                const int nx = x + dx < 0 ? x + dx + a.W : (x + dx >= a.W ? x + dx - a.W : x + dx);
-                const dsr_ref c = a.cell_ref[ny * a.W + nx];
-                if (c != DSR_NULL) n += *dsr_field<int32_t>(H, CELL, c, C_ALIVE);
-            }
-        }
-        *dsr_field<int32_t>(H, CELL, self, C_COUNT) = n;
-    }
+    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref self) { count_cell(H, a, self); }
 };
-
-// (ii) do-all Alive: death when the cell's count is not 2 or 3.
 struct MDie {
     typedef GolArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref self) {
-        const int x = *dsr_field<int32_t>(H, ALIVE, self, A_X);
-        const int y = *dsr_field<int32_t>(H, ALIVE, self, A_Y);
-        const dsr_ref c = a.cell_ref[y * a.W + x];
-        if (c == DSR_NULL) return;
-        const int n = *dsr_field<int32_t>(H, CELL, c, C_COUNT);
-        if (n != 2 && n != 3) {
-            *dsr_field<int32_t>(H, CELL, c, C_ALIVE) = 0;
-            dsr_delete(H, self);
-        }
-    }
+    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref self) { die(H, a, self); }
 };
-
-// (iii) do-all Cell: birth of a dead cell with exactly 3 alive neighbours.
 struct MBirth {
     typedef GolArgs Args;
     static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref self) {
-        int32_t* alive = dsr_field<int32_t>(H, CELL, self, C_ALIVE);
-        if (*alive || *dsr_field<int32_t>(H, CELL, self, C_COUNT) != 3) return;
-        *alive = 1;
-        const int idx = *dsr_field<int32_t>(H, CELL, self, C_IDX);
-        const dsr_ref r = dsr_new(H, ALIVE);
-        if (r == DSR_NULL) return;
-        *dsr_field<int32_t>(H, ALIVE, r, A_X) = idx % a.W;
-        *dsr_field<int32_t>(H, ALIVE, r, A_Y) = idx / a.W;
+        int idx;
+        if (birth(H, self, &idx)) gol_born(H, a, idx, dsr_new(H, ALIVE));
     }
 };
 
-// One thread per cell: create the Cell and, where alive, its Alive object.
-__global__ void k_gol_init(const __grid_constant__ dsr_dev_heap H, const uint8_t* alive0, dsr_ref* cell_ref,
-                           int W, int Hh) {
-    const int n = W * Hh;
-    const int n32 = (n + 31) & ~31;  // warp-uniform trip count
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
-        __syncwarp();  // whole-warp groups for dsr_new
-        if (i >= n) continue;
-        const int alive = alive0[i] ? 1 : 0;
-        const dsr_ref c = dsr_new(H, CELL);
-        cell_ref[i] = c;
-        if (c != DSR_NULL) {
-            *dsr_field<int32_t>(H, CELL, c, C_ALIVE) = alive;
-            *dsr_field<int32_t>(H, CELL, c, C_COUNT) = 0;
-            *dsr_field<int32_t>(H, CELL, c, C_IDX) = i;
-        }
-        if (alive) {
-            const dsr_ref r = dsr_new(H, ALIVE);
-            if (r != DSR_NULL) {
-                *dsr_field<int32_t>(H, ALIVE, r, A_X) = i % W;
-                *dsr_field<int32_t>(H, ALIVE, r, A_Y) = i / W;
-            }
-        }
+// ---- the plain and the batched generation (dsr_steps.cuh) ------------------
+// A: GolArgs (plain form), or GolBatchArgs: heap index h of a group is the
+// instance slot, table[h] its view (cell_ref == nullptr: unused slot).
+struct GolBatchArgs {
+    const GolArgs* table;
+};
+__device__ __forceinline__ const GolArgs& inst_of(const GolArgs& a, uint32_t) { return a; }
+__device__ __forceinline__ const GolArgs& inst_of(const GolBatchArgs& a, uint32_t h) { return a.table[h]; }
+
+struct NoCtx {};
+template <class A>
+struct GolMethod {
+    typedef A Args;
+    typedef GolArgs Inst;
+    typedef NoCtx Ctx;
+    typedef dsr_no_acc Acc;
+    enum { kDefers = DSR_NOTHING, kMarks = 0 };
+    static __device__ __forceinline__ const GolArgs& inst(const A& a, uint32_t h) { return inst_of(a, h); }
+    static __device__ __forceinline__ NoCtx begin(const GolArgs&) { return {}; }
+    static __device__ __forceinline__ void flush(const dsr_dev_heap&, const GolArgs&, dsr_no_acc) {}
+};
+template <class A>
+struct DCount : GolMethod<A> {
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const GolArgs& a, NoCtx, dsr_ref self,
+                                                   dsr_later&, dsr_no_acc&) {
+        count_cell(H, a, self);
+        return 0;
     }
+};
+template <class A>
+struct DDie : GolMethod<A> {
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const GolArgs& a, NoCtx, dsr_ref self,
+                                                   dsr_later&, dsr_no_acc&) {
+        die(H, a, self);
+        return 0;
+    }
+};
+template <class A>
+struct DBirth : GolMethod<A> {
+    enum { kDefers = ALIVE };
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const GolArgs& a, NoCtx, dsr_ref self,
+                                                   dsr_later& later, dsr_no_acc&) {
+        int idx;
+        if (birth(H, self, &idx)) {
+            if (later.on)
+                later.push((dsr_u64)idx);
+            else
+                gol_born(H, a, idx, dsr_new(H, ALIVE));
+        }
+        return 0;
+    }
+    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const GolArgs& a, NoCtx, dsr_u64 idx, dsr_ref r,
+                                                dsr_no_acc&) {
+        gol_born(H, a, (int)idx, r);
+    }
+};
+// One scan lists both types. A birth and a death never meet: a cell that
+// dies has not 3 alive neighbours, and new Alive objects are in no list.
+constexpr dsr_phase kCells{CELL, 0}, kAlive{ALIVE, 1};
+
+// One thread per cell: create the Cell and, where alive, its Alive object.
+__global__ void __launch_bounds__(DSR_BULK_THREADS)
+    k_gol_init(const __grid_constant__ dsr_dev_heap H, const uint8_t* alive0, dsr_ref* cell_ref, int W, int Hh,
+               int rows) {
+    __shared__ dsr_bulk_smem<2> sm;
+    const int types[2] = {CELL, ALIVE};
+    dsr_bulk_create(
+        H, (dsr_u64)W * Hh, rows, types, sm, [&](dsr_u64 i) { return alive0[i] ? 3u : 1u; },
+        [&](dsr_u64 i, unsigned kind, const dsr_ref (&ref)[2]) {
+            cell_ref[i] = ref[0];
+            if (ref[0] != DSR_NULL) {
+                *dsr_field<int32_t>(H, CELL, ref[0], C_ALIVE) = kind >> 1;
+                *dsr_field<int32_t>(H, CELL, ref[0], C_COUNT) = 0;
+                *dsr_field<int32_t>(H, CELL, ref[0], C_IDX) = (int32_t)i;
+            }
+            if (ref[1] != DSR_NULL) {
+                *dsr_field<int32_t>(H, ALIVE, ref[1], A_X) = (int32_t)((uint32_t)i % (uint32_t)W);
+                *dsr_field<int32_t>(H, ALIVE, ref[1], A_Y) = (int32_t)((uint32_t)i / (uint32_t)W);
+            }
+        });
+}
+
+int launch_init(const dsr_heap* heap, int W, int H, const void* alive0_dev, void* cell_ref_dev, cudaStream_t s) {
+    const dsr_u64 n = (dsr_u64)W * H;
+    const int rows = dsr__bulk_rows(n, heap->sm_count);
+    k_gol_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
+        heap->dev, static_cast<const uint8_t*>(alive0_dev), static_cast<dsr_ref*>(cell_ref_dev), W, H, rows);
+    return dsr__check_launch("k_gol_init");
 }
 
 const int kCellFields[3] = {4, 4, 4};
@@ -110,7 +183,7 @@ struct dsr_gol {
     dsr_heap* heap;
     GolArgs args;
     cudaStream_t capture = nullptr;   // stream the generation is captured on
-    cudaGraphExec_t exec = nullptr;   // one generation (6 launches) as a graph
+    cudaGraphExec_t exec = nullptr;   // one generation as a graph
 };
 
 extern "C" int dsr_gol_types(dsr_type_desc* out) {
@@ -134,12 +207,7 @@ extern "C" int dsr_gol_create(dsr_heap* heap, int W, int H, const void* alive0_d
     dsr_gol* g = new dsr_gol;
     g->heap = heap;
     g->args = GolArgs{static_cast<const dsr_ref*>(workspace_dev), W, H};
-    const int n = W * H;
-    int ctas = (n + 255) / 256;
-    if (ctas > heap->sm_count * 8) ctas = heap->sm_count * 8;
-    k_gol_init<<<ctas, 256, 0, dsr__stream(stream)>>>(heap->dev, static_cast<const uint8_t*>(alive0_dev),
-                                                       static_cast<dsr_ref*>(workspace_dev), W, H);
-    int rc = dsr__check_launch("k_gol_init");
+    int rc = launch_init(heap, W, H, alive0_dev, workspace_dev, dsr__stream(stream));
     if (rc) {
         delete g;
         return rc;
@@ -149,13 +217,14 @@ extern "C" int dsr_gol_create(dsr_heap* heap, int W, int H, const void* alive0_d
 }
 
 static int issue_generation(dsr_gol* g, cudaStream_t s) {
-    int rc = dsr__doall<MCount>(g->heap, CELL, g->args, s);
-    if (!rc) rc = dsr__doall<MDie>(g->heap, ALIVE, g->args, s);
-    if (!rc) rc = dsr__doall<MBirth>(g->heap, CELL, g->args, s);
+    typedef GolArgs A;
+    dsr__list_types(g->heap, CELL, ALIVE, 2, 1, s);
+    int rc = dsr__step<DCount<A>>(g->heap, kCells, kCells, g->args, s);
+    if (!rc) rc = dsr__step<DBirth<A>, DDie<A>, true>(g->heap, kCells, kAlive, g->args, s);
     return rc;
 }
 
-// A generation's six launches take a few microseconds each on a 64 x 64
+// A generation's three launches take a few microseconds each on a 64 x 64
 // board, so the generation is captured once into a CUDA graph (its kernel
 // arguments never change) and replayed: one launch per generation.
 extern "C" int dsr_gol_step(dsr_gol* g, int n_gen, void* stream) {
@@ -223,30 +292,8 @@ int dsr__gol_method(dsr_heap* h, int type, int method, const void* args, size_t 
 // ===========================================================================
 // batched form: many game-of-life instances in one heap group
 // ===========================================================================
-#include "dsr_group.cuh"
 
 namespace {
-struct GolBatchArgs {
-    const GolArgs* table;  // slot -> instance view (cell_ref == nullptr: unused slot)
-};
-struct GCount {
-    typedef GolBatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int T, const Args& a, dsr_ref s, uint32_t h) {
-        MCount::run(H, T, a.table[h], s);
-    }
-};
-struct GDie {
-    typedef GolBatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int T, const Args& a, dsr_ref s, uint32_t h) {
-        MDie::run(H, T, a.table[h], s);
-    }
-};
-struct GBirth {
-    typedef GolBatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int T, const Args& a, dsr_ref s, uint32_t h) {
-        MBirth::run(H, T, a.table[h], s);
-    }
-};
 size_t gol_table_bytes(int n) { return ((size_t)n * sizeof(GolArgs) + 1023) / 1024 * 1024; }
 }  // namespace
 
@@ -333,12 +380,7 @@ extern "C" int dsr_gol_batch_add(dsr_gol_batch* b, int W, int H, uint64_t n_bloc
     int rc = dsr_group_add_heap(b->group, n_blocks, ws, stream, &slot, &heap, &extra);
     if (rc) return rc;
     cudaStream_t s = dsr__stream(stream);
-    const int n = W * H;
-    int ctas = (n + 255) / 256;
-    if (ctas > heap->sm_count * 8) ctas = heap->sm_count * 8;
-    k_gol_init<<<ctas, 256, 0, s>>>(heap->dev, static_cast<const uint8_t*>(alive0_dev), static_cast<dsr_ref*>(extra),
-                                    W, H);
-    rc = dsr__check_launch("k_gol_init");
+    rc = launch_init(heap, W, H, alive0_dev, extra, s);
     if (rc) return rc;
     b->table_h[slot] = GolArgs{static_cast<const dsr_ref*>(extra), W, H};
     cudaError_t e = cudaMemcpyAsync(b->table_d + slot, &b->table_h[slot], sizeof(GolArgs), cudaMemcpyHostToDevice, s);
@@ -362,7 +404,7 @@ extern "C" int dsr_gol_batch_remove(dsr_gol_batch* b, int inst) {
     return dsr_group_remove_heap(b->group, inst);
 }
 
-// One batched generation: three group do-alls (6 launches), captured into a
+// One batched generation (the launches of a plain one), captured into a
 // CUDA graph once per set of instances.
 static int ensure_gol_graph(dsr_gol_batch* b) {
     if (b->exec_epoch == b->group->epoch) return DSR_OK;
@@ -375,9 +417,10 @@ static int ensure_gol_graph(dsr_gol_batch* b) {
         return DSR_E_CUDA;
     }
     GolBatchArgs a{b->table_d};
-    int rc = dsr__group_doall<GCount>(b->group, CELL, a, b->capture);
-    if (!rc) rc = dsr__group_doall<GDie>(b->group, ALIVE, a, b->capture);
-    if (!rc) rc = dsr__group_doall<GBirth>(b->group, CELL, a, b->capture);
+    typedef GolBatchArgs A;
+    dsr__group_list_types(b->group, CELL, ALIVE, 2, 1, b->capture);
+    int rc = dsr__group_step<DCount<A>>(b->group, kCells, kCells, a, b->capture);
+    if (!rc) rc = dsr__group_step<DBirth<A>, DDie<A>, true>(b->group, kCells, kAlive, a, b->capture);
     e = cudaStreamEndCapture(b->capture, &graph);
     if (rc) {
         if (graph) cudaGraphDestroy(graph);

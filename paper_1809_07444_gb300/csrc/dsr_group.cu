@@ -4,7 +4,7 @@
 #include <new>
 #include <vector>
 
-#include "dsr_group.cuh"
+#include "dsr_steps.cuh"
 
 // ---------------------------------------------------------------------------
 // fused scan: as the single-heap scan, over chunks of 256 block ids of any
@@ -48,6 +48,69 @@ __global__ void __launch_bounds__(256) k_group_scan(const __grid_constant__ dsr_
         if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs * visits_mult);
         __syncthreads();
     }
+}
+
+// The lists of a batched step (dsr_steps.cuh): as k_list, over the chunks of
+// every heap.
+__global__ void __launch_bounds__(256) k_group_list(const __grid_constant__ dsr_group_dev G, int ta, int tb,
+                                                    unsigned mult_a, unsigned mult_b) {
+    __shared__ unsigned warp_n[2][8];
+    __shared__ unsigned run_base[2];
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint32_t c = blockIdx.x; c < G.n_chunks; c += gridDim.x) {
+        const uint32_t h = G.chunk_heap[c];
+        const bool hok = dsr_check(h < G.n_slots, G.err, G.dbg, 1, c);
+        const dsr_dev_heap& H = G.heaps[hok ? h : 0];
+        const dsr_u64 b = (dsr_u64)G.chunk_base[c] + threadIdx.x;
+        const unsigned fsh = H.free_bm.shift, flo = (1u << fsh) - 1;
+        bool in_a = false, in_b = false;
+        dsr_u64 obj = 0;
+        if (hok && b < H.M) {
+            const dsr_u64 wa = H.alloc_bm[ta].lvl[0][b >> fsh];
+            const dsr_u64 wb = tb >= 0 ? H.alloc_bm[tb].lvl[0][b >> fsh] : 0ull;
+            obj = H.obj[b];
+            in_a = (wa >> (b & flo)) & 1ull;
+            in_b = (wb >> (b & flo)) & 1ull;
+        }
+        const unsigned ba = __ballot_sync(0xFFFFFFFFu, in_a), bb = __ballot_sync(0xFFFFFFFFu, in_b);
+        if (lane == 0) warp_n[0][warp] = __popc(ba), warp_n[1][warp] = __popc(bb);
+        __syncthreads();
+        if (threadIdx.x < 2) {
+            unsigned total = 0;
+            for (int w = 0; w < 8; ++w) {
+                const unsigned n = warp_n[threadIdx.x][w];
+                warp_n[threadIdx.x][w] = total;
+                total += n;
+            }
+            run_base[threadIdx.x] = total ? atomicAdd(G.R_count + (threadIdx.x ? DSR_GROUP_LIST_BACK : 0), total) : 0;
+        }
+        __syncthreads();
+        unsigned objs = 0;
+        if (in_a || in_b) {
+            const int l = in_a ? 0 : 1;
+            const dsr_u64 live = H.valid[in_a ? ta : tb] & ~obj;
+            const dsr_u64 k = run_base[l] + warp_n[l][warp] + __popc((in_a ? ba : bb) & ((1u << lane) - 1));
+            if (dsr_check(k < G.R_cap, G.err, G.dbg, 2, k)) {
+                const dsr_u64 at = in_a ? k : G.R_cap - 1 - k;
+                G.R_heap[at] = h;
+                G.R_bid[at] = (uint32_t)b;
+                G.R_mask[at] = live;
+                objs = __popcll(live) * (in_a ? mult_a : mult_b);
+            }
+        }
+        objs = __reduce_add_sync(0xFFFFFFFFu, objs);
+        if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs);
+        __syncthreads();
+    }
+}
+
+void dsr__group_list_types(const dsr_group* g, int type_a, int type_b, unsigned mult_a, unsigned mult_b,
+                           cudaStream_t s) {
+    if (g->n_chunks == 0) return;
+    unsigned ctas = g->n_chunks;
+    const unsigned cap = (unsigned)g->sm_count * 8;
+    if (ctas > cap) ctas = cap;
+    k_group_list<<<ctas, 256, 0, s>>>(g->dev, type_a, type_b, mult_a, mult_b);
 }
 
 // First failed device check of the group (checked builds): err word and record.

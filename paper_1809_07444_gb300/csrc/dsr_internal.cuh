@@ -124,14 +124,24 @@ int dsr__nbody_method(dsr_heap* h, int type, int method, const void* args, size_
 
 // SplitMix64 finalizer and the object-state hash (same definition as the
 // dsr_heap_hash documentation).
-__device__ __forceinline__ dsr_u64 dsr_mix64(dsr_u64 z) {
+__host__ __device__ __forceinline__ dsr_u64 dsr_mix64(dsr_u64 z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
 }
 #define DSR_GAMMA 0x9E3779B97F4A7C15ull
-__device__ __forceinline__ dsr_u64 dsr_splitmix_at(dsr_u64 s, dsr_u64 n) { return dsr_mix64(s + (n + 1) * DSR_GAMMA); }
-// Counter-based draw keyed on (seed, stream, step, cell).
+__host__ __device__ __forceinline__ dsr_u64 dsr_splitmix_at(dsr_u64 s, dsr_u64 n) { return dsr_mix64(s + (n + 1) * DSR_GAMMA); }
+// Counter-based draw keyed on (seed, stream, step, cell): dsr_splitmix_at of
+// the step's key and the cell. The key is the same for every object of a
+// do-all, so it is computed once, not in every draw (two of its three rounds).
+__host__ __device__ __forceinline__ dsr_u64 dsr_rand_key(dsr_u64 seed, dsr_u64 stream, dsr_u64 step) {
+    return dsr_splitmix_at(dsr_splitmix_at(seed, stream), step);
+}
 __device__ __forceinline__ dsr_u64 dsr_rand(dsr_u64 seed, dsr_u64 stream, dsr_u64 step, dsr_u64 cell) {
-    return dsr_splitmix_at(dsr_splitmix_at(dsr_splitmix_at(seed, stream), step), cell);
+    return dsr_splitmix_at(dsr_rand_key(seed, stream, step), cell);
+}
+// r mod k for k in 1 .. 4. 2^32 = 1 (mod 3), so the two halves of r add up.
+__device__ __forceinline__ unsigned dsr_mod_upto4(dsr_u64 r, unsigned k) {
+    const unsigned m3 = ((unsigned)r % 3u + (unsigned)(r >> 32) % 3u) % 3u;
+    return k == 3 ? m3 : (unsigned)r & (k - 1u);
 }

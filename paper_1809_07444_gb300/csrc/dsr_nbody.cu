@@ -40,7 +40,7 @@
 // grows the same way over tens of steps.
 #include <cfloat>
 #include "dsr_apps.h"
-#include "dsr_internal.cuh"
+#include "dsr_bulk.cuh"
 
 #include <mutex>
 
@@ -930,19 +930,21 @@ __global__ void k_merge(const __grid_constant__ dsr_dev_heap H, const __grid_con
     if (dsr_doall_finish(H)) *a.ws.step += 1;
 }
 
-__global__ void k_nbody_init(const __grid_constant__ dsr_dev_heap H, const float* rows, int n) {
-    const int n32 = (n + 31) & ~31;  // warp-uniform trip count
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += gridDim.x * blockDim.x) {
-        __syncwarp();  // whole-warp groups for dsr_new
-        if (i >= n) continue;
-        const dsr_ref r = dsr_new(H, BODY);
-        if (r == DSR_NULL) continue;
-        *dsr_field<int32_t>(H, BODY, r, ID) = i;
-        for (int f = 0; f < 7; ++f) {
-            *fld(H, r, PX + f) = rows[7 * i + f];
-            *fld(H, r, PX + f + LO) = 0.f;
-        }
-    }
+__global__ void __launch_bounds__(DSR_BULK_THREADS)
+    k_nbody_init(const __grid_constant__ dsr_dev_heap H, const float* rows, int n, int bulk_rows) {
+    __shared__ dsr_bulk_smem<1> sm;
+    const int types[1] = {BODY};
+    dsr_bulk_create(
+        H, (dsr_u64)n, bulk_rows, types, sm, [](dsr_u64) { return 1u; },
+        [&](dsr_u64 i, unsigned, const dsr_ref (&ref)[1]) {
+            const dsr_ref r = ref[0];
+            if (r == DSR_NULL) return;
+            *dsr_field<int32_t>(H, BODY, r, ID) = (int32_t)i;
+            for (int f = 0; f < 7; ++f) {
+                *fld(H, r, PX + f) = rows[7 * i + f];
+                *fld(H, r, PX + f + LO) = 0.f;
+            }
+        });
 }
 
 const int kBodyFields[N_FIELDS] = {4, 4, 4, 4, 4, 4, 4, 4, 4, 4, 4, 4, 4, 4, 4};
@@ -1160,9 +1162,9 @@ extern "C" int dsr_nbody_create(dsr_heap* heap, const dsr_nbody_params* p, const
         delete nb;
         return DSR_E_CUDA;
     }
-    int ctas = (n_bodies + 255) / 256;
-    if (ctas > heap->sm_count * 8) ctas = heap->sm_count * 8;
-    k_nbody_init<<<ctas, 256, 0, s>>>(heap->dev, static_cast<const float*>(rows_dev), n_bodies);
+    const int rows = dsr__bulk_rows((dsr_u64)n_bodies, heap->sm_count);
+    k_nbody_init<<<dsr__bulk_grid((dsr_u64)n_bodies, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
+        heap->dev, static_cast<const float*>(rows_dev), n_bodies, rows);
     int rc = dsr__check_launch("k_nbody_init");
     if (rc) {
         delete nb;

@@ -26,7 +26,7 @@
 #include <climits>
 
 #include "dsr_apps.h"
-#include "dsr_internal.cuh"
+#include "dsr_bulk.cuh"
 
 namespace {
 enum { AGENT = 0 };
@@ -205,19 +205,21 @@ struct MReplace {
 
 // One thread per initial agent (agents0[i] = x, y, sugar, metabolism,
 // vision, age, max_age; distinct cells).
-__global__ void k_sugar_init(const __grid_constant__ dsr_dev_heap H, const int32_t* agents0, int64_t n_agents,
-                             SugarWs ws, int32_t W) {
-    const int64_t n32 = (n_agents + 31) & ~31ll;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += (int64_t)gridDim.x * blockDim.x) {
-        __syncwarp();
-        if (i >= n_agents) continue;
-        const int32_t* src = agents0 + 7 * i;
-        const dsr_ref r = dsr_new(H, AGENT);
-        if (r == DSR_NULL) continue;
-        for (int f = 0; f < 7; ++f) *fld(H, r, f) = src[f];
-        *fld(H, r, F_DEAD) = 0;
-        ws.cell[(int64_t)src[1] * W + src[0]] |= OCC;
-    }
+__global__ void __launch_bounds__(DSR_BULK_THREADS)
+    k_sugar_init(const __grid_constant__ dsr_dev_heap H, const int32_t* agents0, int64_t n_agents, SugarWs ws,
+                 int32_t W, int rows) {
+    __shared__ dsr_bulk_smem<1> sm;
+    const int types[1] = {AGENT};
+    dsr_bulk_create(
+        H, (dsr_u64)n_agents, rows, types, sm, [](dsr_u64) { return 1u; },
+        [&](dsr_u64 i, unsigned, const dsr_ref (&ref)[1]) {
+            const dsr_ref r = ref[0];
+            if (r == DSR_NULL) return;
+            const int32_t* src = agents0 + 7 * i;
+            for (int f = 0; f < 7; ++f) *fld(H, r, f) = src[f];
+            *fld(H, r, F_DEAD) = 0;
+            ws.cell[(int64_t)src[1] * W + src[0]] |= OCC;
+        });
 }
 
 // Cells from the capacities: unoccupied, never harvested.
@@ -317,10 +319,9 @@ extern "C" int dsr_sugarscape_create(dsr_heap* heap, const dsr_sugarscape_params
     const int ctas = heap->sm_count * 4;
     k_sugar_fill<<<ctas, 256, 0, s>>>(w.cell, static_cast<const uint8_t*>(cap_dev), n);
     if (n_agents) {
-        int64_t c2 = (n_agents + 255) / 256;
-        if (c2 > heap->sm_count * 8) c2 = heap->sm_count * 8;
-        k_sugar_init<<<(unsigned)c2, 256, 0, s>>>(heap->dev, static_cast<const int32_t*>(agents0_dev), n_agents, w,
-                                                    p->W);
+        const int rows = dsr__bulk_rows((dsr_u64)n_agents, heap->sm_count);
+        k_sugar_init<<<dsr__bulk_grid((dsr_u64)n_agents, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
+            heap->dev, static_cast<const int32_t*>(agents0_dev), n_agents, w, p->W, rows);
     }
     const int rc = dsr__check_launch("k_sugar_init");
     if (rc) {

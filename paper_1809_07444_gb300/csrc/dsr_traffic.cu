@@ -18,7 +18,7 @@
 // no car reads a cell another car writes: the do-all needs no atomics. After
 // the step `cur` is cleared and the grids swap.
 #include "dsr_apps.h"
-#include "dsr_internal.cuh"
+#include "dsr_bulk.cuh"
 
 namespace {
 enum { CAR = 0, SOURCE = 1 };
@@ -101,35 +101,42 @@ struct MSource {
     }
 };
 
-// One thread per cell: a Car where v0 >= 0, and on open roads a Source per
-// road (made by the thread of cell 0).
-__global__ void k_traffic_init(const __grid_constant__ dsr_dev_heap H, const int8_t* v0, uint8_t* cur,
-                               dsr_traffic_params p) {
+// One thread per cell: a Car where v0 >= 0.
+__global__ void __launch_bounds__(DSR_BULK_THREADS)
+    k_traffic_init(const __grid_constant__ dsr_dev_heap H, const int8_t* v0, uint8_t* cur, dsr_traffic_params p,
+                   int rows) {
+    __shared__ dsr_bulk_smem<1> sm;
+    const int types[1] = {CAR};
     const dsr_u64 n = (dsr_u64)p.R * p.L;
-    const dsr_u64 n32 = (n + 31) & ~31ull;  // warp-uniform trip count
-    for (dsr_u64 i = (dsr_u64)blockIdx.x * blockDim.x + threadIdx.x; i < n32; i += (dsr_u64)gridDim.x * blockDim.x) {
-        __syncwarp();  // whole-warp groups for dsr_new
-        if (i >= n) continue;
-        const int32_t road = (int32_t)(i / p.L), x = (int32_t)(i % p.L);
-        const int v = v0[i];
-        if (v >= 0) {
-            const dsr_ref c = dsr_new(H, CAR);
-            if (c != DSR_NULL) {
-                *fld(H, CAR, c, F_ROAD) = road;
-                *fld(H, CAR, c, F_X) = x;
-                *fld(H, CAR, c, F_V) = v < p.vmax ? v : p.vmax;
-                cur[i] = 1;
-            }
-        }
-        if (!p.periodic && x == 0) {
-            const dsr_ref s = dsr_new(H, SOURCE);
-            if (s != DSR_NULL) {
-                *fld(H, SOURCE, s, S_ROAD) = road;
-                *fld(H, SOURCE, s, S_ENTERED) = 0;
-                *fld(H, SOURCE, s, S_BLOCKED) = 0;
-            }
-        }
-    }
+    const bool small = n <= 0xFFFFFFFFull;  // 32-bit divisions are several times cheaper than 64-bit ones
+    dsr_bulk_create(
+        H, n, rows, types, sm, [&](dsr_u64 i) { return v0[i] >= 0 ? 1u : 0u; },
+        [&](dsr_u64 i, unsigned, const dsr_ref (&ref)[1]) {
+            const dsr_ref c = ref[0];
+            if (c == DSR_NULL) return;
+            const int v = v0[i];
+            const int32_t road = small ? (int32_t)((uint32_t)i / (uint32_t)p.L) : (int32_t)(i / p.L);
+            *fld(H, CAR, c, F_ROAD) = road;
+            *fld(H, CAR, c, F_X) = (int32_t)(i - (dsr_u64)road * p.L);
+            *fld(H, CAR, c, F_V) = v < p.vmax ? v : p.vmax;
+            cur[i] = 1;
+        });
+}
+
+// Open roads: one thread per road, its Source.
+__global__ void __launch_bounds__(DSR_BULK_THREADS)
+    k_traffic_sources(const __grid_constant__ dsr_dev_heap H, int32_t R, int rows) {
+    __shared__ dsr_bulk_smem<1> sm;
+    const int types[1] = {SOURCE};
+    dsr_bulk_create(
+        H, (dsr_u64)R, rows, types, sm, [](dsr_u64) { return 1u; },
+        [&](dsr_u64 i, unsigned, const dsr_ref (&ref)[1]) {
+            const dsr_ref s = ref[0];
+            if (s == DSR_NULL) return;
+            *fld(H, SOURCE, s, S_ROAD) = (int32_t)i;
+            *fld(H, SOURCE, s, S_ENTERED) = 0;
+            *fld(H, SOURCE, s, S_BLOCKED) = 0;
+        });
 }
 
 const int kCarFields[3] = {4, 4, 4};
@@ -193,9 +200,14 @@ extern "C" int dsr_traffic_create(dsr_heap* heap, const dsr_traffic_params* p, c
         return DSR_E_CUDA;
     }
     const dsr_u64 n = (dsr_u64)p->R * p->L;
-    dsr_u64 ctas = (n + 255) / 256;
-    if (ctas > (dsr_u64)heap->sm_count * 8) ctas = (dsr_u64)heap->sm_count * 8;
-    k_traffic_init<<<(unsigned)ctas, 256, 0, s>>>(heap->dev, static_cast<const int8_t*>(v0_dev), t->grid[0], *p);
+    const int rows = dsr__bulk_rows(n, heap->sm_count);
+    k_traffic_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
+        heap->dev, static_cast<const int8_t*>(v0_dev), t->grid[0], *p, rows);
+    if (!p->periodic) {
+        const int srows = dsr__bulk_rows((dsr_u64)p->R, heap->sm_count);
+        k_traffic_sources<<<dsr__bulk_grid((dsr_u64)p->R, srows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
+            heap->dev, p->R, srows);
+    }
     int rc = dsr__check_launch("k_traffic_init");
     if (rc) {
         delete t;

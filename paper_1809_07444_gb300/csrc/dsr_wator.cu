@@ -5,7 +5,7 @@
 // the batched form as group do-alls over the heaps of many instances.
 #include "dsr_apps.h"
 #include "dsr_bitmap_alloc.cuh"
-#include "dsr_group.cuh"
+#include "dsr_steps.cuh"
 
 namespace {
 enum { FISH = 0, SHARK = 1 };
@@ -56,12 +56,21 @@ __device__ __forceinline__ dsr_u64 intent_index(const dsr_bm_dev&, dsr_ref r) {
 // Every claimed cell has a winner (no mover dies between its choose and move
 // phases), so every word is NO_CLAIM again when a choose phase starts.
 
-__device__ __forceinline__ void neighbours(uint32_t c, int W, int H, uint32_t nb[4]) {
-    const int x = (int)(c % (uint32_t)W), y = (int)(c / (uint32_t)W);
-    nb[0] = (uint32_t)((y == 0 ? H - 1 : y - 1) * W + x);  // N
-    nb[1] = (uint32_t)(y * W + (x == W - 1 ? 0 : x + 1));  // E
-    nb[2] = (uint32_t)((y == H - 1 ? 0 : y + 1) * W + x);  // S
-    nb[3] = (uint32_t)(y * W + (x == 0 ? W - 1 : x - 1));  // W
+// The neighbour of cell c = (x, y) in direction d: 0 N, 1 E, 2 S, 3 W.
+__device__ __forceinline__ uint32_t neighbour(uint32_t c, int x, int y, int W, int H, int d) {
+    const uint32_t up = y == 0 ? c + (uint32_t)(H - 1) * (uint32_t)W : c - (uint32_t)W;
+    const uint32_t down = y == H - 1 ? c - (uint32_t)(H - 1) * (uint32_t)W : c + (uint32_t)W;
+    const uint32_t right = x == W - 1 ? c - (uint32_t)(W - 1) : c + 1u;
+    const uint32_t left = x == 0 ? c + (uint32_t)(W - 1) : c - 1u;
+    return d == 0 ? up : d == 1 ? right : d == 2 ? down : left;
+}
+
+// x and y after a move in direction d.
+__device__ __forceinline__ void step_to(int& x, int& y, int W, int H, int d) {
+    if (d == 0) y = y == 0 ? H - 1 : y - 1;
+    if (d == 1) x = x == W - 1 ? 0 : x + 1;
+    if (d == 2) y = y == H - 1 ? 0 : y + 1;
+    if (d == 3) x = x == 0 ? W - 1 : x - 1;
 }
 
 // Checked builds only: the instance exists and c is one of its cells.
@@ -70,41 +79,81 @@ __device__ __forceinline__ bool cell_ok(const HP& H, const WatorInst& I, uint32_
     return dsr_check(I.grid != nullptr && c < (uint32_t)I.p.W * (uint32_t)I.p.H, H.err, H.dbg, code, c);
 }
 
-// The k-th (0-based) set position among the low 4 bits of m, as a neighbour index.
+// The k-th (0-based, k < 4) set position among the low 4 bits of m.
 __device__ __forceinline__ int pick(unsigned m, unsigned k) {
-    for (int d = 0; d < 4; ++d)
-        if ((m >> d) & 1u) {
-            if (k == 0) return d;
-            --k;
-        }
-    return 0;
+    if (k > 0) m &= m - 1;
+    if (k > 1) m &= m - 1;
+    if (k > 2) m &= m - 1;
+    return __ffs(m) - 1;
+}
+
+// The key of this step's draws (stream 0: fish, 1: sharks).
+__device__ __forceinline__ dsr_u64 step_key(const WatorInst& I, dsr_u64 stream) {
+    return dsr_rand_key(I.p.seed, stream, *(volatile dsr_u64*)I.step);
+}
+
+// Births at once, where no do-all defers them (dsr_direct.cuh).
+struct NoDefer {
+    template <class HP>
+    __device__ __forceinline__ void moved(const HP& H) const {
+        dsr_count_lanes(H.ctr, DSR_CTR_APP0);
+    }
+    __device__ __forceinline__ bool defer(uint32_t) const { return false; }
+};
+struct Defer {
+    dsr_later& later;
+    unsigned& moves;
+    __device__ __forceinline__ void moved(const dsr_dev_heap&) const { ++moves; }
+    __device__ __forceinline__ bool defer(uint32_t c) const {
+        if (later.on) later.push(c);
+        return later.on;
+    }
+};
+
+// The choice of a mover in cell c among the candidate directions m (never 0):
+// claims the picked neighbour and returns its direction. Intents are
+// directions: the move phase finds its target and the new x and y by adding
+// to the old ones, without a division.
+__device__ __forceinline__ uint32_t claim_pick(const WatorInst& I, uint32_t c, int x, int y, unsigned m, dsr_u64 key) {
+    const int d = pick(m, dsr_mod_upto4(dsr_splitmix_at(key, c), (unsigned)__popc(m)));
+    atomicMin(I.claim + neighbour(c, x, y, I.p.W, I.p.H, d), c);
+    return (uint32_t)d;
 }
 
 // F1: age, pick an empty neighbour, claim it.
 template <class HP>
-__device__ __forceinline__ void fish_choose(const HP& H, const WatorInst& I, dsr_ref self) {
-    const dsr_u64 t = *(volatile dsr_u64*)I.step;
+__device__ __forceinline__ void fish_choose(const HP& H, const WatorInst& I, dsr_ref self, dsr_u64 key) {
     const int x = *dsr_field<int32_t>(H, FISH, self, X), y = *dsr_field<int32_t>(H, FISH, self, Y);
     *dsr_field<int32_t>(H, FISH, self, TIMER) += 1;
     const uint32_t c = (uint32_t)(y * I.p.W + x);
     if (!cell_ok(H, I, c, 6)) return;
-    uint32_t nb[4];
-    neighbours(c, I.p.W, I.p.H, nb);
+    uint32_t g[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) g[d] = I.grid[neighbour(c, x, y, I.p.W, I.p.H, d)];
     unsigned m = 0;
 #pragma unroll
-    for (int d = 0; d < 4; ++d) m |= (I.grid[nb[d]] == K_EMPTY ? 1u : 0u) << d;
-    uint32_t tgt = NO_MOVE;
-    if (m) {
-        tgt = nb[pick(m, (unsigned)(dsr_rand(I.p.seed, 0, t, c) % (dsr_u64)__popc(m)))];
-        atomicMin(I.claim + tgt, c);
-    }
+    for (int d = 0; d < 4; ++d) m |= (g[d] == K_EMPTY ? 1u : 0u) << d;
+    const uint32_t to = m ? claim_pick(I, c, x, y, m, key) : NO_MOVE;
     const dsr_u64 ix = intent_index(H, self);
-    if (dsr_check(ix < I.n_slots, H.err, H.dbg, 8, ix)) I.intent[ix] = tgt;
+    if (dsr_check(ix < I.n_slots, H.err, H.dbg, 8, ix)) I.intent[ix] = to;
+}
+
+// The fish born in cell c: r's fields and the cell's word.
+template <class HP>
+__device__ __forceinline__ void fish_born(const HP& H, const WatorInst& I, uint32_t c, dsr_ref r) {
+    uint32_t g = K_EMPTY;
+    if (r != DSR_NULL) {
+        *dsr_field<int32_t>(H, FISH, r, X) = (int32_t)(c % (uint32_t)I.p.W);
+        *dsr_field<int32_t>(H, FISH, r, Y) = (int32_t)(c / (uint32_t)I.p.W);
+        *dsr_field<int32_t>(H, FISH, r, TIMER) = 0;
+        g = grid_word(H, r, K_FISH);
+    }
+    I.grid[c] = g;
 }
 
 // F2: winners move and breed.
-template <class HP>
-__device__ __forceinline__ void fish_move(const HP& H, const WatorInst& I, dsr_ref self) {
+template <class HP, class Births>
+__device__ __forceinline__ void fish_move(const HP& H, const WatorInst& I, dsr_ref self, const Births& births) {
     int32_t* px = dsr_field<int32_t>(H, FISH, self, X);
     int32_t* py = dsr_field<int32_t>(H, FISH, self, Y);
     int32_t* timer = dsr_field<int32_t>(H, FISH, self, TIMER);
@@ -112,70 +161,74 @@ __device__ __forceinline__ void fish_move(const HP& H, const WatorInst& I, dsr_r
     if (!dsr_check(ix < I.n_slots, H.err, H.dbg, 8, ix)) return;
     // timer and intent are loaded with x and y: one round trip for all four
     const int32_t age = *timer;
-    const uint32_t tgt = I.intent[ix];
-    const uint32_t c = (uint32_t)(*py * I.p.W + *px);
-    if (!cell_ok(H, I, c, 6)) return;
-    if (tgt != NO_MOVE && !cell_ok(H, I, tgt, 7)) return;
-    if (tgt == NO_MOVE || I.claim[tgt] != c) return;
+    const uint32_t to = I.intent[ix];
+    int x = *px, y = *py;
+    const uint32_t c = (uint32_t)(y * I.p.W + x);
+    if (!cell_ok(H, I, c, 6) || to == NO_MOVE) return;
+    const uint32_t tgt = neighbour(c, x, y, I.p.W, I.p.H, (int)to);
+    if (I.claim[tgt] != c) return;
     I.claim[tgt] = NO_CLAIM;
-    dsr_count_lanes(H.ctr, DSR_CTR_APP0);
+    births.moved(H);
     I.grid[tgt] = grid_word(H, self, K_FISH);
-    *px = (int32_t)(tgt % (uint32_t)I.p.W);
-    *py = (int32_t)(tgt / (uint32_t)I.p.W);
-    uint32_t left = K_EMPTY;
-    if (age >= I.p.fish_breed) {
-        *timer = 0;
-        const dsr_ref n = dsr_new(H, FISH);
-        if (n != DSR_NULL) {
-            *dsr_field<int32_t>(H, FISH, n, X) = (int32_t)(c % (uint32_t)I.p.W);
-            *dsr_field<int32_t>(H, FISH, n, Y) = (int32_t)(c / (uint32_t)I.p.W);
-            *dsr_field<int32_t>(H, FISH, n, TIMER) = 0;
-            left = grid_word(H, n, K_FISH);
-        }
+    step_to(x, y, I.p.W, I.p.H, (int)to);
+    *px = x;
+    *py = y;
+    if (age < I.p.fish_breed) {
+        I.grid[c] = K_EMPTY;
+        return;
     }
-    I.grid[c] = left;
+    *timer = 0;
+    if (!births.defer(c)) fish_born(H, I, c, dsr_new(H, FISH));
 }
 
-// S0: starvation.
+// S0: starvation. Returns whether the shark lives on.
 template <class HP>
-__device__ __forceinline__ void shark_starve(const HP& H, const WatorInst& I, dsr_ref self) {
+__device__ __forceinline__ bool shark_starve(const HP& H, const WatorInst& I, dsr_ref self) {
     int32_t* e = dsr_field<int32_t>(H, SHARK, self, ENERGY);
-    if (--*e > 0) return;
+    if (--*e > 0) return true;
     const int x = *dsr_field<int32_t>(H, SHARK, self, X), y = *dsr_field<int32_t>(H, SHARK, self, Y);
     if (cell_ok(H, I, (uint32_t)(y * I.p.W + x), 6)) I.grid[y * I.p.W + x] = K_EMPTY;
     dsr_delete(H, self);
+    return false;
 }
 
 // S1: age, prefer a neighbouring fish, else an empty cell; claim it.
 template <class HP>
-__device__ __forceinline__ void shark_choose(const HP& H, const WatorInst& I, dsr_ref self) {
-    const dsr_u64 t = *(volatile dsr_u64*)I.step;
+__device__ __forceinline__ void shark_choose(const HP& H, const WatorInst& I, dsr_ref self, dsr_u64 key) {
     const int x = *dsr_field<int32_t>(H, SHARK, self, X), y = *dsr_field<int32_t>(H, SHARK, self, Y);
     *dsr_field<int32_t>(H, SHARK, self, TIMER) += 1;
     const uint32_t c = (uint32_t)(y * I.p.W + x);
     if (!cell_ok(H, I, c, 6)) return;
-    uint32_t nb[4];
-    neighbours(c, I.p.W, I.p.H, nb);
     unsigned mf = 0, me = 0;
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
-        const uint32_t g = I.grid[nb[d]];
+        const uint32_t g = I.grid[neighbour(c, x, y, I.p.W, I.p.H, d)];
         mf |= ((g & 3) == K_FISH ? 1u : 0u) << d;
         me |= (g == K_EMPTY ? 1u : 0u) << d;
     }
     const unsigned m = mf ? mf : me;
-    uint32_t tgt = NO_MOVE;
-    if (m) {
-        tgt = nb[pick(m, (unsigned)(dsr_rand(I.p.seed, 1, t, c) % (dsr_u64)__popc(m)))];
-        atomicMin(I.claim + tgt, c);
-    }
+    const uint32_t to = m ? claim_pick(I, c, x, y, m, key) : NO_MOVE;
     const dsr_u64 ix = intent_index(H, self);
-    if (dsr_check(ix < I.n_slots, H.err, H.dbg, 8, ix)) I.intent[ix] = tgt;
+    if (dsr_check(ix < I.n_slots, H.err, H.dbg, 8, ix)) I.intent[ix] = to;
+}
+
+// The shark born in cell c.
+template <class HP>
+__device__ __forceinline__ void shark_born(const HP& H, const WatorInst& I, uint32_t c, dsr_ref r) {
+    uint32_t g = K_EMPTY;
+    if (r != DSR_NULL) {
+        *dsr_field<int32_t>(H, SHARK, r, X) = (int32_t)(c % (uint32_t)I.p.W);
+        *dsr_field<int32_t>(H, SHARK, r, Y) = (int32_t)(c / (uint32_t)I.p.W);
+        *dsr_field<int32_t>(H, SHARK, r, TIMER) = 0;
+        *dsr_field<int32_t>(H, SHARK, r, ENERGY) = I.p.shark_energy0;
+        g = grid_word(H, r, K_SHARK);
+    }
+    I.grid[c] = g;
 }
 
 // S2: winners move, eat and breed.
-template <class HP>
-__device__ __forceinline__ void shark_move(const HP& H, const WatorInst& I, dsr_ref self) {
+template <class HP, class Births>
+__device__ __forceinline__ void shark_move(const HP& H, const WatorInst& I, dsr_ref self, const Births& births) {
     int32_t* px = dsr_field<int32_t>(H, SHARK, self, X);
     int32_t* py = dsr_field<int32_t>(H, SHARK, self, Y);
     int32_t* timer = dsr_field<int32_t>(H, SHARK, self, TIMER);
@@ -183,48 +236,43 @@ __device__ __forceinline__ void shark_move(const HP& H, const WatorInst& I, dsr_
     const dsr_u64 ix = intent_index(H, self);
     if (!dsr_check(ix < I.n_slots, H.err, H.dbg, 8, ix)) return;
     const int32_t age = *timer, e0 = *energy;  // loaded with x and y
-    const uint32_t tgt = I.intent[ix];
-    const uint32_t c = (uint32_t)(*py * I.p.W + *px);
-    if (!cell_ok(H, I, c, 6)) return;
-    if (tgt != NO_MOVE && !cell_ok(H, I, tgt, 7)) return;
-    if (tgt == NO_MOVE || I.claim[tgt] != c) return;
+    const uint32_t to = I.intent[ix];
+    int x = *px, y = *py;
+    const uint32_t c = (uint32_t)(y * I.p.W + x);
+    if (!cell_ok(H, I, c, 6) || to == NO_MOVE) return;
+    const uint32_t tgt = neighbour(c, x, y, I.p.W, I.p.H, (int)to);
+    const uint32_t g = I.grid[tgt];  // loaded with the claim
+    if (I.claim[tgt] != c) return;
     I.claim[tgt] = NO_CLAIM;
-    dsr_count_lanes(H.ctr, DSR_CTR_APP0);
-    const uint32_t g = I.grid[tgt];
+    births.moved(H);
     if ((g & 3) == K_FISH) {
         dsr_delete(H, grid_ref(H, g));
         *energy = e0 + I.p.shark_gain;
     }
     I.grid[tgt] = grid_word(H, self, K_SHARK);
-    *px = (int32_t)(tgt % (uint32_t)I.p.W);
-    *py = (int32_t)(tgt / (uint32_t)I.p.W);
-    uint32_t left = K_EMPTY;
-    if (age >= I.p.shark_breed) {
-        *timer = 0;
-        const dsr_ref n = dsr_new(H, SHARK);
-        if (n != DSR_NULL) {
-            *dsr_field<int32_t>(H, SHARK, n, X) = (int32_t)(c % (uint32_t)I.p.W);
-            *dsr_field<int32_t>(H, SHARK, n, Y) = (int32_t)(c / (uint32_t)I.p.W);
-            *dsr_field<int32_t>(H, SHARK, n, TIMER) = 0;
-            *dsr_field<int32_t>(H, SHARK, n, ENERGY) = I.p.shark_energy0;
-            left = grid_word(H, n, K_SHARK);
-        }
+    step_to(x, y, I.p.W, I.p.H, (int)to);
+    *px = x;
+    *py = y;
+    if (age < I.p.shark_breed) {
+        I.grid[c] = K_EMPTY;
+        return;
     }
-    I.grid[c] = left;
+    *timer = 0;
+    if (!births.defer(c)) shark_born(H, I, c, dsr_new(H, SHARK));
 }
 
-// ---- plain form: do-all methods over one heap ------------------------------
+// ---- list do-alls over one heap (dsr_parallel_do, BitmapAlloc) -------------
 // (HP: the heap type; dsr_dev_heap, or dsr_bm_dev for the BitmapAlloc
 // comparator)
 template <class HP>
 struct MFishChooseT {
     typedef WatorInst Args;
-    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { fish_choose(H, a, s); }
+    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { fish_choose(H, a, s, step_key(a, 0)); }
 };
 template <class HP>
 struct MFishMoveT {
     typedef WatorInst Args;
-    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { fish_move(H, a, s); }
+    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { fish_move(H, a, s, NoDefer{}); }
 };
 template <class HP>
 struct MSharkStarveT {
@@ -234,13 +282,13 @@ struct MSharkStarveT {
 template <class HP>
 struct MSharkChooseT {
     typedef WatorInst Args;
-    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { shark_choose(H, a, s); }
+    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { shark_choose(H, a, s, step_key(a, 1)); }
 };
 // The last CTA of the last phase advances the step counter.
 template <class HP>
 struct MSharkMoveT {
     typedef WatorInst Args;
-    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { shark_move(H, a, s); }
+    static __device__ void run(const HP& H, int, const Args& a, dsr_ref s) { shark_move(H, a, s, NoDefer{}); }
     static __device__ void finish(const HP&, int, const Args& a) { *a.step += 1; }
 };
 typedef MFishChooseT<dsr_dev_heap> MFishChoose;
@@ -249,74 +297,157 @@ typedef MSharkStarveT<dsr_dev_heap> MSharkStarve;
 typedef MSharkChooseT<dsr_dev_heap> MSharkChoose;
 typedef MSharkMoveT<dsr_dev_heap> MSharkMove;
 
-// ---- batched form: group do-all methods over the heaps of many instances ----
-// Heap index h of a group is the instance slot; table[h] is its view.
+// ---- the plain and the batched step (dsr_steps.cuh) -------------------------
+// A: WatorInst (plain form), or BatchArgs: heap index h of a group is the
+// instance slot, table[h] its view.
 struct BatchArgs {
     const WatorInst* table;
 };
-struct GFishChoose {
-    typedef BatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref s, uint32_t h) {
-        fish_choose(H, a.table[h], s);
+__device__ __forceinline__ const WatorInst& inst_of(const WatorInst& a, uint32_t) { return a; }
+__device__ __forceinline__ const WatorInst& inst_of(const BatchArgs& a, uint32_t h) { return a.table[h]; }
+
+struct NoCtx {};
+template <class A>
+struct WatorMethod {
+    typedef A Args;
+    typedef WatorInst Inst;
+    typedef dsr_no_acc Acc;
+    typedef NoCtx Ctx;
+    enum { kDefers = DSR_NOTHING, kMarks = 0 };
+    static __device__ __forceinline__ const WatorInst& inst(const A& a, uint32_t h) { return inst_of(a, h); }
+    static __device__ __forceinline__ NoCtx begin(const WatorInst&) { return {}; }
+    static __device__ __forceinline__ void flush(const dsr_dev_heap&, const WatorInst&, dsr_no_acc) {}
+};
+// A move phase counts its moves per thread.
+template <class A>
+struct WatorMove : WatorMethod<A> {
+    typedef unsigned Acc;
+    static __device__ __forceinline__ void flush(const dsr_dev_heap& H, const WatorInst&, unsigned moves) {
+        dsr_flush_count(H, DSR_CTR_APP0, moves);
     }
 };
-struct GFishMove {
-    typedef BatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref s, uint32_t h) {
-        fish_move(H, a.table[h], s);
+template <class A>
+struct DFishChoose : WatorMethod<A> {
+    typedef dsr_u64 Ctx;
+    static __device__ __forceinline__ Ctx begin(const WatorInst& I) { return step_key(I, 0); }
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const WatorInst& I, Ctx key, dsr_ref s,
+                                                   dsr_later&, dsr_no_acc&) {
+        fish_choose(H, I, s, key);
+        return 0;
     }
 };
-struct GSharkStarve {
-    typedef BatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref s, uint32_t h) {
-        shark_starve(H, a.table[h], s);
+template <class A>
+struct DFishMove : WatorMove<A> {
+    enum { kDefers = FISH };
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const WatorInst& I, NoCtx, dsr_ref s,
+                                                   dsr_later& later, unsigned& moves) {
+        fish_move(H, I, s, Defer{later, moves});
+        return 0;
+    }
+    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const WatorInst& I, NoCtx, dsr_u64 c, dsr_ref r,
+                                                unsigned&) {
+        fish_born(H, I, (uint32_t)c, r);
     }
 };
-struct GSharkChoose {
-    typedef BatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref s, uint32_t h) {
-        shark_choose(H, a.table[h], s);
+// Marks the survivors, which S1 and S2 then visit.
+template <class A>
+struct DSharkStarve : WatorMethod<A> {
+    typedef unsigned Acc;
+    enum { kMarks = 1 };
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const WatorInst& I, NoCtx, dsr_ref s,
+                                                   dsr_later&, unsigned& survivors) {
+        const unsigned lives = shark_starve(H, I, s) ? 1u : 0u;
+        survivors += lives;
+        return lives;
+    }
+    static __device__ __forceinline__ void flush(const dsr_dev_heap& H, const WatorInst&, unsigned survivors) {
+        dsr_flush_count(H, DSR_CTR_VISITS, 2 * survivors);  // the visits of S1 and S2
     }
 };
-struct GSharkMove {
-    typedef BatchArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref s, uint32_t h) {
-        shark_move(H, a.table[h], s);
+template <class A>
+struct DSharkChoose : WatorMethod<A> {
+    typedef dsr_u64 Ctx;
+    static __device__ __forceinline__ Ctx begin(const WatorInst& I) { return step_key(I, 1); }
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const WatorInst& I, Ctx key, dsr_ref s,
+                                                   dsr_later&, dsr_no_acc&) {
+        shark_choose(H, I, s, key);
+        return 0;
     }
-    // every instance in the batch advances one step
-    static __device__ void finish_group(const dsr_group_dev& G, int, const Args& a) {
+};
+template <class A>
+struct DSharkMove : WatorMove<A> {
+    enum { kDefers = SHARK };
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const WatorInst& I, NoCtx, dsr_ref s,
+                                                   dsr_later& later, unsigned& moves) {
+        shark_move(H, I, s, Defer{later, moves});
+        return 0;
+    }
+    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const WatorInst& I, NoCtx, dsr_u64 c, dsr_ref r,
+                                                unsigned&) {
+        shark_born(H, I, (uint32_t)c, r);
+    }
+};
+// The last CTA of a step's last do-all advances the step counter (of every
+// instance in the batch).
+struct NextStep {
+    static __device__ void finish(const dsr_dev_heap&, const WatorInst& a) { *a.step += 1; }
+    static __device__ void finish_group(const dsr_group_dev& G, const BatchArgs& a) {
         for (uint32_t i = threadIdx.x; i < G.n_slots; i += blockDim.x)
             if (a.table[i].step) *a.table[i].step += 1;
     }
 };
 
-// One thread per cell: create the initial agents and clear the claim state.
+// The do-alls of a step. One scan lists the fish and the sharks. F1 and S1
+// create and delete nothing, so F2 works on the fish listed for F1, and S1 and
+// S2 on the sharks that S0 left. S0 neither reads nor writes a cell that F2
+// does (a fish moves into cells that were empty at the start of the step), so
+// the two share a launch.
+constexpr dsr_phase kFish{FISH, 0}, kSharks{SHARK, 1};
+
+// Creates the agent of cell c (or none), and clears the cell's claim.
 template <class HP>
-__global__ void k_wator_init(const __grid_constant__ HP H, const uint8_t* kind0, WatorInst I) {
+__device__ __forceinline__ void init_cell(const HP& H, const WatorInst& I, uint32_t c, int T, dsr_ref r) {
+    uint32_t g = K_EMPTY;
+    if (r != DSR_NULL) {
+        *dsr_field<int32_t>(H, T, r, X) = (int32_t)(c % (uint32_t)I.p.W);
+        *dsr_field<int32_t>(H, T, r, Y) = (int32_t)(c / (uint32_t)I.p.W);
+        *dsr_field<int32_t>(H, T, r, TIMER) = 0;
+        if (T == SHARK) *dsr_field<int32_t>(H, SHARK, r, ENERGY) = I.p.shark_energy0;
+        g = grid_word(H, r, T == FISH ? K_FISH : K_SHARK);
+    }
+    I.grid[c] = g;
+    I.claim[c] = NO_CLAIM;
+    if (c == 0) *I.step = 0;
+}
+
+// One thread per cell: create the initial agents and clear the claim state.
+__global__ void __launch_bounds__(DSR_BULK_THREADS)
+    k_wator_init(const __grid_constant__ dsr_dev_heap H, const uint8_t* kind0, WatorInst I, int rows) {
+    __shared__ dsr_bulk_smem<2> sm;
+    const int types[2] = {FISH, SHARK};
+    dsr_bulk_create(
+        H, (dsr_u64)I.p.W * I.p.H, rows, types, sm,
+        [&](dsr_u64 c) {
+            const uint8_t k = kind0[c];
+            return k == 1 || k == 2 ? (unsigned)k : 0u;
+        },
+        [&](dsr_u64 c, unsigned kind, const dsr_ref (&ref)[2]) {
+            init_cell(H, I, (uint32_t)c, kind == 2 ? SHARK : FISH, kind == 2 ? ref[1] : ref[0]);
+        });
+}
+
+// The same on the BitmapAlloc comparator, through its dsr_new.
+__global__ void k_wator_bm_init(const __grid_constant__ dsr_bm_dev H, const uint8_t* kind0, WatorInst I) {
     const uint32_t n = (uint32_t)I.p.W * (uint32_t)I.p.H;
     const uint32_t n32 = (n + 31u) & ~31u;  // warp-uniform trip count
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n32; c += gridDim.x * blockDim.x) {
         __syncwarp();  // whole-warp groups for dsr_new
         if (c >= n) continue;
         const uint8_t k = kind0[c];
-        uint32_t g = K_EMPTY;
-        if (k == 1 || k == 2) {
-            // one dsr_new for fish and sharks: the two groups' leaders then
-            // run their reservations side by side rather than one after the
-            // other in two branches
-            const int T = k == 1 ? FISH : SHARK;
-            const dsr_ref r = dsr_new(H, T);
-            if (r != DSR_NULL) {
-                *dsr_field<int32_t>(H, T, r, X) = (int32_t)(c % (uint32_t)I.p.W);
-                *dsr_field<int32_t>(H, T, r, Y) = (int32_t)(c / (uint32_t)I.p.W);
-                *dsr_field<int32_t>(H, T, r, TIMER) = 0;
-                if (T == SHARK) *dsr_field<int32_t>(H, SHARK, r, ENERGY) = I.p.shark_energy0;
-                g = grid_word(H, r, k == 1 ? K_FISH : K_SHARK);
-            }
-        }
-        I.grid[c] = g;
-        I.claim[c] = NO_CLAIM;
-        if (c == 0) *I.step = 0;
+        const int T = k == 1 ? FISH : SHARK;
+        dsr_ref r = DSR_NULL;
+        if (k == 1 || k == 2) r = dsr_new(H, T);
+        init_cell(H, I, c, T, r);
     }
 }
 
@@ -375,9 +506,9 @@ dsr_u64 bm_slots(const dsr_bm_heap* h) {
 
 int launch_init(const dsr_heap* heap, const WatorInst& I, const void* kind0_dev, cudaStream_t s) {
     const uint32_t n = (uint32_t)I.p.W * (uint32_t)I.p.H;
-    unsigned ctas = (n + 255) / 256;
-    if (ctas > (unsigned)heap->sm_count * 8) ctas = (unsigned)heap->sm_count * 8;
-    k_wator_init<dsr_dev_heap><<<ctas, 256, 0, s>>>(heap->dev, static_cast<const uint8_t*>(kind0_dev), I);
+    const int rows = dsr__bulk_rows(n, heap->sm_count);
+    k_wator_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
+        heap->dev, static_cast<const uint8_t*>(kind0_dev), I, rows);
     return dsr__check_launch("k_wator_init");
 }
 
@@ -395,7 +526,7 @@ int launch_kinds(const dsr_heap* heap, const WatorInst& I, void* out, cudaStream
 // ===========================================================================
 constexpr int kPhaseEvents = 11;  // step start, then after each scan and each method kernel
 
-// One step replayed as a CUDA graph: its 8 launches (and, when the step is
+// One step replayed as a CUDA graph: its launches (and, when the step is
 // timed, its event records as event-record nodes, pointed at each step's
 // own events before the launch). Captured on first use, once for untimed
 // steps and once for the current timing selection.
@@ -487,14 +618,31 @@ static int issue_step(dsr_wator* w, cudaStream_t s, const cudaEvent_t* e, int se
         if (!e || (sel >= 0 && k != 2 * sel + 1 && k != 2 * sel + 2)) return nullptr;
         return e[k];
     };
-    // F1 neither creates nor deletes fish, so F2 runs over F1's block list
-    // (the fish live at the start of the step); likewise S2 over S1's (the
-    // sharks that survived S0).
-    int rc = dsr__doall<MFishChoose>(h, FISH, w->inst, s, true, E(1), E(2), 1);
-    if (!rc) rc = dsr__doall<MFishMove>(h, FISH, w->inst, s, false, E(3), E(4));
-    if (!rc) rc = dsr__doall<MSharkStarve>(h, SHARK, w->inst, s, true, E(5), E(6));
-    if (!rc) rc = dsr__doall<MSharkChoose>(h, SHARK, w->inst, s, true, E(7), E(8), 1);
-    if (!rc) rc = dsr__doall<MSharkMove>(h, SHARK, w->inst, s, false, E(9), E(10));
+    typedef WatorInst A;
+    const A& I = w->inst;
+    auto record = [&](int k) {
+        if (E(k)) cudaEventRecordWithFlags(E(k), s, cudaEventRecordExternal);
+    };
+    dsr__list_types(h, FISH, SHARK, 2, 1, s);
+    record(1);
+    int rc = dsr__step<DFishChoose<A>>(h, kFish, kFish, I, s);
+    record(2);
+    record(3);
+    if (!e) {
+        if (!rc) rc = dsr__step<DFishMove<A>, DSharkStarve<A>>(h, kFish, kSharks, I, s);
+    } else {  // timed: every phase in a launch of its own
+        if (!rc) rc = dsr__step<DFishMove<A>>(h, kFish, kFish, I, s);
+        record(4);
+        record(5);
+        if (!rc) rc = dsr__step<DSharkStarve<A>>(h, kSharks, kSharks, I, s);
+        record(6);
+    }
+    record(7);
+    if (!rc) rc = dsr__step<DSharkChoose<A>>(h, kSharks, kSharks, I, s);
+    record(8);
+    record(9);
+    if (!rc) rc = dsr__step<DSharkMove<A>, dsr_no_method, true, NextStep>(h, kSharks, kSharks, I, s);
+    record(10);
     return rc;
 }
 
@@ -734,9 +882,8 @@ extern "C" int dsr_wator_bm_create(dsr_bm_heap* heap, const dsr_wator_params* p,
     const uint32_t n = (uint32_t)p->W * (uint32_t)p->H;
     unsigned ctas = (n + 255) / 256;
     if (ctas > (unsigned)heap->sm_count * 8) ctas = (unsigned)heap->sm_count * 8;
-    k_wator_init<dsr_bm_dev>
-        <<<ctas, 256, 0, dsr__stream(stream)>>>(heap->dev, static_cast<const uint8_t*>(kind0_dev), w->inst);
-    const int rc = dsr__check_launch("k_wator_init");
+    k_wator_bm_init<<<ctas, 256, 0, dsr__stream(stream)>>>(heap->dev, static_cast<const uint8_t*>(kind0_dev), w->inst);
+    const int rc = dsr__check_launch("k_wator_bm_init");
     if (rc) {
         delete w;
         return rc;
@@ -885,17 +1032,16 @@ extern "C" int dsr_wator_batch_remove(dsr_wator_batch* b, int inst) {
 static int issue_batch_step(dsr_wator_batch* b, cudaStream_t s) {
     dsr_group* g = b->group;
     BatchArgs a{b->table_d};
-    // F2 and S2 run over the block lists of F1 and S1 (see dsr_wator_step)
-    int rc = dsr__group_doall<GFishChoose>(g, FISH, a, s, true, 1);
-    if (!rc) rc = dsr__group_doall<GFishMove>(g, FISH, a, s, false);
-    if (!rc) rc = dsr__group_doall<GSharkStarve>(g, SHARK, a, s);
-    if (!rc) rc = dsr__group_doall<GSharkChoose>(g, SHARK, a, s, true, 1);
-    if (!rc) rc = dsr__group_doall<GSharkMove>(g, SHARK, a, s, false);
+    typedef BatchArgs A;
+    dsr__group_list_types(g, FISH, SHARK, 2, 1, s);
+    int rc = dsr__group_step<DFishChoose<A>>(g, kFish, kFish, a, s);
+    if (!rc) rc = dsr__group_step<DFishMove<A>, DSharkStarve<A>>(g, kFish, kSharks, a, s);
+    if (!rc) rc = dsr__group_step<DSharkChoose<A>>(g, kSharks, kSharks, a, s);
+    if (!rc) rc = dsr__group_step<DSharkMove<A>, dsr_no_method, true, NextStep>(g, kSharks, kSharks, a, s);
     return rc;
 }
 
-// One batched step is 10 launches (5 fused scans, 5 method kernels) over all
-// instances; it is captured once into a CUDA graph and replayed until the set
+// One batched step is five launches over all instances (as in dsr_wator_step); it is captured once into a CUDA graph and replayed until the set
 // of instances changes.
 static int ensure_graph(dsr_wator_batch* b) {
     if (b->exec_epoch == b->group->epoch) return DSR_OK;
