@@ -4,8 +4,7 @@
 Workload: wa-tor on a 2048 x 2048 torus (30% fish, 3% sharks, seed 1), the
 plain one-simulation form. A step is one wa-tor step: five parallel do-alls
 with device new/delete for births and deaths, i.e. every row of the hot
-path. Three of them scan and compact the block list; F2 and S2 run over the
-lists of F1 and S1, which create and delete nothing.
+path. One scan lists the blocks of both types for all of them.
 
   value      do-all object-updates/s (objects visited by method kernels per
              second of device time), inputs resident in HBM;
@@ -17,8 +16,8 @@ lists of F1 and S1, which create and delete nothing.
              algorithmic bytes (per-object and per-event byte counts of the
              wa-tor rules, see phase_bytes) over its CUDA-event time, both
              summed over the timed steps, against the measured HBM copy
-             peak. Times come from events recorded around every scan and
-             method kernel inside the timed region; the event counts
+             peak. Times come from events recorded around the method
+             kernel inside the timed region; the event counts
              (objects, blocks, moves, births, deaths) from a replay of the
              same steps, checked against the timed window's visit count;
   cpu_baseline  the oracle (single-threaded C++) on the same workload, and
@@ -302,12 +301,14 @@ class Clocks:
 # the GPU arm
 # ---------------------------------------------------------------------------
 PHASES = ("F1", "F2", "S0", "S1", "S2")
-# kernels of one wa-tor step: a scan and a method kernel for F1, S0 and S1; a
-# method kernel alone for F2 and S2 (they run over the lists of F1 and S1)
-LAUNCHES_PER_STEP = 8
-KERNELS = {"F1": "dsr_doall_kernel<MFishChoose>", "F2": "dsr_doall_kernel<MFishMove>",
-           "S0": "dsr_doall_kernel<MSharkStarve>", "S1": "dsr_doall_kernel<MSharkChoose>",
-           "S2": "dsr_doall_kernel<MSharkMove>"}
+# kernels of one wa-tor step: one scan that lists fish and sharks, and a method
+# kernel per phase, of which F2 and S0 share a launch unless the step is timed
+LAUNCHES_PER_STEP = 5
+LAUNCHES_PER_TIMED_STEP = 6
+LAUNCHES_PER_BITMAP_STEP = 8  # the BitmapAlloc comparator: three scans, five method kernels
+KERNELS = {"F1": "dsr_step_kernel<DFishChoose>", "F2": "dsr_step_kernel<DFishMove>",
+           "S0": "dsr_step_kernel<DSharkStarve>", "S1": "dsr_step_kernel<DSharkChoose>",
+           "S2": "dsr_step_kernel<DSharkMove>"}
 
 
 def phase_bytes(phase, objs, blocks, moves, births, deaths):
@@ -735,7 +736,7 @@ def bench_comparators(steps=50, warmup=5):
         t = sum(a.elapsed_time(b) for a, b in evs) / 1e3
         v = w.visits() - v0
         out[name] = {"ms_per_step": t * 1e3 / steps, "object_updates_per_s": v / t,
-                     "launches_per_step": 5 if aos is not None else LAUNCHES_PER_STEP}
+                     "launches_per_step": 5 if aos is not None else LAUNCHES_PER_BITMAP_STEP}
         del w
     del flush
     torch.cuda.empty_cache()
@@ -1185,7 +1186,7 @@ def main():
         "e2e": {"value": e2e_visits / e2e_s, "unit": UNIT, "h2d_bytes_per_step": r["h2d"] / args.steps,
                 "d2h_bytes_per_step": r["d2h"] / args.steps, "timing": "host wall clock around the C-ABI calls",
                 "device_s": r["e2e_dev_s"], "host_s": e2e_s},
-        "gpu_launches": LAUNCHES_PER_STEP * args.steps,
+        "gpu_launches": LAUNCHES_PER_TIMED_STEP * args.steps,
         "roofline": roofline(r["phases"], peak, peak_kind, args.steps, args.warmup),
     }
     if not args.no_cpu_baseline:

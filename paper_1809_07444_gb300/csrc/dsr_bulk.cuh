@@ -102,6 +102,19 @@ __device__ inline uint32_t dsr_claim_full(const dsr_dev_heap& H, int T, uint32_t
     return n;
 }
 
+// Exclusive prefix sum of v over the calling warp (whole); *total: its sum.
+__device__ __forceinline__ uint32_t dsr_warp_prefix(uint32_t v, uint32_t* total) {
+    const unsigned lane = dsr_lane();
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if ((int)lane >= o) incl += y;
+    }
+    *total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    return incl - v;
+}
+
 // Elements 0 .. n - 1, `rows` (1 .. DSR_BULK_ROWS) x 256 of them a chunk, one
 // chunk per CTA and round. kind(i): bit k set if element i creates an object
 // of types[k]. make(i, kind, refs): runs once for every element; refs[k] is
@@ -138,19 +151,13 @@ __device__ __forceinline__ void dsr_bulk_create(const dsr_dev_heap& H, dsr_u64 n
                 v[q] = at < m ? c[at] : 0u;
                 sum += v[q];
             }
-            uint32_t incl = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if ((int)lane >= o) incl += y;
-            }
-            uint32_t at = incl - sum;
+            uint32_t total;
+            uint32_t at = dsr_warp_prefix(sum, &total);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 if (4 * (int)lane + q < m) c[4 * (int)lane + q] = at;
                 at += v[q];
             }
-            const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
             const int T = types[warp];
             uint32_t want = total / H.cap[T];
             if (want > DSR_BULK_BLOCKS) want = DSR_BULK_BLOCKS;

@@ -114,7 +114,7 @@ struct DDie : GolMethod<A> {
 };
 template <class A>
 struct DBirth : GolMethod<A> {
-    enum { kDefers = ALIVE };
+    enum { kDefers = ALIVE, kDeferBack = 1 };
     static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const GolArgs& a, NoCtx, dsr_ref self,
                                                    dsr_later& later, dsr_no_acc&) {
         int idx;
@@ -126,8 +126,7 @@ struct DBirth : GolMethod<A> {
         }
         return 0;
     }
-    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const GolArgs& a, NoCtx, dsr_u64 idx, dsr_ref r,
-                                                dsr_no_acc&) {
+    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const GolArgs& a, dsr_u64 idx, dsr_ref r) {
         gol_born(H, a, (int)idx, r);
     }
 };

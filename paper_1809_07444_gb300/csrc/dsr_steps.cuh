@@ -4,27 +4,31 @@
 // runs one method over the list in a second. A step of an application is a
 // fixed sequence of do-alls over two types, and it knows which of them leave
 // the live set of a type alone. So a step lists both types in one scan (type
-// A's blocks from the front of H.R_bid / H.R_mask, type B's from the back:
-// together at most M entries), and every do-all of the step runs over those
-// lists. A method that deletes objects replaces its entry's mask by the
-// survivors (kMarks) where a later do-all of the step visits them. Two
-// do-alls that do not depend on each other share a launch.
+// A's blocks from the front of R_bid / R_mask, type B's from the back:
+// together at most as many entries as there are blocks), and every do-all of
+// the step runs over those lists. A method that deletes objects replaces its
+// entry's mask by the survivors (kMarks) where a later do-all of the step
+// visits them. Two do-alls that do not depend on each other share a launch.
 //
-// A warp takes every W-th (block, 32 slots) item. Its 32 lanes load the
-// entries of its next 32 items at once and hand them out by shuffle, so the
-// list costs one round trip per 32 items and warp, not one per item.
+// Every CTA has one stretch of the list, of (block, 32 slots) items as equal
+// in number as can be; its warps take them in turn. A warp's 32 lanes load
+// the entries of its next 32 items at once and hand them out by shuffle, so
+// the list costs one round trip per 32 items and warp, not one per item.
 //
 // Deferred work. A method may put off an object's creation: it pushes a
 // word, and the CTA later creates all pending objects together and calls
 // M::born for each. Births come from the few lanes of a warp whose object
-// breeds; together they are whole blocks' worth, which are claimed many at a
-// time and born full (dsr_claim_full). That is done while few blocks of the
-// type have free slots; else births fill the holes at once through dsr_new,
-// lane group by lane group, as in any other method, so that fragmentation
-// stays as it is there. "Few": less than one block in DSR_BULK_HOLES, by a
-// sample of 32 leaf words of active[T] and allocated[T] when the do-all
-// starts. Work that few objects have (a dead agent's replacement) can be
-// deferred in the same way without a creation: full warps then do it.
+// breeds, and a search by their leader is a chain of five dependent accesses
+// that the rest of the warp waits for, in competition with all other leaders.
+// The list says where the free slots of the created type are: each CTA has a
+// stretch of that type's blocks as well, whose holes are its own to fill, one
+// block per thread, with one atomic each and no search. Only when they are
+// full are whole blocks claimed (dsr_claim_full). A remainder goes to another
+// CTA's partly filled block, if two searches find one; else a block is opened
+// for it if the CTA has at least DSR_OPEN_SHARE blocks already (at most one in
+// that many is then partly filled for this reason), or it goes through dsr_new. Work that
+// few objects have (a dead agent's replacement) can be deferred in the same
+// way without a creation: full warps then do it.
 //
 // A method is a type with
 //   Args; Inst; Ctx; Acc
@@ -32,10 +36,12 @@
 //   static Ctx begin(const Inst&)                        once per do-all (plain) or item (group)
 //   static unsigned run(H, T, const Inst&, const Ctx&, dsr_ref self, dsr_later&, Acc&)
 //   kDefers: DSR_NOTHING, DSR_WORK (M::later(H, I, ctx, word, acc) for each
-//     pushed word) or the type created (M::born(H, I, ctx, word, ref, acc))
+//     pushed word; not in groups) or the type created (M::born(H, I, ctx,
+//     word, ref); words of 32 bits in groups); kDeferBack: whether that type
+//     is listed at the back
 //   kMarks: 1 if run's result (0 or 1) replaces the slot's bit of the list entry
-//   static void flush(H, const Inst&, const Acc&)        by every whole warp at
-//     the end: event counts gathered in Acc go to memory
+//   static void flush(H, const Inst&, const Acc&)        by a whole warp: event
+//     counts gathered in Acc go to memory
 #pragma once
 
 #include <type_traits>
@@ -43,11 +49,11 @@
 #include "dsr_bulk.cuh"
 #include "dsr_group.cuh"
 
-#ifndef DSR_BULK_HOLES
-#define DSR_BULK_HOLES 8
+constexpr int DSR_LIST_BACK = 2;         // R_count[2] counts the entries at the back of the list
+constexpr int DSR_GROUP_LIST_BACK = 32;  // the same for a group's list
+#ifndef DSR_OPEN_SHARE
+#define DSR_OPEN_SHARE 16
 #endif
-constexpr int DSR_PENDING = 2048;  // deferred words of a CTA at a time
-constexpr int DSR_LIST_BACK = 2;   // R_count[2] counts the entries at the back of the list
 
 enum { DSR_NOTHING = -1, DSR_WORK = -2 };
 struct dsr_no_acc {};
@@ -59,72 +65,218 @@ struct dsr_phase {
     int back;
 };
 
+// Deferred words of a CTA at a time: two from every thread at least.
+template <int MAXT>
 struct dsr_later_smem {
-    dsr_u64 pending[DSR_PENDING];
-    uint32_t block[DSR_PENDING / 16];
-    uint32_t np, nb;
-    int few;
+    enum { PENDING = MAXT > 512 ? 2 * MAXT : 1024 };
+    dsr_u64 pending[PENDING];
+    dsr_ref ref[PENDING];
+    uint16_t index[PENDING];  // groups: the pending words of the heap being served
+    uint32_t block[PENDING / 16];
+    uint32_t holes[MAXT / 32];  // per warp
+    uint32_t np, nb, next, n_open, heap;
+    dsr_ref open;  // the first slot of the block opened for the remainder
 };
 
 // push() may be called by any lanes of a warp.
 struct dsr_later {
-    dsr_later_smem* sm;
-    bool on;  // creations are deferred
+    uint32_t* np;
+    dsr_u64* pending;
+    dsr_u64 tag;  // groups: heap index << 32
+    bool on;      // work is deferred
     __device__ __forceinline__ void push(dsr_u64 word) {
         const unsigned act = __activemask();
         const unsigned lane = dsr_lane();
         const int leader = __ffs(act) - 1;
         uint32_t at = 0;
-        if ((int)lane == leader) at = atomicAdd(&sm->np, (uint32_t)__popc(act));
+        if ((int)lane == leader) at = atomicAdd(np, (uint32_t)__popc(act));
         at = __shfl_sync(act, at, leader);
-        sm->pending[at + __popc(act & ((1u << lane) - 1))] = word;
+        pending[at + __popc(act & ((1u << lane) - 1))] = word | tag;
     }
 };
 
-// Whether fewer than one in DSR_BULK_HOLES of the allocated blocks of T has a
-// free slot, by a sample. Called by a whole warp.
-__device__ __forceinline__ bool dsr_few_holes(const dsr_dev_heap& H, int T, unsigned hint) {
-    const uint32_t at = __umulhi(dsr_hash32(hint + dsr_lane() * 0x9E3779B9u), H.active_bm[T].nwords[0]);
-    const unsigned active = __popcll(dsr_ld_relaxed(H.active_bm[T].lvl[0] + at));
-    const unsigned alloc = __popcll(dsr_ld_relaxed(H.alloc_bm[T].lvl[0] + at));
-    return DSR_BULK_HOLES * __reduce_add_sync(0xFFFFFFFFu, active) <= __reduce_add_sync(0xFFFFFFFFu, alloc);
+// The list of a heap, or of all heaps of a group.
+struct dsr_heap_space {
+    static constexpr bool kGroup = false;
+    const dsr_dev_heap& H;
+    __device__ __forceinline__ const dsr_dev_heap& heap(uint32_t) const { return H; }
+    __device__ __forceinline__ uint32_t count(int back) const {
+        return *(volatile uint32_t*)(H.R_count + (back ? DSR_LIST_BACK : 0));
+    }
+    __device__ __forceinline__ uint32_t at(uint32_t e, int back) const { return back ? (uint32_t)H.M - 1 - e : e; }
+    __device__ __forceinline__ uint32_t heap_of(uint32_t) const { return 0; }
+    __device__ __forceinline__ uint32_t bid(uint32_t at) const { return H.R_bid[at]; }
+    __device__ __forceinline__ dsr_u64* mask(uint32_t at) const { return H.R_mask + at; }
+    __device__ __forceinline__ bool ok(uint32_t, uint32_t b) const { return dsr_check(b < H.M, H.err, H.dbg, 10, b); }
+};
+struct dsr_group_space {
+    static constexpr bool kGroup = true;
+    const dsr_group_dev& G;
+    __device__ __forceinline__ const dsr_dev_heap& heap(uint32_t h) const { return G.heaps[h]; }
+    __device__ __forceinline__ uint32_t count(int back) const {
+        return *(volatile uint32_t*)(G.R_count + (back ? DSR_GROUP_LIST_BACK : 0));
+    }
+    __device__ __forceinline__ uint32_t at(uint32_t e, int back) const { return back ? (uint32_t)G.R_cap - 1 - e : e; }
+    __device__ __forceinline__ uint32_t heap_of(uint32_t at) const { return G.R_heap[at]; }
+    __device__ __forceinline__ uint32_t bid(uint32_t at) const { return G.R_bid[at]; }
+    __device__ __forceinline__ dsr_u64* mask(uint32_t at) const { return G.R_mask + at; }
+    __device__ __forceinline__ bool ok(uint32_t h, uint32_t b) const {
+        return dsr_check(h < G.n_slots, G.err, G.dbg, 3, h) && dsr_check(b < G.heaps[h].M, G.err, G.dbg, 4, b);
+    }
+};
+
+// Take up to k of the free slots `snap` of block b, the first ones at or after
+// slot rot, for objects of type T; returns those obtained (an earlier taker's
+// are missing). As in dsr_reserve: while slots of the block are held its type
+// is fixed, and it may not be T, if the block was emptied and reused.
+__device__ __forceinline__ dsr_u64 dsr_take(const dsr_dev_heap& H, int T, dsr_u64 b, dsr_u64 snap, int k, unsigned rot) {
+    if (!snap) return 0;
+    const dsr_u64 take = dsr_rotl(dsr_lowest_bits(dsr_rotr(snap, rot), k), rot);
+    const dsr_u64 prev = dsr_atom_and_acquire(H.obj + b, ~take);
+    const dsr_u64 got = prev & take;
+    if (!got) return 0;
+    const int T2 = dsr_block_type(H, b);
+    if (!(prev & ~take)) dsr_hb_clear(H.active_bm[T2], b, true, H.err);
+    if (T2 == T) return got;
+    dsr_release(H, T2, b, got);
+    return 0;
+}
+__device__ __forceinline__ void dsr_keep(dsr_ref* refs, uint32_t at, dsr_u64 b, dsr_u64 slots) {
+    for (; slots; slots &= slots - 1) refs[at++] = (b << 6) | (dsr_ref)(__ffsll((long long)slots) - 1);
 }
 
-// The deferred work of a CTA. Called by the whole CTA, after a barrier.
-template <class M>
-__device__ __forceinline__ void dsr_do_pending(const dsr_dev_heap& H, const typename M::Inst& I,
-                                               const typename M::Ctx& ctx, typename M::Acc& acc, dsr_later_smem& sm,
-                                               unsigned hint) {
+// Create the pending objects of a CTA. Called by the whole CTA, after a
+// barrier.
+template <class M, class Space, int MAXT>
+__device__ __forceinline__ void dsr_create_pending(const Space& S, const typename M::Args& a, uint32_t cta,
+                                                   uint32_t ctas, dsr_later_smem<MAXT>& sm, unsigned hint) {
+    constexpr int T = M::kDefers;
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const uint32_t np = sm.np;
-    if constexpr (M::kDefers >= 0) {
-        constexpr int T = M::kDefers;
-        const uint32_t cap = H.cap[T];
-        if (threadIdx.x < 32) {
-            uint32_t nb = 0;
-            if (np >= cap && cap >= 16) nb = dsr_claim_full(H, T, np / cap, hint, sm.block);
+    // the CTA's stretch of the created type's blocks, one per thread (read
+    // here and not kept: the method's loop has no registers to spare)
+    const dsr_u64 blocks = S.count(M::kDeferBack);
+    const uint32_t b0 = (uint32_t)(blocks * cta / ctas);
+    const uint32_t share = (uint32_t)(blocks * (cta + 1) / ctas) - b0;
+    uint32_t my_bid = 0, my_heap = 0xFFFFFFFFu;
+    dsr_u64 my_free = 0;
+    if (threadIdx.x < share) {
+        const uint32_t at = S.at(b0 + threadIdx.x, M::kDeferBack);
+        my_heap = S.heap_of(at);
+        my_bid = S.bid(at);
+        my_free = dsr_ld_relaxed(S.heap(my_heap).obj + my_bid);
+    }
+    for (;;) {  // one round per heap that has pending words (one round for a single heap)
+        uint32_t n = np, hp = 0;
+        if constexpr (Space::kGroup) {
             if (threadIdx.x == 0) {
+                sm.heap = 0xFFFFFFFFu;
+                sm.next = 0;
+            }
+            __syncthreads();
+            for (uint32_t p = threadIdx.x; p < np; p += blockDim.x) atomicMin(&sm.heap, (uint32_t)(sm.pending[p] >> 32));
+            __syncthreads();
+            hp = sm.heap;
+            if (hp == 0xFFFFFFFFu) break;
+            for (uint32_t p = threadIdx.x; p < np; p += blockDim.x)
+                if ((uint32_t)(sm.pending[p] >> 32) == hp) sm.index[atomicAdd(&sm.next, 1u)] = (uint16_t)p;
+            __syncthreads();
+            n = sm.next;
+            __syncthreads();  // read before it is used again
+        }
+        const dsr_dev_heap& H = S.heap(hp);
+        const uint32_t cap = H.cap[T];
+        // the CTA's holes, in thread order
+        const bool have = my_free && my_heap == hp;
+        uint32_t in_warp;
+        uint32_t before = dsr_warp_prefix(have ? (uint32_t)__popcll(my_free) : 0u, &in_warp);
+        const unsigned own = __ballot_sync(0xFFFFFFFFu, my_heap == hp);  // blocks of this heap
+        if (lane == 0) sm.holes[warp] = in_warp | ((uint32_t)__popc(own) << 16);
+        if (threadIdx.x == 0) {
+            sm.next = 0;
+            sm.nb = 0;
+            sm.n_open = 0;
+        }
+        __syncthreads();
+        uint32_t holes = 0, own_blocks = 0;
+        for (unsigned w = 0; w < warps; ++w) {
+            if (w == warp) before += holes;
+            holes += sm.holes[w] & 0xFFFFu;
+            own_blocks += sm.holes[w] >> 16;
+        }
+        const uint32_t from_holes = n < holes ? n : holes;
+        const uint32_t rest = n - from_holes;
+        // beyond the holes: whole blocks, claimed by the first warp, and the
+        // remainder, placed by the last
+        if (warp == 0 && rest >= cap && cap >= 16) {
+            const uint32_t nb = dsr_claim_full(H, T, rest / cap, hint, sm.block);
+            if (lane == 0) {
                 sm.nb = nb;
                 if (nb) dsr_count(H.ctr, DSR_CTR_ALLOCS, (dsr_u64)nb * cap);
             }
         }
-        __syncthreads();
-        const uint32_t full = sm.nb * cap;
-        for (uint32_t p0 = threadIdx.x & ~31u; p0 < np; p0 += blockDim.x) {
-            __syncwarp();
-            const uint32_t p = p0 + (threadIdx.x & 31);
-            if (p < np) {
-                const dsr_ref r = p < full ? ((dsr_ref)sm.block[p / cap] << 6) | (p % cap) : dsr_new(H, T);
-                M::born(H, I, ctx, sm.pending[p], r, acc);
+        const uint32_t rem = cap >= 16 ? rest % cap : rest < DSR_OPEN_SHARE ? rest : 0;
+        if (warp == warps - 1 && lane == 0 && rem && !*(volatile uint32_t*)H.inject) {
+            uint32_t left = rem;
+            for (unsigned t = 0; t < 2 && left; ++t) {
+                const unsigned h = dsr_hash32(hint ^ (t + 1) * 0x5bd1e995u);
+                const long long b = dsr_hb_find(H.active_bm[T], h);
+                if (b < 0) break;
+                const dsr_u64 got = dsr_take(H, T, (dsr_u64)b, dsr_ld_relaxed(H.obj + b), (int)left, h >> 26);
+                const uint32_t n = (uint32_t)__popcll(got);
+                if (n) dsr_keep(sm.ref, atomicAdd(&sm.next, n), (dsr_u64)b, got);
+                left -= n;
+            }
+            if (left != rem) dsr_count(H.ctr, DSR_CTR_ALLOCS, rem - left);
+            if (left && own_blocks >= DSR_OPEN_SHARE) {
+                const dsr_grab g = dsr_init_block(H, T, (int)left, hint ^ 0x5bd1e995u);
+                if (!g.status) {
+                    sm.open = g.bid << 6;  // its lowest slots
+                    sm.n_open = left;
+                    dsr_count(H.ctr, DSR_CTR_ALLOCS, left);
+                }
             }
         }
-    } else {
-        for (uint32_t p0 = threadIdx.x & ~31u; p0 < np; p0 += blockDim.x) {
-            __syncwarp();
-            const uint32_t p = p0 + (threadIdx.x & 31);
-            if (p < np) M::later(H, I, ctx, sm.pending[p], acc);
+        __syncwarp();
+        // the holes, one block per thread; an earlier taker's slots are missing from `got`
+        dsr_u64 got = 0;
+        if (have && before < from_holes) {
+            got = dsr_take(H, T, my_bid, my_free, (int)(from_holes - before), 0);
         }
+        __syncwarp();
+        uint32_t served;
+        uint32_t r = dsr_warp_prefix((uint32_t)__popcll(got), &served), base = 0;
+        if (lane == 0 && served) {
+            base = atomicAdd(&sm.next, served);
+            dsr_count(H.ctr, DSR_CTR_ALLOCS, (dsr_u64)served);
+        }
+        r += __shfl_sync(0xFFFFFFFFu, base, 0);
+        dsr_keep(sm.ref, r, my_bid, got);
+        __syncthreads();
+        const uint32_t s0 = sm.next, s1 = s0 + sm.nb * cap, s2 = s1 + sm.n_open;
+        const typename M::Inst& I = M::inst(a, hp);
+        for (uint32_t q0 = threadIdx.x & ~31u; q0 < n; q0 += blockDim.x) {
+            __syncwarp();
+            const uint32_t q = q0 + lane;
+            if (q < n) {
+                dsr_ref r;
+                if (q < s0)
+                    r = sm.ref[q];
+                else if (q < s1)
+                    r = ((dsr_ref)sm.block[(q - s0) / cap] << 6) | ((q - s0) % cap);
+                else if (q < s2)
+                    r = sm.open + (q - s1);
+                else
+                    r = dsr_new(H, T);
+                const uint32_t p = Space::kGroup ? sm.index[q] : q;
+                const dsr_u64 word = sm.pending[p];
+                if (Space::kGroup) sm.pending[p] = ~0ull;
+                M::born(H, I, Space::kGroup ? (dsr_u64)(uint32_t)word : word, r);
+            }
+        }
+        __syncthreads();
+        if (!Space::kGroup) break;
     }
-    __syncthreads();
     if (threadIdx.x == 0) sm.np = 0;
     __syncthreads();
 }
@@ -135,56 +287,51 @@ __device__ __forceinline__ void dsr_flush_count(const dsr_dev_heap& H, unsigned 
     if (dsr_lane() == 0 && v) dsr_count(H.ctr, k, v);
 }
 
-// A do-all over one list of a heap; called by the whole grid. `turn`: the
-// warps take items from the other end, so that those with the fewest items of
-// a do-all before this one in the same launch get the first of this one's.
-template <class M>
-__device__ __forceinline__ void dsr_run_list(const dsr_dev_heap& H, const dsr_phase& ph, const typename M::Args& a,
-                                             bool turn, dsr_later_smem* sm) {
-    const unsigned lane = threadIdx.x & 31;
+// A do-all over one list; called by the whole grid. hsh: log2 of the 32-slot
+// items of a listed block. `turn`: the CTAs take the stretches in reverse
+// order, so that those with the most work in a do-all before this one in the
+// same launch do not have the most again.
+template <class M, class Space, int MAXT>
+__device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph, const typename M::Args& a,
+                                             unsigned hsh, bool turn, dsr_later_smem<MAXT>* sm) {
+    const unsigned lane = threadIdx.x & 31, warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const int T = ph.type;
-    const unsigned hsh = H.span_sh[T] - 5;  // log2 of the 32-slot items of a block
-    const uint32_t W = gridDim.x * (blockDim.x >> 5);
-    const uint32_t w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const uint32_t w = turn ? W - 1 - w0 : w0;
-    // 32 bits hold the items of any heap: a block of more than 32 slots has
-    // at least 256 bytes, a smaller one 128 and one item
-    const uint32_t items = *(volatile uint32_t*)(H.R_count + (ph.back ? DSR_LIST_BACK : 0)) << hsh;
-    const typename M::Inst& I = M::inst(a, 0);
-    const typename M::Ctx ctx = M::begin(I);
-    typename M::Acc acc{};
-    dsr_later later{sm, true};
-    if constexpr (M::kDefers >= 0) {
-        if (threadIdx.x < 32) {
-            const bool few = dsr_few_holes(H, M::kDefers, blockIdx.x);
-            if (threadIdx.x == 0) {
-                sm->few = few;
-                sm->np = 0;
-            }
-        }
-        __syncthreads();
-        later.on = sm->few != 0;
-    } else if constexpr (M::kDefers == DSR_WORK) {
+    const uint32_t cta = turn ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const dsr_u64 items = (dsr_u64)S.count(ph.back) << hsh;
+    // the CTA's stretch: below 2^32 items in all, as a block of more than 32
+    // slots has at least 256 bytes, and one with fewer is one item. Few items
+    // go to few CTAs, one to a warp: what a CTA defers is then worth a block.
+    const dsr_u64 wanted = (items + warps - 1) / warps;
+    const uint32_t ctas = wanted < gridDim.x ? (uint32_t)wanted : gridDim.x;
+    const uint32_t first = cta < ctas ? (uint32_t)(items * cta / ctas) : 0u;
+    const uint32_t last = cta < ctas ? (uint32_t)(items * (cta + 1) / ctas) : 0u;
+    dsr_later later{nullptr, nullptr, 0, M::kDefers != DSR_NOTHING};
+    if constexpr (M::kDefers != DSR_NOTHING) {
+        later.np = &sm->np;
+        later.pending = sm->pending;
         if (threadIdx.x == 0) sm->np = 0;
         __syncthreads();
     }
     // with deferral, CTAs meet after so many items of every warp that the
     // pending words cannot overflow
-    const uint32_t burst = M::kDefers == DSR_NOTHING ? 32u : DSR_PENDING / 2 / blockDim.x;
-    for (uint32_t base = 0; base < items; base += 32 * W) {  // uniform over the grid
+    constexpr uint32_t kHalf = dsr_later_smem<MAXT>::PENDING / 2;
+    const uint32_t burst = M::kDefers == DSR_NOTHING ? 32u : kHalf / blockDim.x;
+    typename M::Acc acc{};
+    typename M::Ctx ctx{};
+    if (!Space::kGroup) ctx = M::begin(M::inst(a, 0));
+    for (uint32_t base = first; base < last; base += 32 * warps) {  // uniform over the CTA
         // lane k holds the warp's k-th item from here
-        const uint32_t mine = base + lane * W + w;
-        uint32_t bid = 0, live = 0, half = 0;
-        uint32_t at = 0;
-        if (mine < items) {
-            const uint32_t e = mine >> hsh;
-            half = mine & ((1u << hsh) - 1);
-            at = ph.back ? (uint32_t)H.M - 1 - e : e;
-            bid = H.R_bid[at];
-            live = reinterpret_cast<const uint32_t*>(H.R_mask + at)[half];
+        const uint32_t item = base + lane * warps + warp;
+        uint32_t bid = 0, live = 0, half = 0, at = 0, heap = 0;
+        if (item < last) {
+            half = item & ((1u << hsh) - 1);
+            at = S.at(item >> hsh, ph.back);
+            heap = S.heap_of(at);
+            bid = S.bid(at);
+            live = reinterpret_cast<const uint32_t*>(S.mask(at))[half];
         }
         for (uint32_t k0 = 0; k0 < 32; k0 += burst) {
-            if (base + k0 * W >= items) break;  // uniform over the grid
+            if (base + k0 * warps >= last) break;  // uniform over the CTA
             for (uint32_t k = k0; k < k0 + burst && k < 32; ++k) {
                 // reconverge: lanes that drifted apart in a method would
                 // otherwise miss each other at warp-wide steps
@@ -193,26 +340,68 @@ __device__ __forceinline__ void dsr_run_list(const dsr_dev_heap& H, const dsr_ph
                 if (!m) continue;
                 const uint32_t b = __shfl_sync(0xFFFFFFFFu, bid, k);
                 const uint32_t hf = __shfl_sync(0xFFFFFFFFu, half, k);
+                const uint32_t h = Space::kGroup ? __shfl_sync(0xFFFFFFFFu, heap, k) : 0u;
+                if (!S.ok(h, b)) continue;
+                const dsr_dev_heap& H = S.heap(h);
+                const typename M::Inst& I = M::inst(a, h);
+                if (Space::kGroup) {
+                    ctx = M::begin(I);
+                    later.tag = (dsr_u64)h << 32;
+                }
                 unsigned mark = 0;
                 if ((m >> lane) & 1u) mark = M::run(H, T, I, ctx, ((dsr_u64)b << 6) | (32 * hf + lane), later, acc);
+                if (Space::kGroup || M::kMarks) __syncwarp();
                 if (M::kMarks) {
                     mark = __ballot_sync(0xFFFFFFFFu, mark);
-                    if (lane == k) reinterpret_cast<uint32_t*>(H.R_mask + at)[half] = mark;
+                    if (lane == k) reinterpret_cast<uint32_t*>(S.mask(at))[half] = mark;
+                }
+                if (Space::kGroup) {
+                    M::flush(H, I, acc);
+                    acc = typename M::Acc{};
                 }
             }
             if constexpr (M::kDefers != DSR_NOTHING) {
                 // the last thread to arrive sees every push: all decide alike
-                if (__syncthreads_or(*(volatile uint32_t*)&sm->np > DSR_PENDING / 2)) dsr_do_pending<M>(H, I, ctx, acc, *sm, dsr_hash32(blockIdx.x + k0));
+                if (__syncthreads_or(*(volatile uint32_t*)&sm->np > kHalf)) {
+                    if constexpr (M::kDefers >= 0)
+                        dsr_create_pending<M, Space, MAXT>(S, a, cta, ctas, *sm, dsr_hash32(cta + k0 * 0x85EBCA77u));
+                    else
+                        M::template later_all<MAXT>(S.heap(0), M::inst(a, 0), ctx, acc, *sm);
+                }
             }
         }
     }
     if constexpr (M::kDefers != DSR_NOTHING) {
         __syncthreads();
-        if (sm->np) dsr_do_pending<M>(H, I, ctx, acc, *sm, dsr_hash32(blockIdx.x * 0x9E3779B1u));
+        if (sm->np) {
+            if constexpr (M::kDefers >= 0)
+                dsr_create_pending<M, Space, MAXT>(S, a, cta, ctas, *sm, dsr_hash32(cta * 0x9E3779B1u));
+            else
+                M::template later_all<MAXT>(S.heap(0), M::inst(a, 0), ctx, acc, *sm);
+        }
         __syncthreads();
     }
-    __syncwarp();
-    M::flush(H, I, acc);
+    if (!Space::kGroup) {
+        __syncwarp();
+        M::flush(S.heap(0), M::inst(a, 0), acc);
+    }
+}
+
+// later_all of a DSR_WORK method: M::later for every pending word, by full
+// warps. Called by the whole CTA, after a barrier.
+template <class M, int MAXT>
+__device__ __forceinline__ void dsr_work_pending(const dsr_dev_heap& H, const typename M::Inst& I,
+                                                 const typename M::Ctx& ctx, typename M::Acc& acc,
+                                                 dsr_later_smem<MAXT>& sm) {
+    const uint32_t np = sm.np;
+    for (uint32_t p0 = threadIdx.x & ~31u; p0 < np; p0 += blockDim.x) {
+        __syncwarp();
+        const uint32_t p = p0 + (threadIdx.x & 31);
+        if (p < np) M::later(H, I, ctx, sm.pending[p], acc);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) sm.np = 0;
+    __syncthreads();
 }
 
 // End of a step's last do-all: true in every thread of the last CTA.
@@ -231,28 +420,55 @@ __device__ __forceinline__ bool dsr_last_cta(uint32_t* done) {
 
 // One do-all, or two that do not depend on each other. END: the last of the
 // step (its last CTA empties the lists). F: a type whose finish(H, args) that
-// CTA's first thread runs.
+// CTA's first thread runs (finish_group: all its threads).
 template <class M1, class M2, bool END, class F, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 6 : 1)
     dsr_step_kernel(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ dsr_phase p1,
                     const __grid_constant__ dsr_phase p2, const __grid_constant__ typename M1::Args a) {
-    constexpr bool two = !std::is_same<M2, dsr_no_method>::value;
-    constexpr int defers = M1::kDefers;
-    dsr_later_smem* sm = nullptr;
-    if constexpr (defers != DSR_NOTHING) {
-        __shared__ dsr_later_smem later;
+    dsr_later_smem<MAXT>* sm = nullptr;
+    if constexpr (M1::kDefers != DSR_NOTHING) {
+        __shared__ dsr_later_smem<MAXT> later;
         sm = &later;
     }
-    dsr_run_list<M1>(H, p1, a, false, sm);
-    if constexpr (two) {
-        static_assert(M2::kDefers == DSR_NOTHING || defers != DSR_NOTHING, "M2 uses M1's shared memory");
-        dsr_run_list<M2>(H, p2, a, true, sm);
+    const dsr_heap_space S{H};
+    dsr_run_list<M1, dsr_heap_space, MAXT>(S, p1, a, H.span_sh[p1.type] - 5, false, sm);
+    if constexpr (!std::is_same<M2, dsr_no_method>::value) {
+        static_assert(M2::kDefers == DSR_NOTHING, "only the first do-all of a launch defers");
+        dsr_run_list<M2, dsr_heap_space, MAXT>(S, p2, a, H.span_sh[p2.type] - 5, true, nullptr);
     }
     if constexpr (END) {
         if (dsr_last_cta(H.R_done) && threadIdx.x == 0) {
             *(volatile uint32_t*)H.R_count = 0;
             *(volatile uint32_t*)(H.R_count + DSR_LIST_BACK) = 0;
             if constexpr (!std::is_same<F, dsr_no_method>::value) F::finish(H, a);
+        }
+    }
+}
+
+template <class M1, class M2, bool END, class F, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 6 : 1)
+    dsr_group_step_kernel(const __grid_constant__ dsr_group_dev G, const __grid_constant__ dsr_phase p1,
+                          const __grid_constant__ dsr_phase p2, const __grid_constant__ typename M1::Args a,
+                          unsigned hsh1, unsigned hsh2) {
+    static_assert(M1::kDefers != DSR_WORK, "group do-alls defer creations only");
+    dsr_later_smem<MAXT>* sm = nullptr;
+    if constexpr (M1::kDefers != DSR_NOTHING) {
+        __shared__ dsr_later_smem<MAXT> later;
+        sm = &later;
+    }
+    const dsr_group_space S{G};
+    dsr_run_list<M1, dsr_group_space, MAXT>(S, p1, a, hsh1, false, sm);
+    if constexpr (!std::is_same<M2, dsr_no_method>::value) {
+        static_assert(M2::kDefers == DSR_NOTHING, "only the first do-all of a launch defers");
+        dsr_run_list<M2, dsr_group_space, MAXT>(S, p2, a, hsh2, true, nullptr);
+    }
+    if constexpr (END) {
+        if (dsr_last_cta(G.R_done)) {
+            if (threadIdx.x == 0) {
+                *(volatile uint32_t*)G.R_count = 0;
+                *(volatile uint32_t*)(G.R_count + DSR_GROUP_LIST_BACK) = 0;
+            }
+            if constexpr (!std::is_same<F, dsr_no_method>::value) F::finish_group(G, a);
         }
     }
 }
@@ -283,80 +499,6 @@ int dsr__step(dsr_heap* h, const dsr_phase& p1, const dsr_phase& p2, const typen
     return dsr__check_launch("dsr_step_kernel");
 }
 
-// Queue the listing of type A (front) and, unless -1, type B (back). mult:
-// visits counted per listed object.
-void dsr__list_types(const dsr_heap* h, int type_a, int type_b, unsigned mult_a, unsigned mult_b, cudaStream_t s);
-
-// ---- heap groups -------------------------------------------------------------
-// The same over the heaps of a group: G.R_heap / R_bid / R_mask hold the
-// entries of all heaps, type A's from the front and type B's from the back.
-constexpr int DSR_GROUP_LIST_BACK = 32;  // index from G.R_count of the back's count
-
-template <class M>
-__device__ __forceinline__ void dsr_run_group_list(const dsr_group_dev& G, const dsr_phase& ph,
-                                                   const typename M::Args& a, unsigned hsh, bool turn) {
-    const unsigned lane = threadIdx.x & 31;
-    const int T = ph.type;
-    const uint32_t W = gridDim.x * (blockDim.x >> 5);
-    const uint32_t w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const uint32_t w = turn ? W - 1 - w0 : w0;
-    const uint32_t items = *(volatile uint32_t*)(G.R_count + (ph.back ? DSR_GROUP_LIST_BACK : 0)) << hsh;
-    dsr_later later{nullptr, false};
-    for (uint32_t base = 0; base < items; base += 32 * W) {
-        const uint32_t mine = base + lane * W + w;
-        uint32_t bid = 0, live = 0, half = 0, heap = 0;
-        uint32_t at = 0;
-        if (mine < items) {
-            const uint32_t e = mine >> hsh;
-            half = mine & ((1u << hsh) - 1);
-            at = ph.back ? (uint32_t)G.R_cap - 1 - e : e;
-            heap = G.R_heap[at];
-            bid = G.R_bid[at];
-            live = reinterpret_cast<const uint32_t*>(G.R_mask + at)[half];
-        }
-        for (uint32_t k = 0; k < 32; ++k) {
-            if (base + k * W >= items) break;
-            __syncwarp();
-            const uint32_t m = __shfl_sync(0xFFFFFFFFu, live, k);
-            if (!m) continue;
-            const uint32_t b = __shfl_sync(0xFFFFFFFFu, bid, k);
-            const uint32_t h = __shfl_sync(0xFFFFFFFFu, heap, k);
-            const uint32_t hf = __shfl_sync(0xFFFFFFFFu, half, k);
-            if (!dsr_check(h < G.n_slots, G.err, G.dbg, 3, h) || !dsr_check(b < G.heaps[h].M, G.err, G.dbg, 4, b)) continue;
-            const dsr_dev_heap& H = G.heaps[h];
-            const typename M::Inst& I = M::inst(a, h);
-            const typename M::Ctx ctx = M::begin(I);
-            typename M::Acc acc{};
-            unsigned mark = 0;
-            if ((m >> lane) & 1u) mark = M::run(H, T, I, ctx, ((dsr_u64)b << 6) | (32 * hf + lane), later, acc);
-            __syncwarp();
-            if (M::kMarks) {
-                mark = __ballot_sync(0xFFFFFFFFu, mark);
-                if (lane == k) reinterpret_cast<uint32_t*>(G.R_mask + at)[half] = mark;
-            }
-            M::flush(H, I, acc);
-        }
-    }
-}
-
-template <class M1, class M2, bool END, class F, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 6 : 1)
-    dsr_group_step_kernel(const __grid_constant__ dsr_group_dev G, const __grid_constant__ dsr_phase p1,
-                          const __grid_constant__ dsr_phase p2, const __grid_constant__ typename M1::Args a,
-                          unsigned hsh1, unsigned hsh2) {
-    dsr_run_group_list<M1>(G, p1, a, hsh1, false);
-    if constexpr (!std::is_same<M2, dsr_no_method>::value) dsr_run_group_list<M2>(G, p2, a, hsh2, true);
-    if constexpr (END) {
-        if (dsr_last_cta(G.R_done)) {
-            if (threadIdx.x == 0) {
-                *(volatile uint32_t*)G.R_count = 0;
-                *(volatile uint32_t*)(G.R_count + DSR_GROUP_LIST_BACK) = 0;
-            }
-            if constexpr (!std::is_same<F, dsr_no_method>::value) F::finish_group(G, a);
-        }
-    }
-}
-
 template <class M1, class M2 = dsr_no_method, bool END = false, class F = dsr_no_method>
 int dsr__group_step(dsr_group* g, const dsr_phase& p1, const dsr_phase& p2, const typename M1::Args& a,
                     cudaStream_t s) {
@@ -372,5 +514,8 @@ int dsr__group_step(dsr_group* g, const dsr_phase& p1, const dsr_phase& p2, cons
     return dsr__check_launch("dsr_group_step_kernel");
 }
 
+// Queue the listing of type A (front) and, unless -1, type B (back). mult:
+// visits counted per listed object.
+void dsr__list_types(const dsr_heap* h, int type_a, int type_b, unsigned mult_a, unsigned mult_b, cudaStream_t s);
 void dsr__group_list_types(const dsr_group* g, int type_a, int type_b, unsigned mult_a, unsigned mult_b,
                            cudaStream_t s);

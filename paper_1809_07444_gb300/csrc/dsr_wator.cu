@@ -338,14 +338,13 @@ struct DFishChoose : WatorMethod<A> {
 };
 template <class A>
 struct DFishMove : WatorMove<A> {
-    enum { kDefers = FISH };
+    enum { kDefers = FISH, kDeferBack = 0 };
     static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const WatorInst& I, NoCtx, dsr_ref s,
                                                    dsr_later& later, unsigned& moves) {
         fish_move(H, I, s, Defer{later, moves});
         return 0;
     }
-    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const WatorInst& I, NoCtx, dsr_u64 c, dsr_ref r,
-                                                unsigned&) {
+    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const WatorInst& I, dsr_u64 c, dsr_ref r) {
         fish_born(H, I, (uint32_t)c, r);
     }
 };
@@ -376,14 +375,13 @@ struct DSharkChoose : WatorMethod<A> {
 };
 template <class A>
 struct DSharkMove : WatorMove<A> {
-    enum { kDefers = SHARK };
+    enum { kDefers = SHARK, kDeferBack = 1 };
     static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const WatorInst& I, NoCtx, dsr_ref s,
                                                    dsr_later& later, unsigned& moves) {
         shark_move(H, I, s, Defer{later, moves});
         return 0;
     }
-    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const WatorInst& I, NoCtx, dsr_u64 c, dsr_ref r,
-                                                unsigned&) {
+    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const WatorInst& I, dsr_u64 c, dsr_ref r) {
         shark_born(H, I, (uint32_t)c, r);
     }
 };
