@@ -728,35 +728,94 @@ struct MClone {
     }
 };
 
-struct DumpArgs {
-    uint32_t* out;
-    dsr_u64* count;
-    dsr_u64 cap;
-    int row;
-};
-struct MDump {
-    typedef DumpArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int T, const Args& a, dsr_ref r) {
-        const dsr_u64 k = atomicAdd(a.count, 1ull);
-        if (k >= a.cap) {
-            atomicOr(H.err, DSR_ERR_CAPACITY);
-            return;
+// Rows of the live objects of type T (dsr_heap_dump) over the block list R,
+// which the last CTA then empties. A row is shorter than the 32-byte sectors
+// it lies in, so a warp gathers its rows in shared memory and writes them out
+// word by word in order; and a CTA takes its rows' places with one atomic for
+// 32 items of 32 slots (one per warp and item queues up on the counter:
+// 6.7 M cars 160 -> 93 us).
+constexpr int DUMP_ITEMS = 4;   // items of a warp at a time (fewer in a short list)
+constexpr int DUMP_ROW = 2 * DSR_MAX_FIELDS + 2;
+__global__ void __launch_bounds__(256) k_dump(const __grid_constant__ dsr_dev_heap H, int T, uint32_t* out,
+                                              dsr_u64* count, dsr_u64 cap, int row) {
+    __shared__ uint32_t stage[8][32 * DUMP_ROW];
+    __shared__ uint32_t warp_n[8];
+    __shared__ dsr_u64 cta_base;
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned hsh = H.span_sh[T] - 5;
+    const dsr_u64 items = (dsr_u64)(*(volatile uint32_t*)H.R_count) << hsh;
+    const uint32_t nf = H.n_fields[T];
+    bool words = true;  // every field has 4 bytes
+    for (uint32_t f = 0; f < nf; ++f) words = words && H.fsize[T][f] == 4;
+    const dsr_u64 share = items / ((dsr_u64)gridDim.x * 8);
+    const unsigned per = share < 1 ? 1u : (share < DUMP_ITEMS ? (unsigned)share : (unsigned)DUMP_ITEMS);
+    uint32_t* mine = stage[warp];
+    for (dsr_u64 base = (dsr_u64)blockIdx.x * 8 * per; base < items; base += (dsr_u64)gridDim.x * 8 * per) {
+        // lane k < per holds the warp's k-th item
+        const dsr_u64 item = base + warp * per + lane;
+        uint32_t bid = 0, live = 0;
+        if (lane < per && item < items) {
+            bid = H.R_bid[item >> hsh];
+            live = (uint32_t)(H.R_mask[item >> hsh] >> (32 * (item & ((1u << hsh) - 1))));
         }
-        uint32_t* row = a.out + k * (dsr_u64)a.row;
-        int w = 0;
-        for (uint32_t f = 0; f < H.n_fields[T]; ++f) {
-            if (H.fsize[T][f] == 4) {
-                row[w++] = *dsr_field<uint32_t>(H, T, r, (int)f);
-            } else {
-                const dsr_u64 x = *dsr_field<dsr_u64>(H, T, r, (int)f);
-                row[w++] = (uint32_t)x;
-                row[w++] = (uint32_t)(x >> 32);
+        const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(live));
+        if (lane == 0) warp_n[warp] = n;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t total = 0;
+            for (int w = 0; w < 8; ++w) {
+                const uint32_t k = warp_n[w];
+                warp_n[w] = total;
+                total += k;
             }
+            cta_base = total ? atomicAdd(count, (dsr_u64)total) : 0;
+            if (cta_base + total > cap) atomicOr(H.err, DSR_ERR_CAPACITY);
         }
-        row[w++] = (uint32_t)r;
-        row[w++] = (uint32_t)(r >> 32);
+        __syncthreads();
+        dsr_u64 at = cta_base + warp_n[warp];
+        for (unsigned k = 0; k < per; ++k) {
+            const uint32_t m = __shfl_sync(0xFFFFFFFFu, live, k), b = __shfl_sync(0xFFFFFFFFu, bid, k);
+            if (!m) continue;
+            const unsigned half = (unsigned)((base + warp * per + k) & ((1u << hsh) - 1));
+            if ((m >> lane) & 1u) {
+                const dsr_ref r = ((dsr_u64)b << 6) | (32 * half + lane);
+                uint32_t* w = mine + __popc(m & ((1u << lane) - 1)) * row;
+                if (words) {
+                    for (uint32_t f = 0; f < nf; f += 4) {  // four fields in flight
+                        uint32_t v[4];
+#pragma unroll
+                        for (uint32_t u = 0; u < 4; ++u)
+                            if (f + u < nf) v[u] = *dsr_field<uint32_t>(H, T, r, (int)(f + u));
+#pragma unroll
+                        for (uint32_t u = 0; u < 4; ++u)
+                            if (f + u < nf) w[f + u] = v[u];
+                    }
+                    w += nf;
+                } else {
+                    for (uint32_t f = 0; f < nf; ++f) {
+                        if (H.fsize[T][f] == 4) {
+                            *w++ = *dsr_field<uint32_t>(H, T, r, (int)f);
+                        } else {
+                            const dsr_u64 x = *dsr_field<dsr_u64>(H, T, r, (int)f);
+                            *w++ = (uint32_t)x;
+                            *w++ = (uint32_t)(x >> 32);
+                        }
+                    }
+                }
+                *w++ = (uint32_t)r;
+                *w++ = (uint32_t)(r >> 32);
+            }
+            __syncwarp();
+            const dsr_u64 rows = at >= cap ? 0 : (cap - at < (dsr_u64)__popc(m) ? cap - at : (dsr_u64)__popc(m));
+            uint32_t* to = out + at * (dsr_u64)row;
+            for (uint32_t i = lane; i < (uint32_t)rows * row; i += 32) to[i] = mine[i];
+            at += __popc(m);
+            __syncwarp();  // the staged rows are read before the next item's replace them
+        }
+        __syncthreads();
     }
-};
+    dsr_doall_finish(H);
+}
 
 struct HashArgs {
     dsr_u64* out;
@@ -800,8 +859,13 @@ extern "C" int dsr_heap_dump(dsr_heap* h, int type, void* out_dev, uint64_t cap,
         dsr__set_cuda_error(e, "dsr_heap_dump");
         return DSR_E_CUDA;
     }
-    DumpArgs a{static_cast<uint32_t*>(out_dev), static_cast<dsr_u64*>(count_dev), cap, dsr_row_words(h, type)};
-    return dsr__doall<MDump>(h, type, a, s, true, nullptr, nullptr, 0, true);
+    dsr__launch_scan(h, type, s, 1, true);
+    const dsr_u64 most = (h->dev.M * 2 + 8 * DUMP_ITEMS - 1) / (8 * DUMP_ITEMS);
+    const dsr_u64 grid = (dsr_u64)h->sm_count * 5;
+    k_dump<<<(unsigned)(grid < most ? grid : most), 256, 0, s>>>(h->dev, type, static_cast<uint32_t*>(out_dev),
+                                                                 static_cast<dsr_u64*>(count_dev), cap,
+                                                                 dsr_row_words(h, type));
+    return dsr__check_launch("k_dump");
 }
 
 extern "C" int dsr_heap_hash(dsr_heap* h, int type, void* hash_dev, void* stream) {

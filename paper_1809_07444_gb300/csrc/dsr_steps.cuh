@@ -10,10 +10,11 @@
 // entry's mask by the survivors (kMarks) where a later do-all of the step
 // visits them. Two do-alls that do not depend on each other share a launch.
 //
-// Every CTA has one stretch of the list, of (block, 32 slots) items as equal
-// in number as can be; its warps take them in turn. A warp's 32 lanes load
-// the entries of its next 32 items at once and hand them out by shuffle, so
-// the list costs one round trip per 32 items and warp, not one per item.
+// A warp takes every W-th (block, 32 slots) item of a heap's list, so that at
+// any time the grid works on neighbouring entries; a CTA of a group do-all takes
+// one stretch, which lies in one or two heaps. A warp's 32 lanes load the entries of its next 32
+// items at once and hand them out by shuffle, so the list costs one round
+// trip per 32 items and warp, not one per item.
 //
 // Deferred work. A method may put off an object's creation: it pushes a
 // word, and the CTA later creates all pending objects together and calls
@@ -287,6 +288,22 @@ __device__ __forceinline__ void dsr_flush_count(const dsr_dev_heap& H, unsigned 
     if (dsr_lane() == 0 && v) dsr_count(H.ctr, k, v);
 }
 
+// M::later for every pending word of a DSR_WORK method, by full warps. Called by the whole CTA, after a barrier.
+template <class M, int MAXT>
+__device__ __forceinline__ void dsr_work_pending(const dsr_dev_heap& H, const typename M::Inst& I,
+                                                 const typename M::Ctx& ctx, typename M::Acc& acc,
+                                                 dsr_later_smem<MAXT>& sm) {
+    const uint32_t np = sm.np;
+    for (uint32_t p0 = threadIdx.x & ~31u; p0 < np; p0 += blockDim.x) {
+        __syncwarp();
+        const uint32_t p = p0 + (threadIdx.x & 31);
+        if (p < np) M::later(H, I, ctx, sm.pending[p], acc);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) sm.np = 0;
+    __syncthreads();
+}
+
 // A do-all over one list; called by the whole grid. hsh: log2 of the 32-slot
 // items of a listed block. `turn`: the CTAs take the stretches in reverse
 // order, so that those with the most work in a do-all before this one in the
@@ -303,8 +320,10 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
     // go to few CTAs, one to a warp: what a CTA defers is then worth a block.
     const dsr_u64 wanted = (items + warps - 1) / warps;
     const uint32_t ctas = wanted < gridDim.x ? (uint32_t)wanted : gridDim.x;
-    const uint32_t first = cta < ctas ? (uint32_t)(items * cta / ctas) : 0u;
-    const uint32_t last = cta < ctas ? (uint32_t)(items * (cta + 1) / ctas) : 0u;
+    // items first, first + 1 .. (groups) or first, first + stride .. of this warp
+    const uint32_t end = Space::kGroup ? (uint32_t)(cta < ctas ? items * (cta + 1) / ctas : 0) : (uint32_t)items;
+    const uint32_t stride = Space::kGroup ? warps : ctas * warps;
+    const uint32_t cta0 = cta >= ctas ? end : Space::kGroup ? (uint32_t)(items * cta / ctas) : cta * warps;
     dsr_later later{nullptr, nullptr, 0, M::kDefers != DSR_NOTHING};
     if constexpr (M::kDefers != DSR_NOTHING) {
         later.np = &sm->np;
@@ -319,11 +338,11 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
     typename M::Acc acc{};
     typename M::Ctx ctx{};
     if (!Space::kGroup) ctx = M::begin(M::inst(a, 0));
-    for (uint32_t base = first; base < last; base += 32 * warps) {  // uniform over the CTA
+    for (uint32_t base = cta0; base < end; base += 32 * stride) {  // uniform over the CTA
         // lane k holds the warp's k-th item from here
-        const uint32_t item = base + lane * warps + warp;
+        const uint32_t item = base + lane * stride + warp;
         uint32_t bid = 0, live = 0, half = 0, at = 0, heap = 0;
-        if (item < last) {
+        if (item < end) {
             half = item & ((1u << hsh) - 1);
             at = S.at(item >> hsh, ph.back);
             heap = S.heap_of(at);
@@ -331,7 +350,7 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
             live = reinterpret_cast<const uint32_t*>(S.mask(at))[half];
         }
         for (uint32_t k0 = 0; k0 < 32; k0 += burst) {
-            if (base + k0 * warps >= last) break;  // uniform over the CTA
+            if (base + k0 * stride >= end) break;  // uniform over the CTA
             for (uint32_t k = k0; k < k0 + burst && k < 32; ++k) {
                 // reconverge: lanes that drifted apart in a method would
                 // otherwise miss each other at warp-wide steps
@@ -366,7 +385,7 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
                     if constexpr (M::kDefers >= 0)
                         dsr_create_pending<M, Space, MAXT>(S, a, cta, ctas, *sm, dsr_hash32(cta + k0 * 0x85EBCA77u));
                     else
-                        M::template later_all<MAXT>(S.heap(0), M::inst(a, 0), ctx, acc, *sm);
+                        dsr_work_pending<M, MAXT>(S.heap(0), M::inst(a, 0), ctx, acc, *sm);
                 }
             }
         }
@@ -377,7 +396,7 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
             if constexpr (M::kDefers >= 0)
                 dsr_create_pending<M, Space, MAXT>(S, a, cta, ctas, *sm, dsr_hash32(cta * 0x9E3779B1u));
             else
-                M::template later_all<MAXT>(S.heap(0), M::inst(a, 0), ctx, acc, *sm);
+                dsr_work_pending<M, MAXT>(S.heap(0), M::inst(a, 0), ctx, acc, *sm);
         }
         __syncthreads();
     }
@@ -385,23 +404,6 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
         __syncwarp();
         M::flush(S.heap(0), M::inst(a, 0), acc);
     }
-}
-
-// later_all of a DSR_WORK method: M::later for every pending word, by full
-// warps. Called by the whole CTA, after a barrier.
-template <class M, int MAXT>
-__device__ __forceinline__ void dsr_work_pending(const dsr_dev_heap& H, const typename M::Inst& I,
-                                                 const typename M::Ctx& ctx, typename M::Acc& acc,
-                                                 dsr_later_smem<MAXT>& sm) {
-    const uint32_t np = sm.np;
-    for (uint32_t p0 = threadIdx.x & ~31u; p0 < np; p0 += blockDim.x) {
-        __syncwarp();
-        const uint32_t p = p0 + (threadIdx.x & 31);
-        if (p < np) M::later(H, I, ctx, sm.pending[p], acc);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) sm.np = 0;
-    __syncthreads();
 }
 
 // End of a step's last do-all: true in every thread of the last CTA.
@@ -418,11 +420,19 @@ __device__ __forceinline__ bool dsr_last_cta(uint32_t* done) {
     return last;
 }
 
-// One do-all, or two that do not depend on each other. END: the last of the
+__device__ __forceinline__ void dsr_empty_lists(const dsr_dev_heap& H) {
+    *(volatile uint32_t*)H.R_count = 0;
+    *(volatile uint32_t*)(H.R_count + DSR_LIST_BACK) = 0;
+}
+
+// One do-all, or two that do not depend on each other. Five CTAs of 256 threads
+// per SM (48 registers; sugarscape 1914 -> 1854, life 1500 x 1000 1632 -> 1565 us
+// a pass against six, whose 40 registers spill); the group form, whose methods
+// wait longer for their heap's view, has six (7440 against 7524). END: the last of the
 // step (its last CTA empties the lists). F: a type whose finish(H, args) that
 // CTA's first thread runs (finish_group: all its threads).
 template <class M1, class M2, bool END, class F, int MAXT>
-__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 6 : 1)
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 5 : 1)
     dsr_step_kernel(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ dsr_phase p1,
                     const __grid_constant__ dsr_phase p2, const __grid_constant__ typename M1::Args a) {
     dsr_later_smem<MAXT>* sm = nullptr;
@@ -438,8 +448,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 6 : 1)
     }
     if constexpr (END) {
         if (dsr_last_cta(H.R_done) && threadIdx.x == 0) {
-            *(volatile uint32_t*)H.R_count = 0;
-            *(volatile uint32_t*)(H.R_count + DSR_LIST_BACK) = 0;
+            dsr_empty_lists(H);
             if constexpr (!std::is_same<F, dsr_no_method>::value) F::finish(H, a);
         }
     }

@@ -18,7 +18,7 @@
 // no car reads a cell another car writes: the do-all needs no atomics. After
 // the step `cur` is cleared and the grids swap.
 #include "dsr_apps.h"
-#include "dsr_bulk.cuh"
+#include "dsr_steps.cuh"
 
 namespace {
 enum { CAR = 0, SOURCE = 1 };
@@ -27,10 +27,10 @@ enum { S_ROAD = 0, S_ENTERED = 1, S_BLOCKED = 2 };  // Source
 enum { CTR_ENTERED = DSR_CTR_APP0, CTR_LEFT, CTR_MOVED, CTR_VSUM };
 
 struct TrafficArgs {
-    const uint8_t* cur;  // [R * L] occupancy at the start of the step
-    uint8_t* next;       // [R * L] occupancy after the step (zero on entry)
+    uint8_t* cur;   // [R * L] occupancy at the start of the step
+    uint8_t* next;  // [R * L] occupancy after the step (zero on entry)
     dsr_traffic_params p;
-    dsr_u64 step;
+    dsr_u64 slow_key, enter_key;  // dsr_rand_key of this step's draws (streams 5 and 6)
 };
 
 __device__ __forceinline__ int32_t* fld(const dsr_dev_heap& H, int T, dsr_ref r, int f) {
@@ -39,67 +39,117 @@ __device__ __forceinline__ int32_t* fld(const dsr_dev_heap& H, int T, dsr_ref r,
 
 __device__ __forceinline__ bool draws_below(dsr_u64 r, dsr_u64 thr) { return (r >> 32) < thr; }
 
-struct MCar {
+// Free cells among the n cells from `cell` on, before the first car: eight
+// cells a load. The grid is an array of 8-byte words (its length is a
+// multiple of 256), so the words that hold any of these cells are inside it;
+// cells read beyond the n are masked out.
+__device__ __forceinline__ int32_t free_run(const uint8_t* grid, dsr_u64 cell, int32_t n) {
+    int32_t g = 0;
+    while (g < n) {
+        const dsr_u64 at = cell + (uint32_t)g;
+        const dsr_u64* w = reinterpret_cast<const dsr_u64*>(grid) + (at >> 3);
+        const unsigned off = (unsigned)at & 7u;
+        int32_t k = n - g < 8 ? n - g : 8;
+        dsr_u64 v = w[0] >> (8 * off);
+        if (off + (unsigned)k > 8u) v |= w[1] << (64 - 8 * off);
+        if (k < 8) v &= (1ull << (8 * k)) - 1;
+        if (v) return g + ((__ffsll((long long)v) - 1) >> 3);
+        g += k;
+    }
+    return n;
+}
+
+struct NoCtx {};
+struct TrafficMethod {
     typedef TrafficArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref self) {
+    typedef TrafficArgs Inst;
+    typedef NoCtx Ctx;
+    enum { kDefers = DSR_NOTHING, kMarks = 0 };
+    static __device__ __forceinline__ const TrafficArgs& inst(const TrafficArgs& a, uint32_t) { return a; }
+    static __device__ __forceinline__ NoCtx begin(const TrafficArgs&) { return {}; }
+};
+
+struct Flow {
+    unsigned moved, vsum;
+};
+struct DCar : TrafficMethod {
+    typedef Flow Acc;
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const TrafficArgs& a, NoCtx,
+                                                   dsr_ref self, dsr_later&, Flow& flow) {
         const int32_t road = *fld(H, CAR, self, F_ROAD), x = *fld(H, CAR, self, F_X), v = *fld(H, CAR, self, F_V);
         const int32_t L = a.p.L;
-        const uint8_t* row = a.cur + (dsr_u64)road * L;
+        const dsr_u64 row = (dsr_u64)(uint32_t)road * (uint32_t)L;
         const int32_t v1 = v + 1 < a.p.vmax ? v + 1 : a.p.vmax;
-        int32_t g = 0;
-        for (; g < v1; ++g) {
-            int32_t ahead = x + g + 1;
-            if (ahead >= L) {
-                if (!a.p.periodic) continue;  // past the end of an open road: free
-                ahead -= L;
-            }
-            if (row[ahead]) break;
-        }
-        int32_t v3 = v1 < g ? v1 : g;
-        if (draws_below(dsr_rand(a.p.seed, 5, a.step, (dsr_u64)road * L + x), a.p.p_thr)) v3 = v3 > 0 ? v3 - 1 : 0;
-        // flow statistics: one atomic per warp for each
-        const unsigned act = __activemask();
-        const unsigned vsum = __reduce_add_sync(act, (unsigned)v3);
-        const unsigned moved = __popc(__ballot_sync(act, v3 > 0));
-        if (dsr_lane() == (unsigned)(__ffs(act) - 1)) {
-            if (moved) dsr_count(H.ctr, CTR_MOVED, moved);
-            if (vsum) dsr_count(H.ctr, CTR_VSUM, vsum);
-        }
+        // cells past the end of an open road are free; a periodic road wraps
+        const int32_t ahead = L - 1 - x < v1 ? L - 1 - x : v1;
+        int32_t g = free_run(a.cur, row + (uint32_t)x + 1, ahead);
+        if (g == ahead && ahead < v1) g = a.p.periodic ? ahead + free_run(a.cur, row, v1 - ahead) : v1;
+        int32_t v3 = g;
+        if (draws_below(dsr_splitmix_at(a.slow_key, row + (uint32_t)x), a.p.p_thr)) v3 = v3 > 0 ? v3 - 1 : 0;
+        flow.moved += v3 > 0;
+        flow.vsum += (unsigned)v3;
         int32_t nx = x + v3;
         if (nx >= L) {
             if (!a.p.periodic) {
                 dsr_count_lanes(H.ctr, CTR_LEFT);
                 dsr_delete(H, self);
-                return;
+                return 0;
             }
             nx -= L;
         }
-        a.next[(dsr_u64)road * L + nx] = 1;
+        a.next[row + (uint32_t)nx] = 1;
         *fld(H, CAR, self, F_X) = nx;
         *fld(H, CAR, self, F_V) = v3;
+        return 0;
+    }
+    static __device__ __forceinline__ void flush(const dsr_dev_heap& H, const TrafficArgs&, const Flow& f) {
+        dsr_flush_count(H, CTR_MOVED, f.moved);
+        dsr_flush_count(H, CTR_VSUM, f.vsum);
     }
 };
 
-struct MSource {
-    typedef TrafficArgs Args;
-    static __device__ void run(const dsr_dev_heap& H, int, const Args& a, dsr_ref self) {
+// An entering car is created with the others of its CTA.
+struct DSource : TrafficMethod {
+    typedef dsr_no_acc Acc;
+    enum { kDefers = CAR, kDeferBack = 0 };
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const TrafficArgs& a, NoCtx,
+                                                   dsr_ref self, dsr_later& later, dsr_no_acc&) {
         const int32_t road = *fld(H, SOURCE, self, S_ROAD);
-        uint8_t* cell0 = a.next + (dsr_u64)road * a.p.L;
-        if (*cell0) {
+        if (a.next[(dsr_u64)(uint32_t)road * (uint32_t)a.p.L]) {
             *fld(H, SOURCE, self, S_BLOCKED) += 1;
-            return;
+            return 0;
         }
-        if (!draws_below(dsr_rand(a.p.seed, 6, a.step, (dsr_u64)road), a.p.a_thr)) return;
-        const dsr_ref c = dsr_new(H, CAR);
+        if (draws_below(dsr_splitmix_at(a.enter_key, (dsr_u64)road), a.p.a_thr)) later.push(self);
+        return 0;
+    }
+    static __device__ __forceinline__ void born(const dsr_dev_heap& H, const TrafficArgs& a, dsr_u64 self, dsr_ref c) {
         if (c == DSR_NULL) return;  // out of memory: DSR_ERR_OOM is set
+        const int32_t road = *fld(H, SOURCE, self, S_ROAD);
         *fld(H, CAR, c, F_ROAD) = road;
         *fld(H, CAR, c, F_X) = 0;
         *fld(H, CAR, c, F_V) = a.p.v_entry;
-        *cell0 = 1;
+        a.next[(dsr_u64)(uint32_t)road * (uint32_t)a.p.L] = 1;
         *fld(H, SOURCE, self, S_ENTERED) += 1;
         dsr_count_lanes(H.ctr, CTR_ENTERED);
     }
+    static __device__ __forceinline__ void flush(const dsr_dev_heap&, const TrafficArgs&, dsr_no_acc) {}
 };
+
+constexpr dsr_phase kCars{CAR, 0};
+
+// The Source do-all of an open road's step, with the clearing of the old
+// occupancy, which nothing reads any more: the few CTAs that have sources
+// wait on their chains of accesses while the others write the grid.
+__global__ void __launch_bounds__(256, 5)
+    k_traffic_sources_step(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ TrafficArgs a) {
+    __shared__ dsr_later_smem<256> later;
+    dsr_run_list<DSource, dsr_heap_space, 256>(dsr_heap_space{H}, dsr_phase{SOURCE, 1}, a, H.span_sh[SOURCE] - 5, false, &later);
+    uint4* w = reinterpret_cast<uint4*>(a.cur);
+    const dsr_u64 n = ((dsr_u64)a.p.R * a.p.L + 255) / 256 * 16;
+    for (dsr_u64 i = (dsr_u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (dsr_u64)gridDim.x * blockDim.x)
+        w[i] = make_uint4(0, 0, 0, 0);
+    if (dsr_last_cta(H.R_done) && threadIdx.x == 0) dsr_empty_lists(H);
+}
 
 // One thread per cell: a Car where v0 >= 0.
 __global__ void __launch_bounds__(DSR_BULK_THREADS)
@@ -221,14 +271,27 @@ extern "C" int dsr_traffic_step(dsr_traffic* t, int n_steps, void* stream) {
     if (!t || n_steps < 0) return DSR_E_INVALID;
     cudaStream_t s = dsr__stream(stream);
     for (int i = 0; i < n_steps; ++i) {
-        TrafficArgs a{t->grid[t->cur], t->grid[1 - t->cur], t->p, t->step};
-        int rc = dsr__doall<MCar>(t->heap, CAR, a, s);
-        if (!rc && !t->p.periodic) rc = dsr__doall<MSource>(t->heap, SOURCE, a, s);
+        TrafficArgs a{t->grid[t->cur], t->grid[1 - t->cur], t->p, dsr_rand_key(t->p.seed, 5, t->step),
+                      dsr_rand_key(t->p.seed, 6, t->step)};
+        const bool open = !t->p.periodic;
+        dsr__list_types(t->heap, CAR, open ? SOURCE : -1, 1, 1, s);
+        int rc = open ? dsr__step<DCar>(t->heap, kCars, kCars, a, s)
+                      : dsr__step<DCar, dsr_no_method, true>(t->heap, kCars, kCars, a, s);
         if (rc) return rc;
-        cudaError_t e = cudaMemsetAsync(t->grid[t->cur], 0, grid_bytes(t->p), s);  // the next step's `next`
-        if (e) {
-            dsr__set_cuda_error(e, "dsr_traffic_step");
-            return DSR_E_CUDA;
+        if (open) {
+            static int per_sm = 0;
+            if (!per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traffic_sources_step, 256, 0) !=
+                                cudaSuccess || per_sm < 1))
+                per_sm = 1;
+            k_traffic_sources_step<<<per_sm * t->heap->sm_count, 256, 0, s>>>(t->heap->dev, a);
+            rc = dsr__check_launch("k_traffic_sources_step");
+            if (rc) return rc;
+        } else {
+            cudaError_t e = cudaMemsetAsync(t->grid[t->cur], 0, grid_bytes(t->p), s);  // the next step's `next`
+            if (e) {
+                dsr__set_cuda_error(e, "dsr_traffic_step");
+                return DSR_E_CUDA;
+            }
         }
         t->cur = 1 - t->cur;
         t->step += 1;
