@@ -70,7 +70,7 @@ struct dsr_dev_heap {
     uint32_t* inject;     /* slow-path allocations left to fail (fault injection) */
     uint32_t* R_bid;      /* do-all block list: block ids */
     dsr_u64* R_mask;      /* do-all block list: occupied-slot snapshot */
-    uint32_t* R_count;    /* entries in R (zero between do-alls); R_count[2]: entries at R's back (application steps) */
+    uint32_t* R_count;    /* entries in R (zero between do-alls); the words from R_count[8]: application steps */
     uint32_t* R_done;     /* CTAs of the current method kernel that finished */
     dsr_u64* ctr;         /* [DSR_CTR_SLOTS][DSR_CTR_COUNT] event counters, one row per SM */
     uint32_t* slow;       /* [DSR_MAX_TYPES] slow-path block initialisations in flight */

@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(256) k_group_list(const __grid_constant__ dsr_
     __shared__ unsigned warp_n[2][8];
     __shared__ unsigned run_base[2];
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t set = dsr_begin_step(G.R_count);
     for (uint32_t c = blockIdx.x; c < G.n_chunks; c += gridDim.x) {
         const uint32_t h = G.chunk_heap[c];
         const bool hok = dsr_check(h < G.n_slots, G.err, G.dbg, 1, c);
@@ -82,7 +83,7 @@ __global__ void __launch_bounds__(256) k_group_list(const __grid_constant__ dsr_
                 warp_n[threadIdx.x][w] = total;
                 total += n;
             }
-            run_base[threadIdx.x] = total ? atomicAdd(G.R_count + (threadIdx.x ? DSR_GROUP_LIST_BACK : 0), total) : 0;
+            run_base[threadIdx.x] = total ? atomicAdd(G.R_count + set + threadIdx.x, total) : 0;
         }
         __syncthreads();
         unsigned objs = 0;
@@ -106,8 +107,7 @@ __global__ void __launch_bounds__(256) k_group_list(const __grid_constant__ dsr_
 
 void dsr__group_list_types(const dsr_group* g, int type_a, int type_b, unsigned mult_a, unsigned mult_b,
                            cudaStream_t s) {
-    if (g->n_chunks == 0) return;
-    unsigned ctas = g->n_chunks;
+    unsigned ctas = g->n_chunks ? g->n_chunks : 1;  // an empty group's lists have length 0
     const unsigned cap = (unsigned)g->sm_count * 8;
     if (ctas > cap) ctas = cap;
     k_group_list<<<ctas, 256, 0, s>>>(g->dev, type_a, type_b, mult_a, mult_b);

@@ -252,55 +252,44 @@ __global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_he
     if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs * visits_mult);
 }
 
-// The lists of a step (dsr_steps.cuh): type A's allocated blocks from the
-// front of R, type B's (unless tb is -1) from the back, as in k_scan. A block
-// has one type, so a thread takes part in one list at most; its bitmap words
-// and its object bitmap load together.
+// The lists of a step (dsr_steps.cuh).
 __global__ void __launch_bounds__(256) k_list(const __grid_constant__ dsr_dev_heap H, int ta, int tb, unsigned mult_a,
                                               unsigned mult_b) {
-    __shared__ unsigned warp_n[2][8];
-    __shared__ unsigned run_base[2];
-    const dsr_u64 M = H.M;
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned fsh = H.free_bm.shift, flo = (1u << fsh) - 1;
-    unsigned objs_a = 0, objs_b = 0;
-    for (dsr_u64 base = (dsr_u64)blockIdx.x * 256; base < M; base += (dsr_u64)gridDim.x * 256) {
-        const dsr_u64 b = base + threadIdx.x;
-        bool in_a = false, in_b = false;
-        dsr_u64 obj = 0;
-        if (b < M) {
-            const dsr_u64 wa = H.alloc_bm[ta].lvl[0][b >> fsh];
-            const dsr_u64 wb = tb >= 0 ? H.alloc_bm[tb].lvl[0][b >> fsh] : 0ull;
-            obj = H.obj[b];
-            in_a = (wa >> (b & flo)) & 1ull;
-            in_b = (wb >> (b & flo)) & 1ull;
-        }
-        const unsigned ba = __ballot_sync(0xFFFFFFFFu, in_a), bb = __ballot_sync(0xFFFFFFFFu, in_b);
-        if (lane == 0) warp_n[0][warp] = __popc(ba), warp_n[1][warp] = __popc(bb);
-        __syncthreads();
-        if (threadIdx.x < 2) {
-            unsigned total = 0;
-            for (int w = 0; w < 8; ++w) {
-                const unsigned n = warp_n[threadIdx.x][w];
-                warp_n[threadIdx.x][w] = total;
-                total += n;
-            }
-            run_base[threadIdx.x] = total ? atomicAdd(H.R_count + (threadIdx.x ? DSR_LIST_BACK : 0), total) : 0;
-        }
-        __syncthreads();
-        if (in_a || in_b) {
-            const int l = in_a ? 0 : 1;
-            const dsr_u64 live = H.valid[in_a ? ta : tb] & ~obj;
-            const dsr_u64 k = run_base[l] + warp_n[l][warp] + __popc((in_a ? ba : bb) & ((1u << lane) - 1));
-            const dsr_u64 at = in_a ? k : M - 1 - k;
-            H.R_bid[at] = (uint32_t)b;
-            H.R_mask[at] = live;
-            (in_a ? objs_a : objs_b) += __popcll(live);
-        }
-        __syncthreads();
-    }
-    const unsigned objs = __reduce_add_sync(0xFFFFFFFFu, objs_a * mult_a + objs_b * mult_b);
-    if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, objs);
+    __shared__ dsr_list_smem<256> sm;
+    dsr_list<256>(H, ta, tb, mult_a, mult_b, dsr_begin_step(H.R_count), sm);
+}
+
+static void cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, cudaStream_t s) {
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3(DSR_CLUSTER);
+    cfg->blockDim = dim3(DSR_CLUSTER_THREADS);
+    cfg->stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = DSR_CLUSTER;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+}
+
+bool dsr__cluster_fits(const void* kernel) {
+    int n = 0;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config(&cfg, &attr, nullptr);
+    const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+    cudaGetLastError();
+    return ok;
+}
+
+int dsr__launch_cluster(const void* kernel, void** args, cudaStream_t s) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config(&cfg, &attr, s);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, args);
+    if (e == cudaSuccess) return DSR_OK;
+    dsr__set_cuda_error(e, "cluster launch");
+    return DSR_E_CUDA;
 }
 
 // Statistics: out[0] free blocks; out[1 + 3T + {0,1,2}] allocated blocks,

@@ -26,8 +26,8 @@
 // block per thread, with one atomic each and no search. Only when they are
 // full are whole blocks claimed (dsr_claim_full). A remainder goes to another
 // CTA's partly filled block, if two searches find one; else a block is opened
-// for it if the CTA has at least DSR_OPEN_SHARE blocks already (at most one in
-// that many is then partly filled for this reason), or it goes through dsr_new. Work that
+// for it if it fills half of it or if the CTA has at least DSR_OPEN_SHARE blocks
+// already (so that few are partly filled), or it goes through dsr_new. Work that
 // few objects have (a dead agent's replacement) can be deferred in the same
 // way without a creation: full warps then do it.
 //
@@ -50,8 +50,17 @@
 #include "dsr_bulk.cuh"
 #include "dsr_group.cuh"
 
-constexpr int DSR_LIST_BACK = 2;         // R_count[2] counts the entries at the back of the list
-constexpr int DSR_GROUP_LIST_BACK = 32;  // the same for a group's list
+// Words from R_count that the lists use. Their lengths live in two sets of
+// (front, back) words, which steps use in turn: the scan of a step adds to one
+// set, whose words are zero then, and the step's last do-all clears the other
+// for the next. DSR_TURN counts the steps; the scan copies it to DSR_TURN_NOW,
+// where the step's do-alls read which set is theirs, and the last do-all
+// advances it. No kernel writes a word that another of its CTAs reads, so a
+// step ends without a rendezvous of its last kernel's CTAs (a fence and an
+// atomic that each waited for, 2 to 3 us a step). R_count[0], the length of
+// dsr_doall_scan's list, stays zero.
+constexpr uint32_t DSR_SET = 8;  // front of set 0; + 1: back; + 2, + 3: set 1
+constexpr uint32_t DSR_TURN = 12, DSR_TURN_NOW = 13;
 #ifndef DSR_OPEN_SHARE
 #define DSR_OPEN_SHARE 16
 #endif
@@ -96,14 +105,42 @@ struct dsr_later {
     }
 };
 
+// The length of this step's front or back list. Called by whole warps: five
+// lanes read the words, one request a warp (read by all lanes word by word,
+// the sector they are in had 36,000 requests from a full grid to answer: 20 us
+// a kernel; read by one warp for the CTA, with a barrier, the car do-all of
+// 6.7 M cars took 82 us instead of 63: its warps then march in step).
+__device__ __forceinline__ uint32_t dsr_list_length(const uint32_t* R_count, int back) {
+    const unsigned lane = dsr_lane();
+    uint32_t v = 0;
+    if (lane < 5) v = *(const volatile uint32_t*)(R_count + (lane < 4 ? DSR_SET + lane : DSR_TURN_NOW));
+    const unsigned turn = __shfl_sync(0xFFFFFFFFu, v, 4);
+    return __shfl_sync(0xFFFFFFFFu, v, 2 * (turn & 1) + (unsigned)back);
+}
+// The scan's part: the first word of the step's set, read by the threads that
+// add to it, and the copy of the turn.
+__device__ __forceinline__ uint32_t dsr_begin_step(uint32_t* R_count) {
+    uint32_t turn = 0;
+    if (threadIdx.x < 2) turn = *(volatile uint32_t*)(R_count + DSR_TURN);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile uint32_t*)(R_count + DSR_TURN_NOW) = turn;
+    return DSR_SET + 2 * (turn & 1);
+}
+// By one thread of a step's last do-all, at any time.
+__device__ __forceinline__ void dsr_end_step(uint32_t* R_count) {
+    volatile uint32_t* w = R_count;
+    const uint32_t next = w[DSR_TURN_NOW] + 1;
+    w[DSR_SET + 2 * (next & 1)] = 0;
+    w[DSR_SET + 2 * (next & 1) + 1] = 0;
+    w[DSR_TURN] = next;
+}
+
 // The list of a heap, or of all heaps of a group.
 struct dsr_heap_space {
     static constexpr bool kGroup = false;
     const dsr_dev_heap& H;
+    const uint32_t* len = nullptr;  // the lists' lengths, in shared memory (small heaps), or by the turn
     __device__ __forceinline__ const dsr_dev_heap& heap(uint32_t) const { return H; }
-    __device__ __forceinline__ uint32_t count(int back) const {
-        return *(volatile uint32_t*)(H.R_count + (back ? DSR_LIST_BACK : 0));
-    }
+    __device__ __forceinline__ uint32_t count(int back) const { return len ? len[back] : dsr_list_length(H.R_count, back); }
     __device__ __forceinline__ uint32_t at(uint32_t e, int back) const { return back ? (uint32_t)H.M - 1 - e : e; }
     __device__ __forceinline__ uint32_t heap_of(uint32_t) const { return 0; }
     __device__ __forceinline__ uint32_t bid(uint32_t at) const { return H.R_bid[at]; }
@@ -114,9 +151,7 @@ struct dsr_group_space {
     static constexpr bool kGroup = true;
     const dsr_group_dev& G;
     __device__ __forceinline__ const dsr_dev_heap& heap(uint32_t h) const { return G.heaps[h]; }
-    __device__ __forceinline__ uint32_t count(int back) const {
-        return *(volatile uint32_t*)(G.R_count + (back ? DSR_GROUP_LIST_BACK : 0));
-    }
+    __device__ __forceinline__ uint32_t count(int back) const { return dsr_list_length(G.R_count, back); }
     __device__ __forceinline__ uint32_t at(uint32_t e, int back) const { return back ? (uint32_t)G.R_cap - 1 - e : e; }
     __device__ __forceinline__ uint32_t heap_of(uint32_t at) const { return G.R_heap[at]; }
     __device__ __forceinline__ uint32_t bid(uint32_t at) const { return G.R_bid[at]; }
@@ -229,7 +264,7 @@ __device__ __forceinline__ void dsr_create_pending(const Space& S, const typenam
                 left -= n;
             }
             if (left != rem) dsr_count(H.ctr, DSR_CTR_ALLOCS, rem - left);
-            if (left && own_blocks >= DSR_OPEN_SHARE) {
+            if (left && (own_blocks >= DSR_OPEN_SHARE || 2 * left >= cap)) {
                 const dsr_grab g = dsr_init_block(H, T, (int)left, hint ^ 0x5bd1e995u);
                 if (!g.status) {
                     sm.open = g.bid << 6;  // its lowest slots
@@ -406,31 +441,111 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
     }
 }
 
-// End of a step's last do-all: true in every thread of the last CTA.
-__device__ __forceinline__ bool dsr_last_cta(uint32_t* done) {
-    __shared__ bool last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(done, 1u) == gridDim.x - 1;
-        if (last) *(volatile uint32_t*)done = 0;
-        __threadfence();
+// The lists of a step: type A's allocated blocks at the front (ta is -1: none),
+// type B's (tb is -1: none) at the back, with a snapshot of their occupied
+// slots; mult: visits counted per listed object. One thread per block id and
+// round of the CTAs cta, cta + ctas ..: a CTA forms the prefix sums of its
+// warps' counts and reserves its runs with one atomic each (`set`: the first
+// word of the lengths, needed in threads 0 and 1). A block has one
+// type, so a thread takes part in one list at most; its bitmap words and its
+// object bitmap load together.
+template <int MAXT>
+struct dsr_list_smem {
+    unsigned n[2][MAXT / 32];
+    unsigned base[2];
+};
+template <int MAXT>
+__device__ __forceinline__ void dsr_list(const dsr_dev_heap& H, int ta, int tb, unsigned mult_a, unsigned mult_b,
+                                         uint32_t set, dsr_list_smem<MAXT>& sm) {
+    const dsr_u64 M = H.M;
+    constexpr unsigned warps = MAXT / 32;  // the CTA has MAXT threads
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned fsh = H.free_bm.shift, flo = (1u << fsh) - 1;
+    dsr_u64 objs = 0;
+    for (dsr_u64 base = (dsr_u64)blockIdx.x * blockDim.x; base < M; base += (dsr_u64)gridDim.x * blockDim.x) {
+        const dsr_u64 b = base + threadIdx.x;
+        bool in_a = false, in_b = false;
+        dsr_u64 obj = 0;
+        if (b < M) {
+            const dsr_u64 wa = ta >= 0 ? H.alloc_bm[ta].lvl[0][b >> fsh] : 0ull;
+            const dsr_u64 wb = tb >= 0 ? H.alloc_bm[tb].lvl[0][b >> fsh] : 0ull;
+            obj = H.obj[b];
+            in_a = (wa >> (b & flo)) & 1ull;
+            in_b = (wb >> (b & flo)) & 1ull;
+        }
+        const unsigned ba = __ballot_sync(0xFFFFFFFFu, in_a), bb = __ballot_sync(0xFFFFFFFFu, in_b);
+        if (lane == 0) sm.n[0][warp] = __popc(ba), sm.n[1][warp] = __popc(bb);
+        __syncthreads();
+        if (threadIdx.x < 2) {
+            unsigned total = 0;
+#pragma unroll
+            for (unsigned w = 0; w < warps; ++w) {
+                const unsigned n = sm.n[threadIdx.x][w];
+                sm.n[threadIdx.x][w] = total;
+                total += n;
+            }
+            sm.base[threadIdx.x] = total ? atomicAdd(H.R_count + set + threadIdx.x, total) : 0;
+        }
+        __syncthreads();
+        if (in_a || in_b) {
+            const int l = in_a ? 0 : 1;
+            const dsr_u64 live = H.valid[in_a ? ta : tb] & ~obj;
+            const dsr_u64 k = sm.base[l] + sm.n[l][warp] + __popc((in_a ? ba : bb) & ((1u << lane) - 1));
+            const dsr_u64 at = in_a ? k : M - 1 - k;
+            H.R_bid[at] = (uint32_t)b;
+            H.R_mask[at] = live;
+            objs += (dsr_u64)__popcll(live) * (in_a ? mult_a : mult_b);
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    return last;
+    for (int o = 16; o; o >>= 1) objs += __shfl_xor_sync(0xFFFFFFFFu, objs, o);
+    if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, objs);
 }
 
-__device__ __forceinline__ void dsr_empty_lists(const dsr_dev_heap& H) {
-    *(volatile uint32_t*)H.R_count = 0;
-    *(volatile uint32_t*)(H.R_count + DSR_LIST_BACK) = 0;
+// ---- small heaps: whole steps in one launch ----------------------------------
+// On a small heap a do-all is a few microseconds of launch and dependent
+// accesses, on a handful of SMs: one thread-block cluster runs the do-alls of
+// many steps one after the other, with the cluster's hardware barrier between
+// them instead of a kernel boundary.
+constexpr int DSR_CLUSTER = 16;           // CTAs (a non-portable size)
+constexpr int DSR_CLUSTER_THREADS = 512;
+constexpr int DSR_CLUSTER_STEPS = 256;    // per launch
+
+// The lengths in set `set` (its front's word), after a barrier.
+__device__ __forceinline__ void dsr_set_lengths(const uint32_t* R_count, uint32_t set, uint32_t* len) {
+    if (threadIdx.x < 2) len[threadIdx.x] = *(const volatile uint32_t*)(R_count + set + threadIdx.x);
+    __syncthreads();
+}
+__device__ __forceinline__ void dsr_clear_set(uint32_t* R_count, uint32_t set) {
+    volatile uint32_t* w = R_count;
+    w[set] = 0;
+    w[set + 1] = 0;
+}
+
+// All writes of the cluster's threads before it are visible to all of them after it.
+__device__ __forceinline__ void dsr_cluster_barrier() {
+    __syncthreads();
+    asm volatile(
+        "barrier.cluster.arrive.release.aligned;\n\t"
+        "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Whether `kernel` can run as one cluster of DSR_CLUSTER CTAs on this device.
+bool dsr__cluster_fits(const void* kernel);
+// Queue it with the given arguments.
+int dsr__launch_cluster(const void* kernel, void** args, cudaStream_t s);
+// Small heaps of the default tuning (a caller that sets threads or CTAs gets
+// the kernels it set them for).
+inline bool dsr__small_heap(const dsr_heap* h, dsr_u64 blocks) {
+    return h->dev.M <= blocks && h->tune.threads == 256 && h->tune.ctas_per_sm <= 0;
 }
 
 // One do-all, or two that do not depend on each other. Five CTAs of 256 threads
 // per SM (48 registers; sugarscape 1914 -> 1854, life 1500 x 1000 1632 -> 1565 us
 // a pass against six, whose 40 registers spill); the group form, whose methods
 // wait longer for their heap's view, has six (7440 against 7524). END: the last of the
-// step (its last CTA empties the lists). F: a type whose finish(H, args) that
-// CTA's first thread runs (finish_group: all its threads).
+// step. F: a type whose finish(H, args) one thread then runs (finish_group:
+// the threads of one CTA), at any time during the do-all.
 template <class M1, class M2, bool END, class F, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 5 : 1)
     dsr_step_kernel(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ dsr_phase p1,
@@ -447,8 +562,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 5 : 1)
         dsr_run_list<M2, dsr_heap_space, MAXT>(S, p2, a, H.span_sh[p2.type] - 5, true, nullptr);
     }
     if constexpr (END) {
-        if (dsr_last_cta(H.R_done) && threadIdx.x == 0) {
-            dsr_empty_lists(H);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            dsr_end_step(H.R_count);
             if constexpr (!std::is_same<F, dsr_no_method>::value) F::finish(H, a);
         }
     }
@@ -472,11 +587,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 6 : 1)
         dsr_run_list<M2, dsr_group_space, MAXT>(S, p2, a, hsh2, true, nullptr);
     }
     if constexpr (END) {
-        if (dsr_last_cta(G.R_done)) {
-            if (threadIdx.x == 0) {
-                *(volatile uint32_t*)G.R_count = 0;
-                *(volatile uint32_t*)(G.R_count + DSR_GROUP_LIST_BACK) = 0;
-            }
+        if (blockIdx.x == 0) {
+            if (threadIdx.x == 0) dsr_end_step(G.R_count);
             if constexpr (!std::is_same<F, dsr_no_method>::value) F::finish_group(G, a);
         }
     }

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256, 5)
     const dsr_u64 n = ((dsr_u64)a.p.R * a.p.L + 255) / 256 * 16;
     for (dsr_u64 i = (dsr_u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (dsr_u64)gridDim.x * blockDim.x)
         w[i] = make_uint4(0, 0, 0, 0);
-    if (dsr_last_cta(H.R_done) && threadIdx.x == 0) dsr_empty_lists(H);
+    if (blockIdx.x == 0 && threadIdx.x == 0) dsr_end_step(H.R_count);
 }
 
 // One thread per cell: a Car where v0 >= 0.

@@ -385,8 +385,8 @@ struct DSharkMove : WatorMove<A> {
         shark_born(H, I, (uint32_t)c, r);
     }
 };
-// The last CTA of a step's last do-all advances the step counter (of every
-// instance in the batch).
+// A step's last do-all, which does not read it, advances the step counter (of
+// every instance in the batch).
 struct NextStep {
     static __device__ void finish(const dsr_dev_heap&, const WatorInst& a) { *a.step += 1; }
     static __device__ void finish_group(const dsr_group_dev& G, const BatchArgs& a) {
@@ -401,6 +401,38 @@ struct NextStep {
 // does (a fish moves into cells that were empty at the start of the step), so
 // the two share a launch.
 constexpr dsr_phase kFish{FISH, 0}, kSharks{SHARK, 1};
+
+// Steps of a small torus in one launch of one cluster (dsr_steps.cuh).
+__global__ void __launch_bounds__(DSR_CLUSTER_THREADS, 1)
+    k_wator_steps(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ WatorInst I, int n) {
+    constexpr int T = DSR_CLUSTER_THREADS;
+    typedef WatorInst A;
+    __shared__ dsr_later_smem<T> later;
+    __shared__ dsr_list_smem<T> list;
+    __shared__ uint32_t len[2];
+    const dsr_heap_space S{H, len};
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    const dsr_phase fish{FISH, 0}, sharks{SHARK, 1};
+    const unsigned hf = H.span_sh[FISH] - 5, hs = H.span_sh[SHARK] - 5;
+    for (int t = 0; t < n; ++t) {
+        const uint32_t set = DSR_SET + 2 * (t & 1), other = DSR_SET + 2 * (~t & 1);
+        dsr_list<T>(H, FISH, SHARK, 2, 1, set, list);
+        dsr_cluster_barrier();
+        dsr_set_lengths(H.R_count, set, len);
+        if (first) dsr_clear_set(H.R_count, other);  // the step before's, no longer read
+        dsr_run_list<DFishChoose<A>, dsr_heap_space, T>(S, fish, I, hf, false, nullptr);
+        dsr_cluster_barrier();
+        dsr_run_list<DFishMove<A>, dsr_heap_space, T>(S, fish, I, hf, false, &later);
+        dsr_run_list<DSharkStarve<A>, dsr_heap_space, T>(S, sharks, I, hs, true, nullptr);
+        dsr_cluster_barrier();
+        dsr_run_list<DSharkChoose<A>, dsr_heap_space, T>(S, sharks, I, hs, false, nullptr);
+        dsr_cluster_barrier();
+        dsr_run_list<DSharkMove<A>, dsr_heap_space, T>(S, sharks, I, hs, false, &later);
+        if (first) *I.step += 1;  // next read after the barrier
+        dsr_cluster_barrier();
+        if (first && t == n - 1) dsr_clear_set(H.R_count, set);
+    }
+}
 
 // Creates the agent of cell c (or none), and clears the cell's claim.
 template <class HP>
@@ -720,6 +752,11 @@ static bool replay_step(dsr_wator* w, cudaStream_t s, const cudaEvent_t* e, int 
     return true;
 }
 
+// Heaps up to this many blocks (a torus of about 130 x 130 with the default
+// heap) run their steps in one cluster: 27 against 31 us a step at 428 blocks,
+// 33 and 34 at 640, 34 and 36 at 940, 40 and 37 at 1324.
+constexpr dsr_u64 kSmallBlocks = 1024;
+
 extern "C" int dsr_wator_step(dsr_wator* w, int n_steps, void* stream) {
     if (!w || n_steps < 0) return DSR_E_INVALID;
     cudaStream_t s = dsr__stream(stream);
@@ -729,6 +766,18 @@ extern "C" int dsr_wator_step(dsr_wator* w, int n_steps, void* stream) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const bool use_graph = !w->graphs_off && cudaStreamIsCapturing(s, &cs) == cudaSuccess &&
                            cs == cudaStreamCaptureStatusNone;
+    // Small heaps: up to DSR_CLUSTER_STEPS steps a launch (kSmallBlocks).
+    static const bool fits = dsr__cluster_fits((const void*)k_wator_steps);
+    if (w->ev.empty() && fits && dsr__small_heap(w->heap, kSmallBlocks)) {
+        for (int i = 0; i < n_steps;) {
+            int n = n_steps - i < DSR_CLUSTER_STEPS ? n_steps - i : DSR_CLUSTER_STEPS;
+            void* args[] = {&w->heap->dev, &w->inst, &n};
+            const int rc = dsr__launch_cluster((const void*)k_wator_steps, args, s);
+            if (rc) return rc;
+            i += n;
+        }
+        return DSR_OK;
+    }
     for (int i = 0; i < n_steps; ++i) {
         cudaEvent_t* e = nullptr;
         if ((size_t)(w->ev_steps + 1) * kPhaseEvents <= w->ev.size())
