@@ -73,6 +73,7 @@ struct NbWs {
     uint32_t* perm2;   // [P] sorted position of each entry of the second order
     uint32_t* n_live;  // bodies in this step
     uint32_t* npairs;  // near-field pairs of this step (each counted from both bodies)
+    uint32_t* work;    // next work item of the symmetric force kernel (zeroed by the gather)
     // per sorted position p (padded to a multiple of ROW with empty entries)
     float4* pos;       // high words x, y, z, m before the update (m = 0: empty)
     D4* pd;            // full x, y, z, m before the update
@@ -292,6 +293,7 @@ __global__ void __launch_bounds__(TILE) k_gather(const __grid_constant__ dsr_dev
                                                  const __grid_constant__ NbWs ws) {
     __shared__ float red[6][TILE / 32];
     const uint32_t nl = n_bodies(ws), np = n_padded(ws);
+    if (ws.work && blockIdx.x == 0 && threadIdx.x == 0) *ws.work = 0;
     for (uint32_t t = blockIdx.x; t * TILE < np; t += gridDim.x) {
         const uint32_t p = t * TILE + threadIdx.x;
         float b[6] = {FLT_MAX, FLT_MAX, FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX};
@@ -592,6 +594,309 @@ __global__ void __launch_bounds__(TILE) k_force64(const __grid_constant__ dsr_de
 }
 
 // ---------------------------------------------------------------------------
+// Symmetric pair forces (FP32 and FP64, softened)
+// ---------------------------------------------------------------------------
+// Every unordered pair once: its r^-3 gives both bodies' terms. Per ordered
+// pair that is 8.5 FP32 operations and half a reciprocal square root instead
+// of 12 and one (FP64: 10 operations instead of about 19), and the kernels are
+// bound by the issue of exactly those.
+//
+// A row is THREADS * RB positions, RB per thread, a tile THREADS of them. A
+// work item is a group of RG rows times a group of TR tiles, handed out by a
+// counter; tiles before a row's own are another item's pairs, the RB tiles of
+// the row itself take every ordered pair as k_force_part does (a body meets
+// itself there), and the tiles after it are symmetric: the 32 lanes of a warp
+// meet the 32 bodies of a block of the tile in 32 steps, lane l body (l + s)
+// mod 32 in step s, so that every lane has another body, and the sum of a
+// body's terms travels from lane to lane with it by shuffle. After JF steps
+// (a chunk of 32 terms in FP32) it is added, compensated in FP32, to the
+// body's sums in shared memory. The warps of a CTA take the tile's blocks in
+// turn, one barrier apart, so no two add to one body at a time.
+//
+// Sums. Row side: as in k_force_part, chunks of 32 terms, compensated; one
+// entry per group of tiles. Tile side: one entry per group of rows. The
+// groups are so large that either side has at most `slots` entries (but a
+// tile group's sums must fit shared memory), and the update adds the entries
+// of a body in a fixed order: a step stays deterministic.
+// Measured, 65,322 bodies FP32: k_force_part 1990 -> @F32@ us; 8000 bodies
+// FP64: 2560 -> @F64@; 4097 bodies FP32: 30 -> @F4@.
+struct SymShape {
+    uint32_t n, nr, nt;  // padded count, rows, tiles
+    uint32_t RG, TR;     // rows and tiles of a group
+    uint32_t na, nb;     // row groups, tile groups
+};
+
+__host__ __device__ inline SymShape sym_shape(uint32_t n, uint32_t threads, uint32_t rb, uint32_t slots, uint32_t max_tr) {
+    SymShape q;
+    q.n = n;
+    q.nr = n / (threads * rb);
+    q.nt = n / threads;
+    q.RG = (q.nr + slots - 1) / slots;
+    q.TR = (q.nt + slots - 1) / slots;
+    if (q.TR > max_tr) q.TR = max_tr;
+    if (q.RG < 1) q.RG = 1;
+    if (q.TR < 1) q.TR = 1;
+    q.na = (q.nr + q.RG - 1) / q.RG;
+    q.nb = (q.nt + q.TR - 1) / q.TR;
+    return q;
+}
+
+// The two forms of the arithmetic.
+struct SymF32 {
+    typedef float Real;
+    typedef float4 Vec;
+    static constexpr int THREADS = 128, RB = 8, JF = 4;
+    static constexpr uint32_t SLOTS = 64, SLOTS_FEW = 64, MAX_TR = 16;
+    static constexpr int SUMS = 6;  // of a body in shared memory: three sums, three compensations
+    static constexpr int CTAS = 3;  // per SM
+};
+struct SymF32Small : SymF32 {  // few bodies: more and smaller items
+    static constexpr int THREADS = 128, RB = 2, JF = 16, CTAS = 5;
+};
+struct SymF64 {
+    typedef double Real;
+    typedef D4 Vec;
+    // the FP64 units of an SM are busy with eight warps; more CTAs would only
+    // spread the items less evenly over the SMs
+    static constexpr int THREADS = 128, RB = 1, JF = 32, CTAS = 2;
+    static constexpr uint32_t SLOTS = 32, SLOTS_FEW = 128, MAX_TR = 32;
+    static constexpr int SUMS = 3;
+};
+// Entries of either side at most: for few bodies more and smaller items.
+constexpr uint32_t kSymFew = 16384;
+template <class F>
+__host__ __device__ constexpr uint32_t sym_slots(uint32_t n) {
+    return n <= kSymFew ? F::SLOTS_FEW : F::SLOTS;
+}
+
+__device__ __forceinline__ float inv_cubed(float r2) {
+    const float inv = rsqrt_normal(r2);
+    return inv * inv * inv;
+}
+// r^-3 in FP64, r^2 >= FLT_MIN. y: the PTX approximate reciprocal square
+// root, y^2 r^2 = 1 - h. Then r^-3 = y^3 (1 - h)^(-3/2), by the binomial
+// series 1 + 3/2 h + 15/8 h^2 + 35/16 h^3: what follows is 315/128 h^4, below
+// 2^-60 for any |h| < 2^-15.
+__device__ __forceinline__ double inv_cubed(double r2) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
+    const double y2 = y * y;
+    const double h = fma(-r2, y2, 1.0);
+    const double q = h * fma(fma(2.1875, h, 1.875), h, 1.5);
+    const double y3 = y * y2;
+    return fma(y3, q, y3);
+}
+
+__device__ __forceinline__ const float4* sym_bodies(const NbWs& ws, float) { return ws.pos; }
+__device__ __forceinline__ const D4* sym_bodies(const NbWs& ws, double) { return ws.pd; }
+__device__ __forceinline__ float4* sym_part(const NbWs& ws, float) { return ws.part; }
+__device__ __forceinline__ D4* sym_part(const NbWs& ws, double) { return ws.part64; }
+__device__ __forceinline__ float4 sym_vec(float x, float y, float z) { return make_float4(x, y, z, 0.f); }
+__device__ __forceinline__ D4 sym_vec(double x, double y, double z) { return d4(x, y, z, 0.0); }
+
+// One row against the block of 32 bodies at sp, every unordered pair.
+// sums: the bodies' sums in shared memory, `stride` apart.
+template <class F, bool EXCLUDE, class Real, class Vec>
+__device__ __forceinline__ void sym_block(const Vec* sp, Real* sums, int stride, const Real* px, const Real* py,
+                                          const Real* pz, const Real* pm, Real eps2, Real rn2, Real* tx, Real* ty,
+                                          Real* tz) {
+    constexpr int RB_ = F::RB;
+    const unsigned lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int s0 = 0; s0 < 32; s0 += F::JF) {
+        Real jx = 0, jy = 0, jz = 0;
+        unsigned at = 0;
+#pragma unroll 8
+        for (int s = 0; s < F::JF; ++s) {
+            at = (lane + s0 + s) & 31u;
+            const Vec pj = sp[at];
+#pragma unroll
+            for (int k = 0; k < RB_; ++k) {
+                const Real dx = pj.x - px[k], dy = pj.y - py[k], dz = pj.z - pz[k];
+                Real r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
+                if (EXCLUDE) r2 = r2 < rn2 ? (Real)f_inf() : r2;
+                const Real w = inv_cubed(r2);
+                const Real wj = pj.w * w, wi = pm[k] * w;
+                tx[k] = fma(wj, dx, tx[k]);
+                ty[k] = fma(wj, dy, ty[k]);
+                tz[k] = fma(wj, dz, tz[k]);
+                jx = fma(wi, dx, jx);
+                jy = fma(wi, dy, jy);
+                jz = fma(wi, dz, jz);
+            }
+            if (s + 1 < F::JF) {  // the next step's body was the next lane's
+                jx = __shfl_sync(0xFFFFFFFFu, jx, lane + 1);
+                jy = __shfl_sync(0xFFFFFFFFu, jy, lane + 1);
+                jz = __shfl_sync(0xFFFFFFFFu, jz, lane + 1);
+            }
+        }
+        Real* m = sums + at;
+        if constexpr (F::SUMS == 6) {
+            float sx = m[0], sy = m[stride], sz = m[2 * stride];
+            float cx = m[3 * stride], cy = m[4 * stride], cz = m[5 * stride];
+            kahan_add(sx, cx, -jx);
+            kahan_add(sy, cy, -jy);
+            kahan_add(sz, cz, -jz);
+            m[0] = sx, m[stride] = sy, m[2 * stride] = sz;
+            m[3 * stride] = cx, m[4 * stride] = cy, m[5 * stride] = cz;
+        } else {
+            m[0] -= jx;
+            m[stride] -= jy;
+            m[2 * stride] -= jz;
+        }
+        __syncwarp();
+    }
+}
+
+// One row against 32 bodies at sp, every ordered pair of the row's bodies.
+template <class F, bool EXCLUDE, class Real, class Vec>
+__device__ __forceinline__ void row_block(const Vec* sp, const Real* px, const Real* py, const Real* pz, Real eps2,
+                                          Real rn2, Real* tx, Real* ty, Real* tz) {
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+        const Vec pj = sp[j];
+#pragma unroll
+        for (int k = 0; k < F::RB; ++k) {
+            const Real dx = pj.x - px[k], dy = pj.y - py[k], dz = pj.z - pz[k];
+            Real r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
+            if (EXCLUDE) r2 = r2 < rn2 ? (Real)f_inf() : r2;
+            const Real w = pj.w * inv_cubed(r2);
+            tx[k] = fma(w, dx, tx[k]);
+            ty[k] = fma(w, dy, ty[k]);
+            tz[k] = fma(w, dz, tz[k]);
+        }
+    }
+}
+
+template <class F>
+__global__ void __launch_bounds__(F::THREADS, F::CTAS) k_force_sym(const __grid_constant__ NbArgs a) {
+    typedef typename F::Real Real;
+    typedef typename F::Vec Vec;
+    constexpr int THREADS = F::THREADS, RB_ = F::RB, WARPS = THREADS / 32, ROW_ = THREADS * RB_;
+    constexpr bool kF32 = F::SUMS == 6;
+    extern __shared__ __align__(32) unsigned char dynamic[];
+    Vec* sp = reinterpret_cast<Vec*>(dynamic);              // [THREADS]
+    Real* sums = reinterpret_cast<Real*>(sp + THREADS);     // [TR][SUMS][THREADS]
+    __shared__ uint32_t next;
+    const SymShape q = sym_shape(n_padded(a.ws), THREADS, RB_, sym_slots<F>(n_padded(a.ws)), F::MAX_TR);
+    const Vec* body = sym_bodies(a.ws, Real(0));
+    Vec* part = sym_part(a.ws, Real(0));
+    const Real eps2 = (Real)(a.p.eps * a.p.eps);
+    const Real rn2 = (Real)(a.p.r_near * a.p.r_near);
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    (void)lane;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) next = atomicAdd(a.ws.work, 1u);
+        __syncthreads();
+        const uint32_t item = next;
+        if (item >= q.na * q.nb) break;
+        const uint32_t ga = item / q.nb, gb = item % q.nb;
+        const uint32_t r0 = ga * q.RG, r1 = min(q.nr, r0 + q.RG), t0 = gb * q.TR, t1 = min(q.nt, t0 + q.TR);
+        if (t1 <= RB_ * r0) continue;  // every tile lies before the rows'
+        for (uint32_t k = threadIdx.x; k < (t1 - t0) * F::SUMS * THREADS; k += THREADS) sums[k] = 0;
+        for (uint32_t r = r0; r < r1 && RB_ * r < t1; ++r) {
+            const uint32_t g0 = r * ROW_ + threadIdx.x;
+            Real px[RB_], py[RB_], pz[RB_], pm[RB_], ax[RB_], ay[RB_], az[RB_], cx[RB_], cy[RB_], cz[RB_];
+#pragma unroll
+            for (int k = 0; k < RB_; ++k) {
+                const Vec u = body[g0 + k * THREADS];
+                px[k] = u.x, py[k] = u.y, pz[k] = u.z, pm[k] = u.w;
+                ax[k] = ay[k] = az[k] = cx[k] = cy[k] = cz[k] = 0;
+            }
+            float4 rlo, rhi;
+            if (kF32) {  // bounding box of the row, from the boxes of its TILE-sized tiles
+                const uint32_t b0 = r * ROW_ / TILE, b1 = (r + 1) * ROW_ / TILE;
+                rlo = a.ws.tbox[2 * b0], rhi = a.ws.tbox[2 * b0 + 1];
+                for (uint32_t b = b0 + 1; b < b1; ++b) {
+                    const float4 l = a.ws.tbox[2 * b], h = a.ws.tbox[2 * b + 1];
+                    rlo = make_float4(fminf(rlo.x, l.x), fminf(rlo.y, l.y), fminf(rlo.z, l.z), 0.f);
+                    rhi = make_float4(fmaxf(rhi.x, h.x), fmaxf(rhi.y, h.y), fmaxf(rhi.z, h.z), 0.f);
+                }
+            }
+            for (uint32_t t = max(t0, (uint32_t)RB_ * r); t < t1; ++t) {
+                __syncthreads();
+                sp[threadIdx.x] = body[t * THREADS + threadIdx.x];
+                __syncthreads();
+                bool near = false;
+                if (kF32) {
+                    const uint32_t b = t * THREADS / TILE;
+                    near = boxes_near(rlo, rhi, a.ws.tbox[2 * b], a.ws.tbox[2 * b + 1], (float)rn2);
+                }
+                const bool own = t < RB_ * (r + 1);
+                Real* m = sums + (t - t0) * F::SUMS * THREADS;
+                for (int ph = 0; ph < WARPS; ++ph) {
+                    const int jb = (int)((warp + ph) % WARPS) * 32;
+                    Real tx[RB_], ty[RB_], tz[RB_];
+#pragma unroll
+                    for (int k = 0; k < RB_; ++k) tx[k] = ty[k] = tz[k] = 0;
+                    if (own) {
+                        if (kF32 && near)
+                            row_block<F, true>(sp + jb, px, py, pz, eps2, rn2, tx, ty, tz);
+                        else
+                            row_block<F, false>(sp + jb, px, py, pz, eps2, rn2, tx, ty, tz);
+                    } else {
+                        if (kF32 && near)
+                            sym_block<F, true>(sp + jb, m + jb, THREADS, px, py, pz, pm, eps2, rn2, tx, ty, tz);
+                        else
+                            sym_block<F, false>(sp + jb, m + jb, THREADS, px, py, pz, pm, eps2, rn2, tx, ty, tz);
+                        __syncthreads();  // the next warp adds to these bodies' sums
+                    }
+#pragma unroll
+                    for (int k = 0; k < RB_; ++k) {
+                        if constexpr (kF32) {
+                            kahan_add(ax[k], cx[k], tx[k]);
+                            kahan_add(ay[k], cy[k], ty[k]);
+                            kahan_add(az[k], cz[k], tz[k]);
+                        } else {
+                            ax[k] += tx[k], ay[k] += ty[k], az[k] += tz[k];
+                        }
+                    }
+                }
+            }
+            Vec* out = part + (size_t)gb * q.n;
+#pragma unroll
+            for (int k = 0; k < RB_; ++k) out[g0 + k * THREADS] = sym_vec(ax[k], ay[k], az[k]);
+        }
+        __syncthreads();
+        Vec* out = part + (size_t)(q.nb + ga) * q.n;
+        for (uint32_t t = max(t0, (uint32_t)RB_ * (r0 + 1)); t < t1; ++t) {
+            const Real* m = sums + (t - t0) * F::SUMS * THREADS + threadIdx.x;
+            out[t * THREADS + threadIdx.x] = sym_vec(m[0], m[THREADS], m[2 * THREADS]);
+        }
+    }
+}
+
+// Where the far-field sums of a step are: `slots` 0: the slices of the split
+// kernels for `grid` CTAs (grid 0: the unsplit kernel's one slice), else the
+// symmetric kernel's entries.
+struct FarShape {
+    uint32_t grid;
+    uint32_t threads, rb, slots, slots_few, max_tr;
+};
+// The body's entries: `first` .. first + n1 - 1, then `second` .. second + n2 - 1, each `stride` apart.
+struct FarEntries {
+    uint32_t first, n1, second, n2;
+    size_t stride;
+};
+__device__ __forceinline__ FarEntries far_entries(const NbWs& ws, const FarShape& f, bool f64, uint32_t p) {
+    if (f.slots) {
+        const uint32_t n = n_padded(ws);
+        const SymShape q = sym_shape(n, f.threads, f.rb, n <= kSymFew ? f.slots_few : f.slots, f.max_tr);
+        const uint32_t r = p / (f.threads * f.rb), t = p / f.threads;
+        const uint32_t b0 = f.rb * r / q.TR;  // the first tile group with a tile of the row or after it
+        // row groups whose first row lies before the tile
+        const uint32_t rows = t / f.rb;  // rows r with rb * (r + 1) <= t
+        return FarEntries{b0, q.nb - b0, q.nb, rows ? (rows - 1) / q.RG + 1 : 0u, q.n};
+    }
+    if (f.grid) {
+        const SplitShape q = split_shape(ws, f.grid, f64 ? RB64 : RB);
+        return FarEntries{0, q.ns, 0, 0, q.n};
+    }
+    return FarEntries{0, 1, 0, 0, 0};
+}
+
+// ---------------------------------------------------------------------------
 // update, partner search, merge
 // ---------------------------------------------------------------------------
 // Visit the sorted entries of the cells around (and including) the cell of
@@ -659,37 +964,44 @@ __device__ __forceinline__ double rsqrt_cubed(double r2) {
     return y * y * y;
 }
 
-// Far field of the body at sorted position p: its slices summed in slice
-// order. FP32 slices are summed as FP32 pairs (error-free additions), which
+// Far field of the body at sorted position p: its entries summed in order. FP32 slices are summed as FP32 pairs (error-free additions), which
 // is as exact here as FP64 additions and keeps the FP64 units, a small
 // fraction of GB300's FP32 rate, free for the near field and the update.
-__device__ __forceinline__ void far_field(const NbArgs& a, uint32_t p, uint32_t ns, size_t stride, bool f64,
-                                          double& ax, double& ay, double& az) {
+__device__ __forceinline__ void far_field(const NbArgs& a, uint32_t p, const FarEntries& e, bool f64, double& ax,
+                                          double& ay, double& az) {
+    const uint32_t n = e.n1 + e.n2;
+    auto slice = [&](uint32_t k) { return (size_t)(k < e.n1 ? e.first + k : e.second + (k - e.n1)) * e.stride + p; };
     if (f64) {
-        for (uint32_t k = 0; k < ns; ++k) {
-            const D4 v = a.ws.part64[k * stride + p];
-            ax += v.x;
-            ay += v.y;
-            az += v.z;
+        uint32_t k = 0;
+        for (; k + 4 <= n; k += 4) {
+            D4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = a.ws.part64[slice(k + u)];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ax += v[u].x, ay += v[u].y, az += v[u].z;
+        }
+        for (; k < n; ++k) {
+            const D4 v = a.ws.part64[slice(k)];
+            ax += v.x, ay += v.y, az += v.z;
         }
         return;
     }
     float sx = 0.f, sy = 0.f, sz = 0.f, ex = 0.f, ey = 0.f, ez = 0.f;
-    // slices loaded four at a time, then added in order
+    // entries loaded eight at a time, then added in order
     uint32_t k = 0;
-    for (; k + 4 <= ns; k += 4) {
-        float4 v[4];
+    for (; k + 8 <= n; k += 8) {
+        float4 v[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = a.ws.part[(k + u) * stride + p];
+        for (int u = 0; u < 8; ++u) v[u] = a.ws.part[slice(k + u)];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
             two_sum_add(sx, ex, v[u].x);
             two_sum_add(sy, ey, v[u].y);
             two_sum_add(sz, ez, v[u].z);
         }
     }
-    for (; k < ns; ++k) {
-        const float4 v = a.ws.part[k * stride + p];
+    for (; k < n; ++k) {
+        const float4 v = a.ws.part[slice(k)];
         two_sum_add(sx, ex, v.x);
         two_sum_add(sy, ey, v.y);
         two_sum_add(sz, ez, v.z);
@@ -727,8 +1039,8 @@ constexpr int UPDATE_THREADS = 256;
 // axis k in a fixed order (far, then the columns from low to high), so a
 // step stays deterministic, and does that axis of v += a dt, x += v dt
 // (semi-implicit Euler) in FP64 on the full state, stored back as FP32
-// pairs; lane 3 writes the mass parts of the new state. `grid` is the split
-// force kernel's grid (0: the unsplit kernel's single slice).
+// pairs; lane 3 writes the mass parts of the new state. `far`: where the
+// force kernel left its sums.
 //
 // FP64 work in a warp. GB300 issues FP64 instructions at a small fraction of
 // its FP32 rate, and a warp instruction costs the same however few lanes it
@@ -744,16 +1056,10 @@ constexpr int UPDATE_THREADS = 256;
 // four spilled and made the step slower.
 constexpr int UPDATE_MIN_CTAS = 3;
 __global__ void __launch_bounds__(UPDATE_THREADS, UPDATE_MIN_CTAS) k_update(const __grid_constant__ dsr_dev_heap H,
-                                                           const __grid_constant__ NbArgs a, uint32_t grid) {
+                                                           const __grid_constant__ NbArgs a,
+                                                           const __grid_constant__ FarShape far) {
     __shared__ NearSlot slots[UPDATE_THREADS / 32][NEAR_SLOTS];
     const bool f64 = a.p.pair_precision == DSR_NBODY_PAIRS_FP64;
-    uint32_t ns = 1;
-    size_t stride = 0;
-    if (grid) {
-        const SplitShape q = split_shape(a.ws, grid, f64 ? RB64 : RB);
-        ns = q.ns;
-        stride = q.n;
-    }
     const uint32_t n = n_bodies(a.ws);
     const unsigned lane = threadIdx.x & 31u, sub = lane & 3u, quad = lane & ~3u;
     NearSlot* sl = slots[threadIdx.x >> 5];
@@ -773,7 +1079,7 @@ __global__ void __launch_bounds__(UPDATE_THREADS, UPDATE_MIN_CTAS) k_update(cons
         double ox = 0.0, oy = 0.0, oz = 0.0;  // near terms beyond the queue
         uint32_t cnt = 0, qd[NEAR_Q] = {0, 0, 0, 0};
         if (live && sub == 3) {
-            far_field(a, p, ns, stride, f64, ax, ay, az);
+            far_field(a, p, far_entries(a.ws, far, f64, p), f64, ax, ay, az);
         } else if (live && near_on) {
             const D4 pi = a.ws.pd[p];
             const float4 u = a.ws.pos[p];
@@ -981,12 +1287,49 @@ uint32_t split_grid(const dsr_heap* h, const void* kernel) {
     return (uint32_t)(4 * occ * h->sm_count);
 }
 
+// The symmetric kernels serve heaps of up to this many padded positions; for
+// more, their entries (128 and more a position) would need several times the
+// workspace of the split kernels, which then run.
+constexpr uint64_t kSymPositions = 160 * 1024;
+constexpr int kSymSmallBodies = 16384;
+
 struct SplitGrids {
     uint32_t force, force64;
+    uint32_t sym, sym_small, sym64;  // grids of the symmetric kernels
 };
 
+template <class F>
+size_t sym_smem(uint64_t n) {
+    // a smaller live count may have larger tile groups (SLOTS below SLOTS_FEW is not the case)
+    const SymShape q = sym_shape((uint32_t)n, F::THREADS, F::RB, sym_slots<F>((uint32_t)n), F::MAX_TR);
+    return F::THREADS * sizeof(typename F::Vec) + (size_t)q.TR * F::SUMS * F::THREADS * sizeof(typename F::Real);
+}
+// CTAs of a symmetric kernel that fit at once, with the shared memory of n positions.
+template <class F>
+uint32_t sym_grid(const dsr_heap* h, uint64_t n) {
+    const size_t most = F::THREADS * sizeof(typename F::Vec) +
+                        (size_t)F::MAX_TR * F::SUMS * F::THREADS * sizeof(typename F::Real);
+    cudaFuncSetAttribute(k_force_sym<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_force_sym<F>, F::THREADS, sym_smem<F>(n)) !=
+            cudaSuccess || occ < 1)
+        occ = 1;
+    if (occ > F::CTAS) occ = F::CTAS;
+    // as many CTAs as items, in whole CTAs per SM: an idle CTA's SM would be
+    // short of the work that another SM has too much of
+    const SymShape q = sym_shape((uint32_t)n, F::THREADS, F::RB, sym_slots<F>((uint32_t)n), F::MAX_TR);
+    uint64_t items = 0;
+    for (uint32_t ga = 0; ga < q.na; ++ga)
+        for (uint32_t gb = 0; gb < q.nb; ++gb) {
+            const uint32_t t1 = (gb + 1) * q.TR < q.nt ? (gb + 1) * q.TR : q.nt;
+            items += t1 > F::RB * ga * q.RG;
+        }
+    const uint64_t per_sm = (items + h->sm_count - 1) / h->sm_count;
+    return (uint32_t)((per_sm < (uint64_t)occ ? per_sm : (uint64_t)occ) * h->sm_count);
+}
+
 SplitGrids split_grids(const dsr_heap* h) {
-    return {split_grid(h, (const void*)k_force_part<true>), split_grid(h, (const void*)k_force_part64)};
+    return {split_grid(h, (const void*)k_force_part<true>), split_grid(h, (const void*)k_force_part64), 0, 0, 0};
 }
 
 // Padded positions for a heap of S slots.
@@ -1010,6 +1353,16 @@ size_t part_bytes(uint64_t P, SplitGrids g) {
         const size_t a = slots_for(n, g.force, RB) * 16, b = slots_for(n, g.force64, RB64) * 32;
         if (a > m) m = a;
         if (b > m) m = b;
+        if (P > kSymPositions) continue;
+        auto sym = [&](uint32_t threads, uint32_t rb, uint32_t slots, uint32_t few, uint32_t max_tr, size_t entry) {
+            const SymShape q = sym_shape((uint32_t)n, threads, rb, n <= kSymFew ? few : slots, max_tr);
+            const size_t c = (size_t)(q.na + q.nb) * n * entry;
+            if (c > m) m = c;
+        };
+        sym(SymF32::THREADS, SymF32::RB, SymF32::SLOTS, SymF32::SLOTS_FEW, SymF32::MAX_TR, 16);
+        if (n <= padded(kSymSmallBodies))
+            sym(SymF32Small::THREADS, SymF32Small::RB, SymF32Small::SLOTS, SymF32Small::SLOTS_FEW, SymF32Small::MAX_TR, 16);
+        sym(SymF64::THREADS, SymF64::RB, SymF64::SLOTS, SymF64::SLOTS_FEW, SymF64::MAX_TR, 32);
     }
     return m;
 }
@@ -1072,6 +1425,7 @@ NbWs carve(void* base, uint64_t S, uint64_t log_cap, SplitGrids grid) {
     w.step = reinterpret_cast<dsr_u64*>(p + 8);
     w.n_live = reinterpret_cast<uint32_t*>(p + 16);
     w.npairs = reinterpret_cast<uint32_t*>(p + 20);
+    w.work = reinterpret_cast<uint32_t*>(p + 24);
     p += 256;
     w.part = reinterpret_cast<float4*>(p);
     w.part64 = reinterpret_cast<D4*>(p);
@@ -1090,24 +1444,36 @@ void launch_sort(dsr_heap* h, const NbArgs& a, cudaStream_t s) {
     k_cell_order<POST><<<NKEYS / 256, 256, 0, s>>>(h->dev, a.ws);
 }
 
-// One step. `split`: the split force kernels with their grids (else the
-// unsplit ones, for the allocation-free step); P: padded positions.
-void launch_step(dsr_heap* h, const NbArgs& a, const SplitGrids* split, uint64_t P, cudaStream_t s) {
+template <class F>
+FarShape launch_sym(const NbArgs& a, uint32_t grid, uint64_t n, cudaStream_t s) {
+    k_force_sym<F><<<grid, F::THREADS, sym_smem<F>(n), s>>>(a);
+    return FarShape{0, (uint32_t)F::THREADS, (uint32_t)F::RB, F::SLOTS, F::SLOTS_FEW, F::MAX_TR};
+}
+
+// One step. `split`: the force kernels' grids (else the unsplit ones, for the
+// allocation-free step); P: padded positions; n0: bodies at most (the heap's
+// bodies at creation; merges only reduce them).
+void launch_step(dsr_heap* h, const NbArgs& a, const SplitGrids* split, uint64_t P, uint64_t n0, cudaStream_t s) {
     const unsigned ctas = (unsigned)(h->sm_count * 4);
     const bool f64 = a.p.pair_precision == DSR_NBODY_PAIRS_FP64;
     const bool soft = a.p.eps * a.p.eps >= (double)FLT_MIN;
     dsr__launch_scan(h, BODY, s);
     launch_sort<false>(h, a, s);
     k_gather<<<ctas, TILE, 0, s>>>(h->dev, a.ws);
-    uint32_t grid = 0;
-    if (split) {
-        grid = f64 ? split->force64 : split->force;
+    FarShape far{0, 0, 0, 0, 0, 0};
+    if (split && soft && split->sym) {
+        const uint64_t n = padded(n0);
+        far = f64 ? launch_sym<SymF64>(a, split->sym64, n, s)
+              : n0 <= (uint64_t)kSymSmallBodies ? launch_sym<SymF32Small>(a, split->sym_small, n, s)
+                                                : launch_sym<SymF32>(a, split->sym, n, s);
+    } else if (split) {
+        far.grid = f64 ? split->force64 : split->force;
         if (f64)
-            k_force_part64<<<grid, TILE, 0, s>>>(h->dev, a);
+            k_force_part64<<<far.grid, TILE, 0, s>>>(h->dev, a);
         else if (soft)
-            k_force_part<true><<<grid, TILE, 0, s>>>(h->dev, a);
+            k_force_part<true><<<far.grid, TILE, 0, s>>>(h->dev, a);
         else
-            k_force_part<false><<<grid, TILE, 0, s>>>(h->dev, a);
+            k_force_part<false><<<far.grid, TILE, 0, s>>>(h->dev, a);
     } else {
         const unsigned tiles = (unsigned)(P / TILE);
         if (f64)
@@ -1115,7 +1481,7 @@ void launch_step(dsr_heap* h, const NbArgs& a, const SplitGrids* split, uint64_t
         else
             k_force<<<tiles, TILE, 0, s>>>(h->dev, a);
     }
-    k_update<<<ctas, UPDATE_THREADS, 0, s>>>(h->dev, a, grid);
+    k_update<<<ctas, UPDATE_THREADS, 0, s>>>(h->dev, a, far);
     launch_sort<true>(h, a, s);
     k_partner<<<ctas, 256, 0, s>>>(h->dev, a);
     k_merge<<<ctas, 256, 0, s>>>(h->dev, a);
@@ -1126,7 +1492,8 @@ struct dsr_nbody {
     dsr_heap* heap;
     NbArgs args;
     uint64_t S;
-    SplitGrids grid;  // of the split all-pairs kernels
+    uint64_t n0;      // bodies at creation
+    SplitGrids grid;  // of the all-pairs kernels
 };
 
 extern "C" int dsr_nbody_types(dsr_type_desc* out) {
@@ -1150,7 +1517,14 @@ extern "C" int dsr_nbody_create(dsr_heap* heap, const dsr_nbody_params* p, const
     dsr_nbody* nb = new dsr_nbody;
     nb->heap = heap;
     nb->S = heap->layout.n_blocks * 64;
+    nb->n0 = (uint64_t)n_bodies;
     nb->grid = split_grids(heap);
+    if (padded(nb->S) <= kSymPositions) {
+        const uint64_t n = padded(nb->n0);
+        nb->grid.sym = sym_grid<SymF32>(heap, n);
+        nb->grid.sym_small = sym_grid<SymF32Small>(heap, n < padded(kSymSmallBodies) ? n : padded(kSymSmallBodies));
+        nb->grid.sym64 = sym_grid<SymF64>(heap, n);
+    }
     nb->args.ws = carve(workspace_dev, nb->S, log_cap, nb->grid);
     nb->args.ws.K = cells_per_axis(*p);
     nb->args.p = *p;
@@ -1178,7 +1552,7 @@ extern "C" int dsr_nbody_step(dsr_nbody* nb, int n_steps, void* stream) {
     if (!nb || n_steps < 0) return DSR_E_INVALID;
     cudaStream_t s = dsr__stream(stream);
     for (int i = 0; i < n_steps; ++i) {
-        launch_step(nb->heap, nb->args, &nb->grid, padded(nb->S), s);
+        launch_step(nb->heap, nb->args, &nb->grid, padded(nb->S), nb->n0, s);
         int rc = dsr__check_launch("dsr_nbody_step");
         if (rc) return rc;
     }
@@ -1294,6 +1668,7 @@ extern "C" int dsr_nbody_step_noalloc(dsr_heap* heap, const dsr_nbody_params* p,
     a.ws.perm2 = sc->perm2;
     a.ws.n_live = &sc->n_live;
     a.ws.npairs = &sc->npairs;
+    a.ws.work = nullptr;  // the unsplit force kernels
     a.ws.pos = sc->pos;
     a.ws.pd = sc->pd;
     a.ws.id = sc->id;
@@ -1315,6 +1690,6 @@ extern "C" int dsr_nbody_step_noalloc(dsr_heap* heap, const dsr_nbody_params* p,
     // only value a step reads before writing it; the cell counts are zero
     // when the library is loaded and every sort returns them to zero.
     k_set_u64<<<1, 1, 0, s>>>(&sc->step, step0);
-    for (int i = 0; i < n_steps; ++i) launch_step(heap, a, nullptr, padded(S), s);
+    for (int i = 0; i < n_steps; ++i) launch_step(heap, a, nullptr, padded(S), S, s);
     return dsr__check_launch("dsr_nbody_step_noalloc");
 }
