@@ -744,12 +744,23 @@ __global__ void dsr_doall_kernel_vec4(const __grid_constant__ dsr_dev_heap H, in
     const unsigned sh = dsr_span_shift(H, T) - 2;  // quads per listed block: 16 (or 8)
     const dsr_u64 total = (dsr_u64)(*(volatile uint32_t*)H.R_count) << sh;
     const dsr_u64 stride = (dsr_u64)gridDim.x * blockDim.x;
-    for (dsr_u64 g = (dsr_u64)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
-        const dsr_u64 i = g >> sh;
+    // the list entry of the next quad is loaded while this one's fields are:
+    // at 75% fill of 2^26 objects with two fields 210 -> 190 us
+    dsr_u64 g = (dsr_u64)blockIdx.x * blockDim.x + threadIdx.x, mask = 0;
+    uint32_t next = 0;
+    if (g < total) {
+        mask = H.R_mask[g >> sh];
+        next = H.R_bid[g >> sh];
+    }
+    for (; g < total; g += stride) {
         const unsigned q = (unsigned)(g & ((1u << sh) - 1));
-        const unsigned live = (unsigned)(H.R_mask[i] >> (4 * q)) & 0xFu;
-        const uint32_t bid = H.R_bid[i];
-        if (live && dsr_check(bid < H.M, H.err, H.dbg, 10, i)) Method::run4(H, T, args, bid, 4 * q, live);
+        const unsigned live = (unsigned)(mask >> (4 * q)) & 0xFu;
+        const uint32_t bid = next;
+        if (g + stride < total) {
+            mask = H.R_mask[(g + stride) >> sh];
+            next = H.R_bid[(g + stride) >> sh];
+        }
+        if (live && dsr_check(bid < H.M, H.err, H.dbg, 10, g >> sh)) Method::run4(H, T, args, bid, 4 * q, live);
     }
     if (dsr_doall_finish(H, keep_list != 0)) dsr_call_finish<Method>(H, T, args, 0);
 }
