@@ -52,7 +52,7 @@ struct dsr_group {
 int dsr__group_take_bytes(dsr_group* g, size_t bytes, void** out);
 void dsr__group_give_bytes(dsr_group* g, void* p, size_t bytes);
 
-void dsr__group_launch_scan(const dsr_group* g, int type, cudaStream_t s, unsigned visits_per_object = 1);
+void dsr__group_launch_scan(const dsr_group* g, int type, cudaStream_t s);
 int dsr__group_grid(const dsr_group* g, const void* kernel, int threads);
 
 // Slots of a block of type T covered per listed block (log2): 5 for
@@ -64,23 +64,17 @@ inline unsigned dsr__group_span(const dsr_group* g, int type) {
 }
 
 // A group do-all: fused scan over every heap, then the method kernel.
-// with_scan / reuse as in dsr__doall: reuse > 0 keeps the block list for
-// that many following do-alls over the same live set, which pass
-// with_scan = false.
 template <class M>
-int dsr__group_doall(dsr_group* g, int type, const typename M::Args& args, cudaStream_t s, bool with_scan = true,
-                     int reuse = 0) {
+int dsr__group_doall(dsr_group* g, int type, const typename M::Args& args, cudaStream_t s) {
     if (type < 0 || type >= g->n_types) return DSR_E_INVALID;
-    if (with_scan) dsr__group_launch_scan(g, type, s, 1u + (unsigned)reuse);
+    dsr__group_launch_scan(g, type, s);
     const int threads = g->tune.threads > 0 ? g->tune.threads : 256;
     if (threads <= 256) {
         const int grid = dsr__group_grid(g, (const void*)dsr_group_doall_kernel_256<M>, threads);
-        dsr_group_doall_kernel_256<M><<<grid, threads, 0, s>>>(g->dev, type, dsr__group_span(g, type), args,
-                                                               reuse > 0 ? 1 : 0);
+        dsr_group_doall_kernel_256<M><<<grid, threads, 0, s>>>(g->dev, type, dsr__group_span(g, type), args, 0);
     } else {
         const int grid = dsr__group_grid(g, (const void*)dsr_group_doall_kernel<M>, threads);
-        dsr_group_doall_kernel<M><<<grid, threads, 0, s>>>(g->dev, type, dsr__group_span(g, type), args,
-                                                           reuse > 0 ? 1 : 0);
+        dsr_group_doall_kernel<M><<<grid, threads, 0, s>>>(g->dev, type, dsr__group_span(g, type), args, 0);
     }
     return dsr__check_launch("dsr_group_doall_kernel");
 }

@@ -210,8 +210,7 @@ __global__ void k_heap_mark_free(const __grid_constant__ dsr_dev_heap H, dsr_u64
 // within a round, so consecutive entries are usually neighbouring blocks.
 // `types` is a bit mask: a do-all over a type with subtypes lists the blocks
 // of every type in its subtree, one type after the other.
-__global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_heap H, uint32_t types,
-                                              unsigned visits_mult) {
+__global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_heap H, uint32_t types) {
     __shared__ unsigned warp_n[8];
     __shared__ unsigned run_base;
     const dsr_u64 M = H.M;
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_he
         }
     }
     objs = __reduce_add_sync(0xFFFFFFFFu, objs);
-    if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs * visits_mult);
+    if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs);
 }
 
 // The lists of a step (dsr_steps.cuh).
@@ -339,9 +338,9 @@ int dsr__scan_grid(const dsr_heap* h, int type) {
     return ctas < 1 ? 1 : (int)ctas;
 }
 
-void dsr__launch_scan(const dsr_heap* h, int type, cudaStream_t s, unsigned visits_per_object, bool exact) {
+void dsr__launch_scan(const dsr_heap* h, int type, cudaStream_t s, bool exact) {
     const uint32_t types = exact ? (1u << type) : h->dev.sub[type];
-    k_scan<<<dsr__scan_grid(h, type), 256, 0, s>>>(h->dev, types, visits_per_object);
+    k_scan<<<dsr__scan_grid(h, type), 256, 0, s>>>(h->dev, types);
 }
 
 void dsr__list_types(const dsr_heap* h, int type_a, int type_b, unsigned mult_a, unsigned mult_b, cudaStream_t s) {
@@ -847,7 +846,7 @@ extern "C" int dsr_heap_dump(dsr_heap* h, int type, void* out_dev, uint64_t cap,
         dsr__set_cuda_error(e, "dsr_heap_dump");
         return DSR_E_CUDA;
     }
-    dsr__launch_scan(h, type, s, 1, true);
+    dsr__launch_scan(h, type, s, true);
     const dsr_u64 most = (h->dev.M * 2 + 8 * DUMP_ITEMS - 1) / (8 * DUMP_ITEMS);
     const dsr_u64 grid = (dsr_u64)h->sm_count * 5;
     k_dump<<<(unsigned)(grid < most ? grid : most), 256, 0, s>>>(h->dev, type, static_cast<uint32_t*>(out_dev),
@@ -859,7 +858,7 @@ extern "C" int dsr_heap_dump(dsr_heap* h, int type, void* out_dev, uint64_t cap,
 extern "C" int dsr_heap_hash(dsr_heap* h, int type, void* hash_dev, void* stream) {
     if (!h || !hash_dev || type < 0 || type >= (int)h->layout.n_types) return DSR_E_INVALID;
     HashArgs a{static_cast<dsr_u64*>(hash_dev)};
-    return dsr__doall<MHash>(h, type, a, dsr__stream(stream), true, nullptr, nullptr, 0, true);
+    return dsr__doall<MHash>(h, type, a, dsr__stream(stream), true, true);
 }
 
 template <class M>

@@ -45,22 +45,16 @@ int dsr__scan_grid(const dsr_heap* h, int type);
 // block and the capacity is a multiple of 4 (vector methods may run).
 bool dsr__vec4_ok(const dsr_heap* h, int type);
 // exact: list the blocks of `type` only, not those of its subtypes.
-void dsr__launch_scan(const dsr_heap* h, int type, cudaStream_t s, unsigned visits_per_object = 1, bool exact = false);
+void dsr__launch_scan(const dsr_heap* h, int type, cudaStream_t s, bool exact = false);
 
 // Run a do-all: scan + compaction of allocated[type] into R, then the method
 // kernel over the listed blocks.
-// ev_scan / ev_run (optional): recorded on s after the scan and after the
-// method kernel, for per-phase timing (as external records, so that under
-// stream capture they become event-record nodes of the graph). reuse > 0: the block list is kept for
-// `reuse` more do-alls over the same live set, and the scan counts each
-// listed object 1 + reuse times as visited (the visits those do-alls make).
 // exact: visit the objects of `type` only, not those of its subtypes.
 template <class M>
 int dsr__doall(dsr_heap* h, int type, const typename M::Args& args, cudaStream_t s, bool with_scan = true,
-               cudaEvent_t ev_scan = nullptr, cudaEvent_t ev_run = nullptr, int reuse = 0, bool exact = false) {
+               bool exact = false) {
     if (type < 0 || type >= h->dev.n_types) return DSR_E_INVALID;
-    if (with_scan) dsr__launch_scan(h, type, s, 1u + (unsigned)reuse, exact);
-    if (ev_scan) cudaEventRecordWithFlags(ev_scan, s, cudaEventRecordExternal);
+    if (with_scan) dsr__launch_scan(h, type, s, exact);
     // The occupancy-limited grid of this kernel and CTA size is looked up
     // once and cached; a heap whose tuning fixes the CTAs per SM computes its
     // own and leaves the cache alone (other heaps keep the occupancy limit).
@@ -86,7 +80,6 @@ int dsr__doall(dsr_heap* h, int type, const typename M::Args& args, cudaStream_t
     int g = (int)g64;
     if ((dsr_u64)g > cap_grid) g = (int)cap_grid;
     if (g < 1) g = 1;
-    int rc;
     if constexpr (dsr_has_run4<M>::value) {
         if (dsr__vec4_ok(h, type)) {
             static int vgrid_cache[17] = {0};
@@ -99,19 +92,15 @@ int dsr__doall(dsr_heap* h, int type, const typename M::Args& args, cudaStream_t
                 vgrid = cached;
             }
             int gv = vgrid < g ? vgrid : g;
-            dsr_doall_kernel_vec4<M><<<gv, threads, 0, s>>>(h->dev, type, args, reuse > 0 ? 1 : 0);
-            rc = dsr__check_launch("dsr_doall_kernel_vec4");
-            if (ev_run) cudaEventRecordWithFlags(ev_run, s, cudaEventRecordExternal);
-            return rc;
+            dsr_doall_kernel_vec4<M><<<gv, threads, 0, s>>>(h->dev, type, args, 0);
+            return dsr__check_launch("dsr_doall_kernel_vec4");
         }
     }
     if (small)
-        dsr_doall_kernel_256<M><<<g, threads, 0, s>>>(h->dev, type, args, reuse > 0 ? 1 : 0);
+        dsr_doall_kernel_256<M><<<g, threads, 0, s>>>(h->dev, type, args, 0);
     else
-        dsr_doall_kernel<M><<<g, threads, 0, s>>>(h->dev, type, args, reuse > 0 ? 1 : 0);
-    rc = dsr__check_launch("dsr_doall_kernel");
-    if (ev_run) cudaEventRecordWithFlags(ev_run, s, cudaEventRecordExternal);
-    return rc;
+        dsr_doall_kernel<M><<<g, threads, 0, s>>>(h->dev, type, args, 0);
+    return dsr__check_launch("dsr_doall_kernel");
 }
 
 // Application method dispatch (defined in the application files).
