@@ -15,7 +15,7 @@
 // Objects of consecutive elements get consecutive slots, so their fields are
 // written coalesced, and later do-alls find neighbours in the same block.
 // Measured (us, dsr_new per thread -> this): 8192 x 4096 traffic cells with
-// 6.7 M cars 1730 -> 342, 1500 x 1000 life cells 761 -> 52, 1.68 M sugarscape
+// 6.7 M cars 1730 -> 161, 1500 x 1000 life cells 761 -> 52, 1.68 M sugarscape
 // agents 434 -> 45, 2048 x 2048 wa-tor 302 -> 74, 4097 bodies 131 -> 13.
 #pragma once
 
@@ -23,17 +23,19 @@
 
 constexpr int DSR_BULK_THREADS = 256;
 constexpr int DSR_BULK_WARPS = DSR_BULK_THREADS / 32;
-constexpr int DSR_BULK_ROWS = 16;     // elements per thread and chunk at most
-constexpr int DSR_BULK_BLOCKS = 256;  // blocks claimed per type and chunk at most
-constexpr int DSR_BULK_REST = 64;     // objects of a chunk beyond its full blocks (a block has at most 64 slots)
-
 template <int NT>
+constexpr int dsr_bulk_rows_max = 32 / NT;  // elements per thread and chunk at most: their kinds fill one word
+constexpr int DSR_BULK_BLOCKS = 256;        // blocks claimed per type and chunk at most
+constexpr int DSR_BULK_REST = 64;           // objects of a chunk beyond its full blocks (a block has at most 64 slots)
+
+template <int NT, bool SPARSE = false>
 struct dsr_bulk_smem {
-    uint32_t before[NT][DSR_BULK_ROWS * DSR_BULK_WARPS];  // objects of the chunk before each (row, warp)
+    uint32_t before[NT][dsr_bulk_rows_max<NT> * DSR_BULK_WARPS];  // objects of the chunk before each (row, warp)
     uint32_t total[NT];
     uint32_t n_blocks[NT];
     uint32_t block[NT][DSR_BULK_BLOCKS];
     dsr_ref rest[NT][DSR_BULK_REST];
+    uint16_t order[SPARSE ? dsr_bulk_rows_max<NT> * DSR_BULK_THREADS : 1];  // of object `rank`: its element in the chunk
 };
 
 // Claim up to `want` free blocks as full blocks of type T (every slot taken
@@ -115,47 +117,60 @@ __device__ __forceinline__ uint32_t dsr_warp_prefix(uint32_t v, uint32_t* total)
     return incl - v;
 }
 
-// Elements 0 .. n - 1, `rows` (1 .. DSR_BULK_ROWS) x 256 of them a chunk, one
+// Elements 0 .. n - 1, `rows` (1 .. dsr_bulk_rows_max<NT>) x 256 of them a chunk, one
 // chunk per CTA and round. kind(i): bit k set if element i creates an object
 // of types[k]. make(i, kind, refs): runs once for every element; refs[k] is
 // the object for bit k (DSR_NULL if the bit is clear or memory ran out).
+// SPARSE (one type): make runs for the elements that create an object only,
+// and 32 of those at a time: the CTA lists them by rank first. With one cell
+// in five holding a car a warp otherwise goes through make for six of its
+// lanes (traffic's initial state, 33.5 M cells: 270 -> 161 us).
 // Called by all 256 threads of every CTA of the grid.
-template <int NT, class Kind, class Make>
+template <int NT, bool SPARSE, class Kind, class Make>
 __device__ __forceinline__ void dsr_bulk_create(const dsr_dev_heap& H, dsr_u64 n, int rows, const int (&types)[NT],
-                                                dsr_bulk_smem<NT>& sm, Kind kind, Make make) {
-    static_assert(NT * DSR_BULK_ROWS <= 32, "a thread keeps its elements' kinds in one word");
+                                                dsr_bulk_smem<NT, SPARSE>& sm, Kind kind, Make make) {
+    static_assert(!SPARSE || NT == 1, "a list of one type's objects");
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1;
     const dsr_u64 chunk = (dsr_u64)rows * DSR_BULK_THREADS;
     for (dsr_u64 base = blockIdx.x * chunk; base < n; base += gridDim.x * chunk) {
         unsigned kinds = 0;
-        for (int r = 0; r < rows; ++r) {
-            const dsr_u64 i = base + r * DSR_BULK_THREADS + threadIdx.x;
-            const unsigned m = i < n ? kind(i) : 0u;
-            kinds |= m << (NT * r);
+        for (int r0 = 0; r0 < rows; r0 += 8) {  // eight elements of a thread are loaded at a time
+            unsigned m[8];
 #pragma unroll
-            for (int k = 0; k < NT; ++k) {
-                const unsigned b = __ballot_sync(0xFFFFFFFFu, (m >> k) & 1u);
-                if (lane == 0) sm.before[k][r * DSR_BULK_WARPS + warp] = __popc(b);
+            for (int q = 0; q < 8; ++q) {
+                const dsr_u64 i = base + (r0 + q) * DSR_BULK_THREADS + threadIdx.x;
+                m[q] = r0 + q < rows && i < n ? kind(i) : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (r0 + q >= rows) break;
+                kinds |= m[q] << (NT * (r0 + q));
+#pragma unroll
+                for (int k = 0; k < NT; ++k) {
+                    const unsigned b = __ballot_sync(0xFFFFFFFFu, (m[q] >> k) & 1u);
+                    if (lane == 0) sm.before[k][(r0 + q) * DSR_BULK_WARPS + warp] = __popc(b);
+                }
             }
         }
         __syncthreads();
         if (warp < NT) {
-            // exclusive prefix sum over the (row, warp) counts, four a lane
+            // exclusive prefix sum over the (row, warp) counts, some of them a lane
+            constexpr int PER = dsr_bulk_rows_max<NT> * DSR_BULK_WARPS / 32;
             uint32_t* c = sm.before[warp];
             const int m = rows * DSR_BULK_WARPS;
-            uint32_t v[4], sum = 0;
+            uint32_t v[PER], sum = 0;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int at = 4 * (int)lane + q;
+            for (int q = 0; q < PER; ++q) {
+                const int at = PER * (int)lane + q;
                 v[q] = at < m ? c[at] : 0u;
                 sum += v[q];
             }
             uint32_t total;
             uint32_t at = dsr_warp_prefix(sum, &total);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (4 * (int)lane + q < m) c[4 * (int)lane + q] = at;
+            for (int q = 0; q < PER; ++q) {
+                if (PER * (int)lane + q < m) c[PER * (int)lane + q] = at;
                 at += v[q];
             }
             const int T = types[warp];
@@ -176,6 +191,33 @@ __device__ __forceinline__ void dsr_bulk_create(const dsr_dev_heap& H, dsr_u64 n
             const uint32_t at = (warp & 1) * 32 + lane;
             const uint32_t full = sm.n_blocks[k] * H.cap[types[k]];
             if (full + at < sm.total[k]) sm.rest[k][at] = dsr_new(H, types[k]);
+        }
+        if constexpr (SPARSE) {
+            for (int r = 0; r < rows; ++r) {
+                const bool set = (kinds >> r) & 1u;
+                const unsigned b = __ballot_sync(0xFFFFFFFFu, set);
+                if (set)
+                    sm.order[sm.before[0][r * DSR_BULK_WARPS + warp] + __popc(b & below)] =
+                        (uint16_t)(r * DSR_BULK_THREADS + threadIdx.x);
+            }
+            __syncthreads();
+            const uint32_t total = sm.total[0], cap = H.cap[types[0]], full = sm.n_blocks[0] * cap;
+            for (uint32_t at = warp * 32; at < total; at += DSR_BULK_THREADS) {
+                const uint32_t rank = at + lane;
+                if (rank < total) {
+                    dsr_ref ref[1];
+                    if (rank < full)
+                        ref[0] = ((dsr_ref)sm.block[0][rank / cap] << 6) | (rank % cap);
+                    else if (rank - full < DSR_BULK_REST)
+                        ref[0] = sm.rest[0][rank - full];
+                    else
+                        ref[0] = dsr_new(H, types[0]);  // the free bitmap gave fewer blocks than asked for
+                    make(base + sm.order[rank], 1u, ref);
+                }
+                __syncwarp();  // whole-warp groups for dsr_new
+            }
+            __syncthreads();  // the tables are reused by the next chunk
+            continue;
         }
         __syncthreads();
         for (int r = 0; r < rows; ++r) {
@@ -205,12 +247,14 @@ __device__ __forceinline__ void dsr_bulk_create(const dsr_dev_heap& H, dsr_u64 n
     }
 }
 
-// Rows of a chunk for n elements: enough chunks for about four CTAs on every
-// SM, and as many elements a chunk (up to 4096) as that allows, so that few
-// of a chunk's objects fall outside its full blocks.
+// Rows of a chunk for n elements of which each may create objects of NT
+// types: enough chunks for about four CTAs on every SM, and as many elements a
+// chunk as that allows, so that few of a chunk's objects fall outside its full
+// blocks.
+template <int NT>
 inline int dsr__bulk_rows(dsr_u64 n, int sm_count) {
     const dsr_u64 r = n / ((dsr_u64)DSR_BULK_THREADS * 4 * (dsr_u64)sm_count);
-    return r < 1 ? 1 : (r > DSR_BULK_ROWS ? DSR_BULK_ROWS : (int)r);
+    return r < 1 ? 1 : (r > (dsr_u64)dsr_bulk_rows_max<NT> ? dsr_bulk_rows_max<NT> : (int)r);
 }
 inline unsigned dsr__bulk_grid(dsr_u64 n, int rows, int sm_count) {
     const dsr_u64 c = (n + (dsr_u64)rows * DSR_BULK_THREADS - 1) / ((dsr_u64)rows * DSR_BULK_THREADS);

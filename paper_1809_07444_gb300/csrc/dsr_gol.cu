@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(DSR_BULK_THREADS)
 
 int launch_init(const dsr_heap* heap, int W, int H, const void* alive0_dev, void* cell_ref_dev, cudaStream_t s) {
     const dsr_u64 n = (dsr_u64)W * H;
-    const int rows = dsr__bulk_rows(n, heap->sm_count);
+    const int rows = dsr__bulk_rows<2>(n, heap->sm_count);
     k_gol_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
         heap->dev, static_cast<const uint8_t*>(alive0_dev), static_cast<dsr_ref*>(cell_ref_dev), W, H, rows);
     return dsr__check_launch("k_gol_init");

@@ -720,7 +720,7 @@ struct MClone {
 // it lies in, so a warp gathers its rows in shared memory and writes them out
 // word by word in order; and a CTA takes its rows' places with one atomic for
 // 32 items of 32 slots (one per warp and item queues up on the counter:
-// 6.7 M cars 160 -> 93 us).
+// 6.7 M cars 160 -> 61 us).
 constexpr int DUMP_ITEMS = 4;   // items of a warp at a time (fewer in a short list)
 constexpr int DUMP_ROW = 2 * DSR_MAX_FIELDS + 2;
 __global__ void __launch_bounds__(256) k_dump(const __grid_constant__ dsr_dev_heap H, int T, uint32_t* out,

@@ -618,8 +618,8 @@ __global__ void __launch_bounds__(TILE) k_force64(const __grid_constant__ dsr_de
 // groups are so large that either side has at most `slots` entries (but a
 // tile group's sums must fit shared memory), and the update adds the entries
 // of a body in a fixed order: a step stays deterministic.
-// Measured, 65,322 bodies FP32: k_force_part 1990 -> @F32@ us; 8000 bodies
-// FP64: 2560 -> @F64@; 4097 bodies FP32: 30 -> @F4@.
+// Measured, 65,322 bodies FP32: k_force_part 1990 -> 1477 us; 8000 bodies
+// FP64: 2560 -> 1312; 4097 bodies FP32: 30 -> 19.
 struct SymShape {
     uint32_t n, nr, nt;  // padded count, rows, tiles
     uint32_t RG, TR;     // rows and tiles of a group
@@ -1536,7 +1536,7 @@ extern "C" int dsr_nbody_create(dsr_heap* heap, const dsr_nbody_params* p, const
         delete nb;
         return DSR_E_CUDA;
     }
-    const int rows = dsr__bulk_rows((dsr_u64)n_bodies, heap->sm_count);
+    const int rows = dsr__bulk_rows<1>((dsr_u64)n_bodies, heap->sm_count);
     k_nbody_init<<<dsr__bulk_grid((dsr_u64)n_bodies, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
         heap->dev, static_cast<const float*>(rows_dev), n_bodies, rows);
     int rc = dsr__check_launch("k_nbody_init");

@@ -383,7 +383,7 @@ extern "C" int dsr_sugarscape_create(dsr_heap* heap, const dsr_sugarscape_params
     const int ctas = heap->sm_count * 8;
     k_sugar_fill<<<ctas, 256, 0, s>>>(w.cell, static_cast<const uint8_t*>(cap_dev), n);
     if (n_agents) {
-        const int rows = dsr__bulk_rows((dsr_u64)n_agents, heap->sm_count);
+        const int rows = dsr__bulk_rows<1>((dsr_u64)n_agents, heap->sm_count);
         k_sugar_init<<<dsr__bulk_grid((dsr_u64)n_agents, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
             heap->dev, static_cast<const int32_t*>(agents0_dev), n_agents, w, p->W, rows);
     }

@@ -151,11 +151,11 @@ __global__ void __launch_bounds__(256, 5)
     if (blockIdx.x == 0 && threadIdx.x == 0) dsr_end_step(H.R_count);
 }
 
-// One thread per cell: a Car where v0 >= 0.
+// A Car for every cell where v0 >= 0.
 __global__ void __launch_bounds__(DSR_BULK_THREADS)
     k_traffic_init(const __grid_constant__ dsr_dev_heap H, const int8_t* v0, uint8_t* cur, dsr_traffic_params p,
                    int rows) {
-    __shared__ dsr_bulk_smem<1> sm;
+    __shared__ dsr_bulk_smem<1, true> sm;
     const int types[1] = {CAR};
     const dsr_u64 n = (dsr_u64)p.R * p.L;
     const bool small = n <= 0xFFFFFFFFull;  // 32-bit divisions are several times cheaper than 64-bit ones
@@ -250,11 +250,11 @@ extern "C" int dsr_traffic_create(dsr_heap* heap, const dsr_traffic_params* p, c
         return DSR_E_CUDA;
     }
     const dsr_u64 n = (dsr_u64)p->R * p->L;
-    const int rows = dsr__bulk_rows(n, heap->sm_count);
+    const int rows = dsr__bulk_rows<1>(n, heap->sm_count);
     k_traffic_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
         heap->dev, static_cast<const int8_t*>(v0_dev), t->grid[0], *p, rows);
     if (!p->periodic) {
-        const int srows = dsr__bulk_rows((dsr_u64)p->R, heap->sm_count);
+        const int srows = dsr__bulk_rows<1>((dsr_u64)p->R, heap->sm_count);
         k_traffic_sources<<<dsr__bulk_grid((dsr_u64)p->R, srows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
             heap->dev, p->R, srows);
     }

@@ -536,7 +536,7 @@ dsr_u64 bm_slots(const dsr_bm_heap* h) {
 
 int launch_init(const dsr_heap* heap, const WatorInst& I, const void* kind0_dev, cudaStream_t s) {
     const uint32_t n = (uint32_t)I.p.W * (uint32_t)I.p.H;
-    const int rows = dsr__bulk_rows(n, heap->sm_count);
+    const int rows = dsr__bulk_rows<2>(n, heap->sm_count);
     k_wator_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
         heap->dev, static_cast<const uint8_t*>(kind0_dev), I, rows);
     return dsr__check_launch("k_wator_init");

@@ -165,3 +165,25 @@ def test_dump_rows_and_capacity(fields, n, narrow):
     assert int(cnt.item()) == len(handles)
     assert (out[cap * row:] == -1).all()
     assert h.stats()["error_flags"] != 0
+
+
+@pytest.mark.parametrize("R,L,density", [(1, 2, 1.0), (3, 85, 0.5), (64, 64, 1.0), (63, 65, 0.01), (701, 997, 0.03),
+                                         (4096, 300, 0.2), (128, 8192, 1.0)])
+@pytest.mark.parametrize("tuning", [None, {"cap_min": 32}, {"fanout": 16}])
+def test_traffic_initial_cars(R, L, density, tuning):
+    from paper_1809_07444_gb300.apps import TRAFFIC_TYPES, Traffic
+    from paper_1809_07444_gb300.heap import heap_bytes_for_blocks
+
+    from helpers import check_stats
+
+    v0 = WL.traffic_initial(R, L, R + L, density=density, vmax=1)
+    road, x = np.nonzero(v0 >= 0)
+    # a heap with few more slots than cars, and one with room
+    cap = 32 if tuning and "cap_min" in tuning else 64
+    for blocks in (17 * len(x) // (16 * cap) + 64, 4 * (len(x) // cap) + 256):
+        g = Traffic(R, L, v0, 1, vmax=1, periodic=True, tuning=tuning,
+                    heap_bytes=heap_bytes_for_blocks(TRAFFIC_TYPES, blocks, tuning))
+        cars, _ = g.dump()
+        assert np.array_equal(cars, np.stack([road, x, v0[road, x]], 1))
+        st = check_stats(g.heap)
+        assert st["error_flags"] == 0 and st["live_objects"][0] == len(x)
