@@ -10,9 +10,9 @@
 // entry's mask by the survivors (kMarks) where a later do-all of the step
 // visits them. Two do-alls that do not depend on each other share a launch.
 //
-// A warp takes every W-th (block, 32 slots) item of a heap's list, so that at
-// any time the grid works on neighbouring entries; a CTA of a group do-all takes
-// one stretch, which lies in one or two heaps. A warp's 32 lanes load the entries of its next 32
+// A warp takes every W-th (block, 32 slots) item of the list, so that at any
+// time the grid works on neighbouring entries; a CTA of a group do-all that
+// creates takes one stretch, which lies in one or two heaps. A warp's 32 lanes load the entries of its next 32
 // items at once and hand them out by shuffle, so the list costs one round
 // trip per 32 items and warp, not one per item.
 //
@@ -355,10 +355,16 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
     // go to few CTAs, one to a warp: what a CTA defers is then worth a block.
     const dsr_u64 wanted = (items + warps - 1) / warps;
     const uint32_t ctas = wanted < gridDim.x ? (uint32_t)wanted : gridDim.x;
-    // items first, first + 1 .. (groups) or first, first + stride .. of this warp
-    const uint32_t end = Space::kGroup ? (uint32_t)(cta < ctas ? items * (cta + 1) / ctas : 0) : (uint32_t)items;
-    const uint32_t stride = Space::kGroup ? warps : ctas * warps;
-    const uint32_t cta0 = cta >= ctas ? end : Space::kGroup ? (uint32_t)(items * cta / ctas) : cta * warps;
+    // Group do-alls that create take a stretch of items per CTA, so that a
+    // CTA's births belong to one or two heaps. All others take every
+    // (ctas * warps)-th item per warp: the grid is then at one place of the
+    // list, and of the instances' grids, at a time (256 wa-tor instances, 46.6 M
+    // cells, several times what L2 holds: with stretches the fish-choice
+    // kernel took 1389 us, with every n-th item 629).
+    constexpr bool kStretch = Space::kGroup && M::kDefers != DSR_NOTHING;
+    const uint32_t end = kStretch ? (uint32_t)(cta < ctas ? items * (cta + 1) / ctas : 0) : (uint32_t)items;
+    const uint32_t stride = kStretch ? warps : ctas * warps;
+    const uint32_t cta0 = cta >= ctas ? end : kStretch ? (uint32_t)(items * cta / ctas) : cta * warps;
     dsr_later later{nullptr, nullptr, 0, M::kDefers != DSR_NOTHING};
     if constexpr (M::kDefers != DSR_NOTHING) {
         later.np = &sm->np;
