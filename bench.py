@@ -696,8 +696,8 @@ def bench_gol(W=64, gens=100, reps=3):
         del g
     lat.sort()
     return {"workload": "game of life %dx%d, %d generations" % (W, W, gens), "gens_per_s": statistics.median(rates),
-            "gen_ms_p50": lat[len(lat) // 2], "gen_ms_p99": lat[int(len(lat) * 0.99)], "kernels_per_gen": 6,
-            "graph": "one graph launch per generation"}
+            "gen_ms_p50": lat[len(lat) // 2], "gen_ms_p99": lat[int(len(lat) * 0.99)], "kernels_per_gen": 1,
+            "graph": "none: one cluster launch per call (one generation a call here)"}
 
 
 def bench_comparators(steps=50, warmup=5):
@@ -790,7 +790,7 @@ def bench_traffic(steps=30, warmup=3):
             "cars_at_start": cars0, "flow_per_cell": vsum / (R * L * steps),
             "entered": ctr1["app0"] - ctr0["app0"], "left": ctr1["app1"] - ctr0["app1"],
             "algorithmic_gbs": alg / t / 1e9, "hbm_frac": alg / t / 1e9 / peak, "peak_gbs": peak,
-            "peak_kind": peak_kind, "launches_per_step": 4, "memsets_per_step": 1}
+            "peak_kind": peak_kind, "launches_per_step": 3, "memsets_per_step": 0}
 
 
 SUGAR_SIDE = 4096
@@ -1016,7 +1016,7 @@ def bench_served(seconds=20.0, n_jobs=10000, arena_gb=64, lo=128, hi=4096, steps
 # the (steps, warmup) window it was taken on. The bench reports it only when
 # it runs that window (the population, hence the bytes of a launch, changes
 # from step to step); a kernel changed since its capture has no entry.
-TRAFFIC = {"F2": {"bytes": 68276505, "steps": 20, "warmup": 5, "cache_control": "none",
+TRAFFIC = {"F2": {"bytes": 68980237, "steps": 20, "warmup": 5, "cache_control": "none",
                   "source": "profiles/wator2048_fish_move_traffic.md"}}
 
 

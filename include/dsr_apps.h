@@ -42,15 +42,17 @@ int dsr_gol_workspace_bytes(int W, int H, size_t* out);
  * initial Alive objects inside the heap. */
 int dsr_gol_create(dsr_heap* heap, int W, int H, const void* alive0_dev, void* workspace_dev, void* stream,
                    dsr_gol** out);
-/* The first call captures one generation (its launches) into a CUDA
- * graph on a stream of its own; every generation is then one graph launch
- * on `stream`. Make the first call outside any stream capture. */
+/* A small heap (up to 768 blocks, default threads and CTAs per SM) runs all
+ * its generations in one launch of a thread-block cluster. Otherwise the
+ * first call captures one generation (its launches) into a CUDA graph on a
+ * stream of its own; every generation is then one graph launch on `stream`.
+ * Make the first call outside any stream capture. */
 int dsr_gol_step(dsr_gol* g, int n_gen, void* stream);
 int dsr_gol_destroy(dsr_gol* g);
 
 /* Batched game of life: many instances, each with its own heap in one heap
- * group, advanced together by three group do-alls per generation captured
- * into a CUDA graph (same conventions as the batched wa-tor below). */
+ * group, advanced together by one list and two group kernels per generation,
+ * captured into a CUDA graph (same conventions as the batched wa-tor below). */
 typedef struct dsr_gol_batch dsr_gol_batch;
 int dsr_gol_batch_create(void* arena_dev, size_t arena_bytes, int max_instances, const dsr_tuning* tune, void* stream,
                          dsr_gol_batch** out);
@@ -120,7 +122,9 @@ int dsr_wator_workspace_bytes(const dsr_heap* heap, int W, int H, size_t* out);
 int dsr_wator_create(dsr_heap* heap, const dsr_wator_params* p, const void* kind0_dev, void* workspace_dev,
                      void* stream, dsr_wator** out);
 /* Advances n_steps steps on `stream` (each step: F1, F2, S0, S1, S2 as
- * do-alls). A step is replayed from a CUDA graph of its launches that the
+ * do-alls). A small heap (up to 1024 blocks, default threads and CTAs per SM,
+ * no phase timing) runs all n_steps in one launch of a thread-block cluster.
+ * Otherwise a step is replayed from a CUDA graph of its launches that the
  * handle captures on first use on a private stream (one for untimed steps,
  * one for the current dsr_wator_phase_timing / _phase_select setting, which
  * is captured when that setting is made); while `stream` is itself being
@@ -201,8 +205,8 @@ int dsr_wator_static_destroy(dsr_wator_static* w);
  * Many independent wa-tor instances (each with its own sizes, parameters and
  * seed) advance together: every instance has its own heap in a heap group
  * (dsr_group_* in dsr.h) carved from one caller-owned arena, and one batched
- * step is five group do-alls (one fused scan and one method kernel each) over
- * all instances, captured once into a CUDA graph and replayed until an
+ * step is five group do-alls (one list of both types, four kernels) over all
+ * instances, captured once into a CUDA graph and replayed until an
  * instance is added or removed. Each instance follows exactly the rules and
  * results of the plain form. The arena must be 256-byte aligned; its first
  * bytes hold the instance table. */
@@ -266,9 +270,11 @@ int dsr_wator_batch_destroy(dsr_wator_batch* b);
  * body. Every sum has a fixed order: a step is deterministic.
  * Workspace (dsr_nbody_workspace_bytes): the cell counts and offsets, the
  * sorted per-body arrays for all M * 64 slots of the heap (rounded up to
- * 1024), the slice buffers of the split all-pairs kernels (sized from the
- * device's SM count and the kernels' occupancy, so query it on the device
- * that will run the step), and a merge log of log_cap entries. */
+ * 1024), the partial sums of the all-pairs kernels (for up to 163,840
+ * positions those of the kernels that take every unordered pair once, 315 MB
+ * at 65,536 bodies; otherwise sized from the device's SM count and the
+ * kernels' occupancy, so query it on the device that will run the step), and
+ * a merge log of log_cap entries. */
 #define DSR_NBODY_PAIRS_FP32 0
 #define DSR_NBODY_PAIRS_FP64 1
 typedef struct {
