@@ -149,6 +149,8 @@ __global__ void __launch_bounds__(DSR_CLUSTER_THREADS, 1)
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     const dsr_phase cells{CELL, 0}, alive{ALIVE, 1};
     const unsigned hc = H.span_sh[CELL] - 5, ha = H.span_sh[ALIVE] - 5;
+    dsr_clear_sets(H.R_count, first);
+    dsr_cluster_barrier();
     // the cells' list length stays in set 0's front word, the Alive objects'
     // take turns in the two back words
     dsr_list<T>(H, CELL, -1, 2u * (unsigned)n, 0, DSR_SET, list);
@@ -166,10 +168,7 @@ __global__ void __launch_bounds__(DSR_CLUSTER_THREADS, 1)
         dsr_run_list<DDie<A>, dsr_heap_space, T>(S, alive, a, ha, true, nullptr);
         dsr_cluster_barrier();
     }
-    if (first) {
-        dsr_clear_set(H.R_count, DSR_SET);
-        dsr_clear_set(H.R_count, DSR_SET + 2);
-    }
+    dsr_clear_sets(H.R_count, first);
 }
 
 // One thread per cell: create the Cell and, where alive, its Alive object.

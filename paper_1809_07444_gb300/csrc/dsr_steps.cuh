@@ -527,6 +527,16 @@ __device__ __forceinline__ void dsr_clear_set(uint32_t* R_count, uint32_t set) {
     w[set] = 0;
     w[set + 1] = 0;
 }
+// The first thing a cluster's kernel does (`first`: one thread of the grid):
+// both sets are zero behind the next cluster barrier. A step of the general
+// form leaves its own set's lengths for the step after it to clear, and a heap
+// can take both forms in turn (timed wa-tor steps are general ones).
+__device__ __forceinline__ void dsr_clear_sets(uint32_t* R_count, bool first) {
+    if (first) {
+        dsr_clear_set(R_count, DSR_SET);
+        dsr_clear_set(R_count, DSR_SET + 2);
+    }
+}
 
 // All writes of the cluster's threads before it are visible to all of them after it.
 __device__ __forceinline__ void dsr_cluster_barrier() {

@@ -414,6 +414,8 @@ __global__ void __launch_bounds__(DSR_CLUSTER_THREADS, 1)
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     const dsr_phase fish{FISH, 0}, sharks{SHARK, 1};
     const unsigned hf = H.span_sh[FISH] - 5, hs = H.span_sh[SHARK] - 5;
+    dsr_clear_sets(H.R_count, first);
+    dsr_cluster_barrier();
     for (int t = 0; t < n; ++t) {
         const uint32_t set = DSR_SET + 2 * (t & 1), other = DSR_SET + 2 * (~t & 1);
         dsr_list<T>(H, FISH, SHARK, 2, 1, set, list);
