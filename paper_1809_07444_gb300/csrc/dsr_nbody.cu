@@ -1293,31 +1293,47 @@ uint32_t split_grid(const dsr_heap* h, const void* kernel) {
 constexpr uint64_t kSymPositions = 160 * 1024;
 constexpr int kSymSmallBodies = 16384;
 
+// Grid and dynamic shared memory of a symmetric kernel; grid 0: it does not run.
+struct SymLaunch {
+    uint32_t grid = 0;
+    size_t smem = 0;
+};
 struct SplitGrids {
     uint32_t force, force64;
-    uint32_t sym, sym_small, sym64;  // grids of the symmetric kernels
+    SymLaunch sym, sym_small, sym64;
 };
 
 template <class F>
-size_t sym_smem(uint64_t n) {
-    // a smaller live count may have larger tile groups (SLOTS below SLOTS_FEW is not the case)
-    const SymShape q = sym_shape((uint32_t)n, F::THREADS, F::RB, sym_slots<F>((uint32_t)n), F::MAX_TR);
-    return F::THREADS * sizeof(typename F::Vec) + (size_t)q.TR * F::SUMS * F::THREADS * sizeof(typename F::Real);
+SymShape sym_shape_of(uint64_t n) {
+    return sym_shape((uint32_t)n, F::THREADS, F::RB, sym_slots<F>((uint32_t)n), F::MAX_TR);
 }
-// CTAs of a symmetric kernel that fit at once, with the shared memory of n positions.
+// Launch of a symmetric kernel on a heap of P padded positions. A step takes
+// its shape from the bodies it finds in the heap, which may be more than the
+// n_bodies placed at creation (a heap that held bodies before, or whose
+// program creates some): the shared memory has room for the largest tile
+// group of any padded count up to P. The grid, which any count can run with,
+// suits n_bodies.
 template <class F>
-uint32_t sym_grid(const dsr_heap* h, uint64_t n) {
-    const size_t most = F::THREADS * sizeof(typename F::Vec) +
-                        (size_t)F::MAX_TR * F::SUMS * F::THREADS * sizeof(typename F::Real);
-    cudaFuncSetAttribute(k_force_sym<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+SymLaunch sym_launch(const dsr_heap* h, uint64_t n_bodies, uint64_t P) {
+    auto smem = [](uint32_t tr) {
+        return F::THREADS * sizeof(typename F::Vec) + (size_t)tr * F::SUMS * F::THREADS * sizeof(typename F::Real);
+    };
+    uint32_t tr = 1;
+    for (uint64_t n = ROW; n <= P; n += ROW) {
+        const uint32_t t = sym_shape_of<F>(n).TR;
+        if (t > tr) tr = t;
+    }
+    SymLaunch l;
+    l.smem = smem(tr);
+    cudaFuncSetAttribute(k_force_sym<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(F::MAX_TR));
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_force_sym<F>, F::THREADS, sym_smem<F>(n)) !=
-            cudaSuccess || occ < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_force_sym<F>, F::THREADS, l.smem) != cudaSuccess ||
+        occ < 1)
         occ = 1;
     if (occ > F::CTAS) occ = F::CTAS;
     // as many CTAs as items, in whole CTAs per SM: an idle CTA's SM would be
     // short of the work that another SM has too much of
-    const SymShape q = sym_shape((uint32_t)n, F::THREADS, F::RB, sym_slots<F>((uint32_t)n), F::MAX_TR);
+    const SymShape q = sym_shape_of<F>(n_bodies);
     uint64_t items = 0;
     for (uint32_t ga = 0; ga < q.na; ++ga)
         for (uint32_t gb = 0; gb < q.nb; ++gb) {
@@ -1325,11 +1341,12 @@ uint32_t sym_grid(const dsr_heap* h, uint64_t n) {
             items += t1 > F::RB * ga * q.RG;
         }
     const uint64_t per_sm = (items + h->sm_count - 1) / h->sm_count;
-    return (uint32_t)((per_sm < (uint64_t)occ ? per_sm : (uint64_t)occ) * h->sm_count);
+    l.grid = (uint32_t)((per_sm < (uint64_t)occ ? per_sm : (uint64_t)occ) * h->sm_count);
+    return l;
 }
 
 SplitGrids split_grids(const dsr_heap* h) {
-    return {split_grid(h, (const void*)k_force_part<true>), split_grid(h, (const void*)k_force_part64), 0, 0, 0};
+    return {split_grid(h, (const void*)k_force_part<true>), split_grid(h, (const void*)k_force_part64), {}, {}, {}};
 }
 
 // Padded positions for a heap of S slots.
@@ -1354,15 +1371,13 @@ size_t part_bytes(uint64_t P, SplitGrids g) {
         if (a > m) m = a;
         if (b > m) m = b;
         if (P > kSymPositions) continue;
-        auto sym = [&](uint32_t threads, uint32_t rb, uint32_t slots, uint32_t few, uint32_t max_tr, size_t entry) {
-            const SymShape q = sym_shape((uint32_t)n, threads, rb, n <= kSymFew ? few : slots, max_tr);
+        auto sym = [&](const SymShape& q, size_t entry) {
             const size_t c = (size_t)(q.na + q.nb) * n * entry;
             if (c > m) m = c;
         };
-        sym(SymF32::THREADS, SymF32::RB, SymF32::SLOTS, SymF32::SLOTS_FEW, SymF32::MAX_TR, 16);
-        if (n <= padded(kSymSmallBodies))
-            sym(SymF32Small::THREADS, SymF32Small::RB, SymF32Small::SLOTS, SymF32Small::SLOTS_FEW, SymF32Small::MAX_TR, 16);
-        sym(SymF64::THREADS, SymF64::RB, SymF64::SLOTS, SymF64::SLOTS_FEW, SymF64::MAX_TR, 32);
+        sym(sym_shape_of<SymF32>(n), 16);
+        sym(sym_shape_of<SymF32Small>(n), 16);
+        sym(sym_shape_of<SymF64>(n), 32);
     }
     return m;
 }
@@ -1445,14 +1460,14 @@ void launch_sort(dsr_heap* h, const NbArgs& a, cudaStream_t s) {
 }
 
 template <class F>
-FarShape launch_sym(const NbArgs& a, uint32_t grid, uint64_t n, cudaStream_t s) {
-    k_force_sym<F><<<grid, F::THREADS, sym_smem<F>(n), s>>>(a);
+FarShape launch_sym(const NbArgs& a, const SymLaunch& l, cudaStream_t s) {
+    k_force_sym<F><<<l.grid, F::THREADS, l.smem, s>>>(a);
     return FarShape{0, (uint32_t)F::THREADS, (uint32_t)F::RB, F::SLOTS, F::SLOTS_FEW, F::MAX_TR};
 }
 
 // One step. `split`: the force kernels' grids (else the unsplit ones, for the
-// allocation-free step); P: padded positions; n0: bodies at most (the heap's
-// bodies at creation; merges only reduce them).
+// allocation-free step); P: padded positions; n0: bodies placed at creation,
+// by which the FP32 form is chosen (either form takes any count up to P).
 void launch_step(dsr_heap* h, const NbArgs& a, const SplitGrids* split, uint64_t P, uint64_t n0, cudaStream_t s) {
     const unsigned ctas = (unsigned)(h->sm_count * 4);
     const bool f64 = a.p.pair_precision == DSR_NBODY_PAIRS_FP64;
@@ -1461,11 +1476,10 @@ void launch_step(dsr_heap* h, const NbArgs& a, const SplitGrids* split, uint64_t
     launch_sort<false>(h, a, s);
     k_gather<<<ctas, TILE, 0, s>>>(h->dev, a.ws);
     FarShape far{0, 0, 0, 0, 0, 0};
-    if (split && soft && split->sym) {
-        const uint64_t n = padded(n0);
-        far = f64 ? launch_sym<SymF64>(a, split->sym64, n, s)
-              : n0 <= (uint64_t)kSymSmallBodies ? launch_sym<SymF32Small>(a, split->sym_small, n, s)
-                                                : launch_sym<SymF32>(a, split->sym, n, s);
+    if (split && soft && split->sym.grid) {
+        far = f64 ? launch_sym<SymF64>(a, split->sym64, s)
+              : n0 <= (uint64_t)kSymSmallBodies ? launch_sym<SymF32Small>(a, split->sym_small, s)
+                                                : launch_sym<SymF32>(a, split->sym, s);
     } else if (split) {
         far.grid = f64 ? split->force64 : split->force;
         if (f64)
@@ -1520,10 +1534,10 @@ extern "C" int dsr_nbody_create(dsr_heap* heap, const dsr_nbody_params* p, const
     nb->n0 = (uint64_t)n_bodies;
     nb->grid = split_grids(heap);
     if (padded(nb->S) <= kSymPositions) {
-        const uint64_t n = padded(nb->n0);
-        nb->grid.sym = sym_grid<SymF32>(heap, n);
-        nb->grid.sym_small = sym_grid<SymF32Small>(heap, n < padded(kSymSmallBodies) ? n : padded(kSymSmallBodies));
-        nb->grid.sym64 = sym_grid<SymF64>(heap, n);
+        const uint64_t n = padded(nb->n0), P = padded(nb->S);
+        nb->grid.sym = sym_launch<SymF32>(heap, n, P);
+        nb->grid.sym_small = sym_launch<SymF32Small>(heap, n < padded(kSymSmallBodies) ? n : padded(kSymSmallBodies), P);
+        nb->grid.sym64 = sym_launch<SymF64>(heap, n, P);
     }
     nb->args.ws = carve(workspace_dev, nb->S, log_cap, nb->grid);
     nb->args.ws.K = cells_per_axis(*p);
