@@ -133,6 +133,8 @@ struct DBirth : GolMethod<A> {
 // One scan lists both types. A birth and a death never meet: a cell that
 // dies has not 3 alive neighbours, and new Alive objects are in no list.
 constexpr dsr_phase kCells{CELL, 0}, kAlive{ALIVE, 1};
+// A list of its own for each do-all, of a type and its subtypes.
+constexpr dsr_phase kAliveTree{ALIVE, 0};
 
 // Generations of a small board in one launch of one cluster (dsr_steps.cuh).
 // No Cell is ever created or deleted after the first list, which so serves
@@ -252,8 +254,19 @@ extern "C" int dsr_gol_create(dsr_heap* heap, int W, int H, const void* alive0_d
     return DSR_OK;
 }
 
+static bool has_subtypes(const dsr_heap* h) { return dsr__has_subtypes(h, CELL) || dsr__has_subtypes(h, ALIVE); }
+
 static int issue_generation(dsr_gol* g, cudaStream_t s) {
     typedef GolArgs A;
+    if (has_subtypes(g->heap)) {
+        dsr__list_tree(g->heap, CELL, 1, s);
+        int rc = dsr__step<DCount<A>, dsr_no_method, true>(g->heap, kCells, kCells, g->args, s);
+        dsr__list_tree(g->heap, ALIVE, 1, s);
+        if (!rc) rc = dsr__step<DDie<A>, dsr_no_method, true>(g->heap, kAliveTree, kAliveTree, g->args, s);
+        dsr__list_tree(g->heap, CELL, 1, s);
+        if (!rc) rc = dsr__step<DBirth<A>, dsr_no_method, true>(g->heap, kCells, kCells, g->args, s);
+        return rc;
+    }
     dsr__list_types(g->heap, CELL, ALIVE, 2, 1, s);
     int rc = dsr__step<DCount<A>>(g->heap, kCells, kCells, g->args, s);
     if (!rc) rc = dsr__step<DBirth<A>, DDie<A>, true>(g->heap, kCells, kAlive, g->args, s);
@@ -272,7 +285,7 @@ extern "C" int dsr_gol_step(dsr_gol* g, int n_gen, void* stream) {
     if (!g || n_gen < 0) return DSR_E_INVALID;
     cudaStream_t s = dsr__stream(stream);
     static const bool fits = dsr__cluster_fits((const void*)k_gol_steps);
-    if (fits && dsr__small_heap(g->heap, kSmallBlocks)) {
+    if (fits && dsr__small_heap(g->heap, kSmallBlocks) && !has_subtypes(g->heap)) {
         for (int i = 0; i < n_gen;) {
             int n = n_gen - i < DSR_CLUSTER_STEPS ? n_gen - i : DSR_CLUSTER_STEPS;
             void* args[] = {&g->heap->dev, &g->args, &n};

@@ -210,7 +210,9 @@ __global__ void k_heap_mark_free(const __grid_constant__ dsr_dev_heap H, dsr_u64
 // within a round, so consecutive entries are usually neighbouring blocks.
 // `types` is a bit mask: a do-all over a type with subtypes lists the blocks
 // of every type in its subtree, one type after the other.
-__global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_heap H, uint32_t types) {
+// `count` (used by thread 0): the list's length. Returns the objects listed by
+// the calling warp.
+__device__ __forceinline__ unsigned scan_types(const dsr_dev_heap& H, uint32_t types, uint32_t* count) {
     __shared__ unsigned warp_n[8];
     __shared__ unsigned run_base;
     const dsr_u64 M = H.M;
@@ -234,7 +236,7 @@ __global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_he
                     warp_n[w] = total;
                     total += n;
                 }
-                run_base = total ? atomicAdd(H.R_count, total) : 0;
+                run_base = total ? atomicAdd(count, total) : 0;
             }
             __syncthreads();
             if (set) {
@@ -247,8 +249,12 @@ __global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_he
             __syncthreads();
         }
     }
-    objs = __reduce_add_sync(0xFFFFFFFFu, objs);
-    if (lane == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs);
+    return __reduce_add_sync(0xFFFFFFFFu, objs);
+}
+
+__global__ void __launch_bounds__(256) k_scan(const __grid_constant__ dsr_dev_heap H, uint32_t types) {
+    const unsigned objs = scan_types(H, types, H.R_count);
+    if (dsr_lane() == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs);
 }
 
 // The lists of a step (dsr_steps.cuh).
@@ -256,6 +262,13 @@ __global__ void __launch_bounds__(256) k_list(const __grid_constant__ dsr_dev_he
                                               unsigned mult_b) {
     __shared__ dsr_list_smem<256> sm;
     dsr_list<256>(H, ta, tb, mult_a, mult_b, dsr_begin_step(H.R_count), sm);
+}
+
+// The front list of a do-all over a type with subtypes (dsr_steps.cuh).
+__global__ void __launch_bounds__(256) k_list_tree(const __grid_constant__ dsr_dev_heap H, uint32_t types,
+                                                   unsigned mult) {
+    const unsigned objs = scan_types(H, types, H.R_count + dsr_begin_step(H.R_count));
+    if (dsr_lane() == 0 && objs) dsr_count(H.ctr, DSR_CTR_VISITS, (dsr_u64)objs * mult);
 }
 
 static void cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, cudaStream_t s) {
@@ -345,6 +358,10 @@ void dsr__launch_scan(const dsr_heap* h, int type, cudaStream_t s, bool exact) {
 
 void dsr__list_types(const dsr_heap* h, int type_a, int type_b, unsigned mult_a, unsigned mult_b, cudaStream_t s) {
     k_list<<<dsr__scan_grid(h, type_a), 256, 0, s>>>(h->dev, type_a, type_b, mult_a, mult_b);
+}
+
+void dsr__list_tree(const dsr_heap* h, int type, unsigned mult, cudaStream_t s) {
+    k_list_tree<<<dsr__scan_grid(h, type), 256, 0, s>>>(h->dev, h->dev.sub[type], mult);
 }
 
 int dsr__persistent_grid(const dsr_heap* h, const void* kernel, int threads) {

@@ -43,6 +43,14 @@
 //   kMarks: 1 if run's result (0 or 1) replaces the slot's bit of the list entry
 //   static void flush(H, const Inst&, const Acc&)        by a whole warp: event
 //     counts gathered in Acc go to memory
+//
+// Subtypes. A do-all over a type visits the objects of its subtypes as well
+// (dsr_heap_set_bases), whose blocks the two-type scan does not list, and one
+// of the two types may be a subtype of the other. The steps of a heap with
+// such types (dsr__has_subtypes) go do-all by do-all, as dsr_parallel_do would:
+// dsr__list_tree lists one type with its subtypes, and END follows where the
+// live set has changed. A kDefers method then finds no list of the type it
+// creates, or one with blocks of subtypes, which dsr_take gives back.
 #pragma once
 
 #include <type_traits>
@@ -654,5 +662,8 @@ int dsr__group_step(dsr_group* g, const dsr_phase& p1, const dsr_phase& p2, cons
 // Queue the listing of type A (front) and, unless -1, type B (back). mult:
 // visits counted per listed object.
 void dsr__list_types(const dsr_heap* h, int type_a, int type_b, unsigned mult_a, unsigned mult_b, cudaStream_t s);
+// The same for one type and its subtypes, at the front.
+void dsr__list_tree(const dsr_heap* h, int type, unsigned mult, cudaStream_t s);
+inline bool dsr__has_subtypes(const dsr_heap* h, int type) { return h->dev.sub[type] != (1u << type); }
 void dsr__group_list_types(const dsr_group* g, int type_a, int type_b, unsigned mult_a, unsigned mult_b,
                            cudaStream_t s);

@@ -404,7 +404,10 @@ extern "C" int dsr_sugarscape_step(dsr_sugarscape* g, int n_steps, void* stream)
         // list for A3 and A4. (All four count as visits of every agent.)
         SugarArgs& a = g->args;
         for (int k = 0; k < N_KEYS; ++k) a.key[k] = dsr_rand_key(a.p.seed, 8 + k, (dsr_u64)a.step);
-        dsr__list_types(g->heap, AGENT, -1, 4, 0, s);
+        if (dsr__has_subtypes(g->heap, AGENT))
+            dsr__list_tree(g->heap, AGENT, 4, s);
+        else
+            dsr__list_types(g->heap, AGENT, -1, 4, 0, s);
         int rc = dsr__step<DChoose>(g->heap, kAgents, kAgents, a, s);
         if (!rc) rc = dsr__step<DMove>(g->heap, kAgents, kAgents, a, s);
         if (!rc) rc = dsr__step<DReplaceClaim>(g->heap, kAgents, kAgents, a, s);

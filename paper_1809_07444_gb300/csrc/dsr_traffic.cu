@@ -141,9 +141,10 @@ constexpr dsr_phase kCars{CAR, 0};
 // occupancy, which nothing reads any more: the few CTAs that have sources
 // wait on their chains of accesses while the others write the grid.
 __global__ void __launch_bounds__(256, 5)
-    k_traffic_sources_step(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ TrafficArgs a) {
+    k_traffic_sources_step(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ dsr_phase sources,
+                           const __grid_constant__ TrafficArgs a) {
     __shared__ dsr_later_smem<256> later;
-    dsr_run_list<DSource, dsr_heap_space, 256>(dsr_heap_space{H}, dsr_phase{SOURCE, 1}, a, H.span_sh[SOURCE] - 5, false, &later);
+    dsr_run_list<DSource, dsr_heap_space, 256>(dsr_heap_space{H}, sources, a, H.span_sh[SOURCE] - 5, false, &later);
     uint4* w = reinterpret_cast<uint4*>(a.cur);
     const dsr_u64 n = ((dsr_u64)a.p.R * a.p.L + 255) / 256 * 16;
     for (dsr_u64 i = (dsr_u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (dsr_u64)gridDim.x * blockDim.x)
@@ -274,16 +275,21 @@ extern "C" int dsr_traffic_step(dsr_traffic* t, int n_steps, void* stream) {
         TrafficArgs a{t->grid[t->cur], t->grid[1 - t->cur], t->p, dsr_rand_key(t->p.seed, 5, t->step),
                       dsr_rand_key(t->p.seed, 6, t->step)};
         const bool open = !t->p.periodic;
-        dsr__list_types(t->heap, CAR, open ? SOURCE : -1, 1, 1, s);
-        int rc = open ? dsr__step<DCar>(t->heap, kCars, kCars, a, s)
-                      : dsr__step<DCar, dsr_no_method, true>(t->heap, kCars, kCars, a, s);
+        const bool trees = dsr__has_subtypes(t->heap, CAR) || dsr__has_subtypes(t->heap, SOURCE);
+        if (trees)
+            dsr__list_tree(t->heap, CAR, 1, s);
+        else
+            dsr__list_types(t->heap, CAR, open ? SOURCE : -1, 1, 1, s);
+        int rc = open && !trees ? dsr__step<DCar>(t->heap, kCars, kCars, a, s)
+                                : dsr__step<DCar, dsr_no_method, true>(t->heap, kCars, kCars, a, s);
         if (rc) return rc;
+        if (open && trees) dsr__list_tree(t->heap, SOURCE, 1, s);
         if (open) {
             static int per_sm = 0;
             if (!per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traffic_sources_step, 256, 0) !=
                                 cudaSuccess || per_sm < 1))
                 per_sm = 1;
-            k_traffic_sources_step<<<per_sm * t->heap->sm_count, 256, 0, s>>>(t->heap->dev, a);
+            k_traffic_sources_step<<<per_sm * t->heap->sm_count, 256, 0, s>>>(t->heap->dev, dsr_phase{SOURCE, trees ? 0 : 1}, a);
             rc = dsr__check_launch("k_traffic_sources_step");
             if (rc) return rc;
         } else {

@@ -401,6 +401,8 @@ struct NextStep {
 // does (a fish moves into cells that were empty at the start of the step), so
 // the two share a launch.
 constexpr dsr_phase kFish{FISH, 0}, kSharks{SHARK, 1};
+// The sharks' list of a heap with subtypes: one list at a time.
+constexpr dsr_phase kSharkTree{SHARK, 0};
 
 // Steps of a small torus in one launch of one cluster (dsr_steps.cuh).
 __global__ void __launch_bounds__(DSR_CLUSTER_THREADS, 1)
@@ -640,6 +642,8 @@ extern "C" int dsr_wator_attach(dsr_heap* heap, const dsr_wator_params* p, void*
     return DSR_OK;
 }
 
+static bool has_subtypes(const dsr_heap* h) { return dsr__has_subtypes(h, FISH) || dsr__has_subtypes(h, SHARK); }
+
 // The launches of one step on s; e: the step's kPhaseEvents events (null:
 // untimed), of which only the selected phase's two are recorded when sel >= 0.
 static int issue_step(dsr_wator* w, cudaStream_t s, const cudaEvent_t* e, int sel) {
@@ -655,9 +659,30 @@ static int issue_step(dsr_wator* w, cudaStream_t s, const cudaEvent_t* e, int se
     auto record = [&](int k) {
         if (E(k)) cudaEventRecordWithFlags(E(k), s, cudaEventRecordExternal);
     };
+    int rc = DSR_OK;
+    if (has_subtypes(h)) {
+        dsr__list_tree(h, FISH, 2, s);
+        record(1);
+        rc = dsr__step<DFishChoose<A>>(h, kFish, kFish, I, s);
+        record(2);
+        record(3);
+        if (!rc) rc = dsr__step<DFishMove<A>, dsr_no_method, true>(h, kFish, kFish, I, s);
+        record(4);
+        dsr__list_tree(h, SHARK, 1, s);
+        record(5);
+        if (!rc) rc = dsr__step<DSharkStarve<A>>(h, kSharkTree, kSharkTree, I, s);
+        record(6);
+        record(7);
+        if (!rc) rc = dsr__step<DSharkChoose<A>>(h, kSharkTree, kSharkTree, I, s);
+        record(8);
+        record(9);
+        if (!rc) rc = dsr__step<DSharkMove<A>, dsr_no_method, true, NextStep>(h, kSharkTree, kSharkTree, I, s);
+        record(10);
+        return rc;
+    }
     dsr__list_types(h, FISH, SHARK, 2, 1, s);
     record(1);
-    int rc = dsr__step<DFishChoose<A>>(h, kFish, kFish, I, s);
+    rc = dsr__step<DFishChoose<A>>(h, kFish, kFish, I, s);
     record(2);
     record(3);
     if (!e) {
@@ -770,7 +795,7 @@ extern "C" int dsr_wator_step(dsr_wator* w, int n_steps, void* stream) {
                            cs == cudaStreamCaptureStatusNone;
     // Small heaps: up to DSR_CLUSTER_STEPS steps a launch (kSmallBlocks).
     static const bool fits = dsr__cluster_fits((const void*)k_wator_steps);
-    if (w->ev.empty() && fits && dsr__small_heap(w->heap, kSmallBlocks)) {
+    if (w->ev.empty() && fits && dsr__small_heap(w->heap, kSmallBlocks) && !has_subtypes(w->heap)) {
         for (int i = 0; i < n_steps;) {
             int n = n_steps - i < DSR_CLUSTER_STEPS ? n_steps - i : DSR_CLUSTER_STEPS;
             void* args[] = {&w->heap->dev, &w->inst, &n};
