@@ -284,8 +284,9 @@ constexpr dsr_u64 kSmallBlocks = 768;
 extern "C" int dsr_gol_step(dsr_gol* g, int n_gen, void* stream) {
     if (!g || n_gen < 0) return DSR_E_INVALID;
     cudaStream_t s = dsr__stream(stream);
-    static const bool fits = dsr__cluster_fits((const void*)k_gol_steps);
-    if (fits && dsr__small_heap(g->heap, kSmallBlocks) && !has_subtypes(g->heap)) {
+    static dsr_per_device fits;
+    if (dsr__small_heap(g->heap, kSmallBlocks) && !has_subtypes(g->heap) &&
+        dsr__cluster_fits(g->heap, (const void*)k_gol_steps, &fits)) {
         for (int i = 0; i < n_gen;) {
             int n = n_gen - i < DSR_CLUSTER_STEPS ? n_gen - i : DSR_CLUSTER_STEPS;
             void* args[] = {&g->heap->dev, &g->args, &n};

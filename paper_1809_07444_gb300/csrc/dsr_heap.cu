@@ -283,15 +283,18 @@ static void cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, c
     cfg->numAttrs = 1;
 }
 
-bool dsr__cluster_fits(const void* kernel) {
-    int n = 0;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
-    cluster_config(&cfg, &attr, nullptr);
-    const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                    cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
-    cudaGetLastError();
-    return ok;
+bool dsr__cluster_fits(const dsr_heap* h, const void* kernel, dsr_per_device* known) {
+    return known->get(h->device, [&] {
+        int n = 0;
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        cluster_config(&cfg, &attr, nullptr);
+        const bool ok =
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+        cudaGetLastError();
+        return ok;
+    });
 }
 
 int dsr__launch_cluster(const void* kernel, void** args, cudaStream_t s) {

@@ -57,6 +57,7 @@
 
 #include "dsr_bulk.cuh"
 #include "dsr_group.cuh"
+#include "dsr_per_device.h"
 
 // Words from R_count that the lists use. Their lengths live in two sets of
 // (front, back) words, which steps use in turn: the scan of a step adds to one
@@ -554,8 +555,9 @@ __device__ __forceinline__ void dsr_cluster_barrier() {
         "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Whether `kernel` can run as one cluster of DSR_CLUSTER CTAs on this device.
-bool dsr__cluster_fits(const void* kernel);
+// Whether `kernel` can run as one cluster of DSR_CLUSTER CTAs on the heap's
+// device, which its first use there also allows it to. known: the kernel's own.
+bool dsr__cluster_fits(const dsr_heap* h, const void* kernel, dsr_per_device* known);
 // Queue it with the given arguments.
 int dsr__launch_cluster(const void* kernel, void** args, cudaStream_t s);
 // Small heaps of the default tuning (a caller that sets threads or CTAs gets

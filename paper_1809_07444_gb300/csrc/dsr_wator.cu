@@ -794,8 +794,9 @@ extern "C" int dsr_wator_step(dsr_wator* w, int n_steps, void* stream) {
     const bool use_graph = !w->graphs_off && cudaStreamIsCapturing(s, &cs) == cudaSuccess &&
                            cs == cudaStreamCaptureStatusNone;
     // Small heaps: up to DSR_CLUSTER_STEPS steps a launch (kSmallBlocks).
-    static const bool fits = dsr__cluster_fits((const void*)k_wator_steps);
-    if (w->ev.empty() && fits && dsr__small_heap(w->heap, kSmallBlocks) && !has_subtypes(w->heap)) {
+    static dsr_per_device fits;
+    if (w->ev.empty() && dsr__small_heap(w->heap, kSmallBlocks) && !has_subtypes(w->heap) &&
+        dsr__cluster_fits(w->heap, (const void*)k_wator_steps, &fits)) {
         for (int i = 0; i < n_steps;) {
             int n = n_steps - i < DSR_CLUSTER_STEPS ? n_steps - i : DSR_CLUSTER_STEPS;
             void* args[] = {&w->heap->dev, &w->inst, &n};
