@@ -74,6 +74,7 @@ struct NbWs {
     uint32_t* n_live;  // bodies in this step
     uint32_t* npairs;  // near-field pairs of this step (each counted from both bodies)
     uint32_t* work;    // next work item of the symmetric force kernel (zeroed by the gather)
+    uint32_t* wide;    // not 0: some body's coordinate is beyond kNarrowReach
     // per sorted position p (padded to a multiple of ROW with empty entries)
     float4* pos;       // high words x, y, z, m before the update (m = 0: empty)
     D4* pd;            // full x, y, z, m before the update
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(1024) k_cell_scan(const __grid_constant__ NbWs
         if (!post) {
             *ws.n_live = before + v;
             *ws.npairs = 0;
+            if (ws.wide) *ws.wide = 0;
         }
     }
 }
@@ -285,6 +287,12 @@ __global__ void k_cell_order(const __grid_constant__ dsr_dev_heap H, const __gri
         }
     }
 }
+
+// inv_cubed (below) is a normal FP32 number for r^2 from kNarrowMin (1.5 times
+// the r^2 whose r^-3 is 2^128) to half the one whose r^-3 is 2^-126, which two
+// bodies with no coordinate beyond kNarrowReach stay below. Beyond, r^-3
+// overflows or loses its digits where a mass times it need not.
+constexpr float kNarrowMin = 3.1e-26f, kNarrowReach = 8.9e11f;
 
 // Sorted positions: one CTA per tile of 256. Each position gets its body's
 // state (or an empty entry past the live bodies), each tile the bounding box
@@ -331,6 +339,10 @@ __global__ void __launch_bounds__(TILE) k_gather(const __grid_constant__ dsr_dev
                 for (int k = 0; k < 6; ++k) b[k] = k < 3 ? fminf(b[k], red[k][w]) : fmaxf(b[k], red[k][w]);
             ws.tbox[2 * t] = make_float4(b[0], b[1], b[2], 0.f);
             ws.tbox[2 * t + 1] = make_float4(b[3], b[4], b[5], 0.f);
+            float reach = 0.f;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) reach = fmaxf(reach, fabsf(b[k]));
+            if (ws.wide && b[0] <= b[3] && !(reach <= kNarrowReach)) *ws.wide = 1;
         }
     }
 }
@@ -641,8 +653,11 @@ __host__ __device__ inline SymShape sym_shape(uint32_t n, uint32_t threads, uint
     return q;
 }
 
-// The two forms of the arithmetic.
+// The forms of the arithmetic, and how a step whose FP32 pairs go beyond
+// inv_cubed's range differs: not at all (FP64), by another kernel, by a branch.
+enum { SYM_NARROW, SYM_KERNEL, SYM_BRANCH };
 struct SymF32 {
+    static constexpr int WIDE = SYM_KERNEL;
     typedef float Real;
     typedef float4 Vec;
     static constexpr int THREADS = 128, RB = 8, JF = 4;
@@ -652,8 +667,10 @@ struct SymF32 {
 };
 struct SymF32Small : SymF32 {  // few bodies: more and smaller items
     static constexpr int THREADS = 128, RB = 2, JF = 16, CTAS = 5;
+    static constexpr int WIDE = SYM_BRANCH;
 };
 struct SymF64 {
+    static constexpr int WIDE = SYM_NARROW;
     typedef double Real;
     typedef D4 Vec;
     // the FP64 units of an SM are busy with eight warps; more CTAs would only
@@ -672,6 +689,12 @@ __host__ __device__ constexpr uint32_t sym_slots(uint32_t n) {
 __device__ __forceinline__ float inv_cubed(float r2) {
     const float inv = rsqrt_normal(r2);
     return inv * inv * inv;
+}
+// The term's factor with the mass multiplied in first, as k_force_part does:
+// two operations more an unordered pair, in the range of the result.
+__device__ __forceinline__ float mass_inv_cubed(float m, float r2) {
+    const float inv = rsqrt_normal(r2);
+    return m * inv * inv * inv;
 }
 // r^-3 in FP64, r^2 >= FLT_MIN. y: the PTX approximate reciprocal square
 // root, y^2 r^2 = 1 - h. Then r^-3 = y^3 (1 - h)^(-3/2), by the binomial
@@ -696,7 +719,7 @@ __device__ __forceinline__ D4 sym_vec(double x, double y, double z) { return d4(
 
 // One row against the block of 32 bodies at sp, every unordered pair.
 // sums: the bodies' sums in shared memory, `stride` apart.
-template <class F, bool EXCLUDE, class Real, class Vec>
+template <class F, bool EXCLUDE, bool WIDE, class Real, class Vec>
 __device__ __forceinline__ void sym_block(const Vec* sp, Real* sums, int stride, const Real* px, const Real* py,
                                           const Real* pz, const Real* pm, Real eps2, Real rn2, Real* tx, Real* ty,
                                           Real* tz) {
@@ -715,8 +738,13 @@ __device__ __forceinline__ void sym_block(const Vec* sp, Real* sums, int stride,
                 const Real dx = pj.x - px[k], dy = pj.y - py[k], dz = pj.z - pz[k];
                 Real r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
                 if (EXCLUDE) r2 = r2 < rn2 ? (Real)f_inf() : r2;
-                const Real w = inv_cubed(r2);
-                const Real wj = pj.w * w, wi = pm[k] * w;
+                Real wj, wi;
+                if constexpr (WIDE) {
+                    wj = mass_inv_cubed(pj.w, r2), wi = mass_inv_cubed(pm[k], r2);
+                } else {
+                    const Real w = inv_cubed(r2);
+                    wj = pj.w * w, wi = pm[k] * w;
+                }
                 tx[k] = fma(wj, dx, tx[k]);
                 ty[k] = fma(wj, dy, ty[k]);
                 tz[k] = fma(wj, dz, tz[k]);
@@ -749,7 +777,7 @@ __device__ __forceinline__ void sym_block(const Vec* sp, Real* sums, int stride,
 }
 
 // One row against 32 bodies at sp, every ordered pair of the row's bodies.
-template <class F, bool EXCLUDE, class Real, class Vec>
+template <class F, bool EXCLUDE, bool WIDE, class Real, class Vec>
 __device__ __forceinline__ void row_block(const Vec* sp, const Real* px, const Real* py, const Real* pz, Real eps2,
                                           Real rn2, Real* tx, Real* ty, Real* tz) {
 #pragma unroll 4
@@ -760,7 +788,11 @@ __device__ __forceinline__ void row_block(const Vec* sp, const Real* px, const R
             const Real dx = pj.x - px[k], dy = pj.y - py[k], dz = pj.z - pz[k];
             Real r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
             if (EXCLUDE) r2 = r2 < rn2 ? (Real)f_inf() : r2;
-            const Real w = pj.w * inv_cubed(r2);
+            Real w;
+            if constexpr (WIDE)
+                w = mass_inv_cubed(pj.w, r2);
+            else
+                w = pj.w * inv_cubed(r2);
             tx[k] = fma(w, dx, tx[k]);
             ty[k] = fma(w, dy, ty[k]);
             tz[k] = fma(w, dz, tz[k]);
@@ -768,13 +800,23 @@ __device__ __forceinline__ void row_block(const Vec* sp, const Real* px, const R
     }
 }
 
-template <class F>
+// WIDE: the terms in the range of the result. Few programs need that, and the
+// narrow loop must not pay for it: a step runs wide if a body is far out, or
+// by its softening. With both in one loop two steps of 65,536 bodies took 3455
+// us instead of 3340, so SymF32 has a kernel for each, of which one returns at
+// once (3341); five steps of 4097 bodies took 592 us instead of 591 so, and
+// 616 with a second launch.
+template <class F, bool WIDE>
 __global__ void __launch_bounds__(F::THREADS, F::CTAS) k_force_sym(const __grid_constant__ NbArgs a) {
+    bool wide = false;
+    if constexpr (F::WIDE != SYM_NARROW) wide = *a.ws.wide || (float)(a.p.eps * a.p.eps) < kNarrowMin;
+    if (F::WIDE == SYM_KERNEL && wide != WIDE) return;
+    constexpr bool kBranch = F::WIDE == SYM_BRANCH;
+    extern __shared__ __align__(32) unsigned char dynamic[];
     typedef typename F::Real Real;
     typedef typename F::Vec Vec;
     constexpr int THREADS = F::THREADS, RB_ = F::RB, WARPS = THREADS / 32, ROW_ = THREADS * RB_;
     constexpr bool kF32 = F::SUMS == 6;
-    extern __shared__ __align__(32) unsigned char dynamic[];
     Vec* sp = reinterpret_cast<Vec*>(dynamic);              // [THREADS]
     Real* sums = reinterpret_cast<Real*>(sp + THREADS);     // [TR][SUMS][THREADS]
     __shared__ uint32_t next;
@@ -831,15 +873,19 @@ __global__ void __launch_bounds__(F::THREADS, F::CTAS) k_force_sym(const __grid_
 #pragma unroll
                     for (int k = 0; k < RB_; ++k) tx[k] = ty[k] = tz[k] = 0;
                     if (own) {
-                        if (kF32 && near)
-                            row_block<F, true>(sp + jb, px, py, pz, eps2, rn2, tx, ty, tz);
+                        if (kBranch && wide)
+                            row_block<F, true, kBranch>(sp + jb, px, py, pz, eps2, rn2, tx, ty, tz);
+                        else if (kF32 && near)
+                            row_block<F, true, WIDE>(sp + jb, px, py, pz, eps2, rn2, tx, ty, tz);
                         else
-                            row_block<F, false>(sp + jb, px, py, pz, eps2, rn2, tx, ty, tz);
+                            row_block<F, false, WIDE>(sp + jb, px, py, pz, eps2, rn2, tx, ty, tz);
                     } else {
-                        if (kF32 && near)
-                            sym_block<F, true>(sp + jb, m + jb, THREADS, px, py, pz, pm, eps2, rn2, tx, ty, tz);
+                        if (kBranch && wide)
+                            sym_block<F, true, kBranch>(sp + jb, m + jb, THREADS, px, py, pz, pm, eps2, rn2, tx, ty, tz);
+                        else if (kF32 && near)
+                            sym_block<F, true, WIDE>(sp + jb, m + jb, THREADS, px, py, pz, pm, eps2, rn2, tx, ty, tz);
                         else
-                            sym_block<F, false>(sp + jb, m + jb, THREADS, px, py, pz, pm, eps2, rn2, tx, ty, tz);
+                            sym_block<F, false, WIDE>(sp + jb, m + jb, THREADS, px, py, pz, pm, eps2, rn2, tx, ty, tz);
                         __syncthreads();  // the next warp adds to these bodies' sums
                     }
 #pragma unroll
@@ -1325,9 +1371,11 @@ SymLaunch sym_launch(const dsr_heap* h, uint64_t n_bodies, uint64_t P) {
     }
     SymLaunch l;
     l.smem = smem(tr);
-    cudaFuncSetAttribute(k_force_sym<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(F::MAX_TR));
+    cudaFuncSetAttribute(k_force_sym<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(F::MAX_TR));
+    if constexpr (F::WIDE == SYM_KERNEL)
+        cudaFuncSetAttribute(k_force_sym<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(F::MAX_TR));
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_force_sym<F>, F::THREADS, l.smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_force_sym<F, false>, F::THREADS, l.smem) != cudaSuccess ||
         occ < 1)
         occ = 1;
     if (occ > F::CTAS) occ = F::CTAS;
@@ -1441,6 +1489,7 @@ NbWs carve(void* base, uint64_t S, uint64_t log_cap, SplitGrids grid) {
     w.n_live = reinterpret_cast<uint32_t*>(p + 16);
     w.npairs = reinterpret_cast<uint32_t*>(p + 20);
     w.work = reinterpret_cast<uint32_t*>(p + 24);
+    w.wide = reinterpret_cast<uint32_t*>(p + 28);
     p += 256;
     w.part = reinterpret_cast<float4*>(p);
     w.part64 = reinterpret_cast<D4*>(p);
@@ -1461,7 +1510,8 @@ void launch_sort(dsr_heap* h, const NbArgs& a, cudaStream_t s) {
 
 template <class F>
 FarShape launch_sym(const NbArgs& a, const SymLaunch& l, cudaStream_t s) {
-    k_force_sym<F><<<l.grid, F::THREADS, l.smem, s>>>(a);
+    k_force_sym<F, false><<<l.grid, F::THREADS, l.smem, s>>>(a);
+    if constexpr (F::WIDE == SYM_KERNEL) k_force_sym<F, true><<<l.grid, F::THREADS, l.smem, s>>>(a);
     return FarShape{0, (uint32_t)F::THREADS, (uint32_t)F::RB, F::SLOTS, F::SLOTS_FEW, F::MAX_TR};
 }
 
@@ -1682,7 +1732,7 @@ extern "C" int dsr_nbody_step_noalloc(dsr_heap* heap, const dsr_nbody_params* p,
     a.ws.perm2 = sc->perm2;
     a.ws.n_live = &sc->n_live;
     a.ws.npairs = &sc->npairs;
-    a.ws.work = nullptr;  // the unsplit force kernels
+    a.ws.work = a.ws.wide = nullptr;  // the unsplit force kernels
     a.ws.pos = sc->pos;
     a.ws.pd = sc->pd;
     a.ws.id = sc->id;
