@@ -131,7 +131,9 @@ struct DBirth : GolMethod<A> {
     }
 };
 // One scan lists both types. A birth and a death never meet: a cell that
-// dies has not 3 alive neighbours, and new Alive objects are in no list.
+// dies has not 3 alive neighbours, and new Alive objects are in no list. They
+// share a launch where memory never runs short while no death has given its
+// slot back (deaths_may_wait); else the deaths come first.
 constexpr dsr_phase kCells{CELL, 0}, kAlive{ALIVE, 1};
 // A list of its own for each do-all, of a type and its subtypes.
 constexpr dsr_phase kAliveTree{ALIVE, 0};
@@ -141,7 +143,7 @@ constexpr dsr_phase kAliveTree{ALIVE, 0};
 // all generations; the Alive objects are listed while the cells count, which
 // leaves them alone: two barriers a generation.
 __global__ void __launch_bounds__(DSR_CLUSTER_THREADS, 1)
-    k_gol_steps(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ GolArgs a, int n) {
+    k_gol_steps(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ GolArgs a, int n, int apart) {
     constexpr int T = DSR_CLUSTER_THREADS;
     typedef GolArgs A;
     __shared__ dsr_later_smem<T> later;
@@ -166,8 +168,12 @@ __global__ void __launch_bounds__(DSR_CLUSTER_THREADS, 1)
         dsr_cluster_barrier();
         if (threadIdx.x == 0) len[1] = *(volatile uint32_t*)(H.R_count + set + 1);
         __syncthreads();
+        if (apart) {
+            dsr_run_list<DDie<A>, dsr_heap_space, T>(S, alive, a, ha, false, nullptr);
+            dsr_cluster_barrier();
+        }
         dsr_run_list<DBirth<A>, dsr_heap_space, T>(S, cells, a, hc, false, &later);
-        dsr_run_list<DDie<A>, dsr_heap_space, T>(S, alive, a, ha, true, nullptr);
+        if (!apart) dsr_run_list<DDie<A>, dsr_heap_space, T>(S, alive, a, ha, true, nullptr);
         dsr_cluster_barrier();
     }
     dsr_clear_sets(H.R_count, first);
@@ -201,6 +207,18 @@ int launch_init(const dsr_heap* heap, int W, int H, const void* alive0_dev, void
     k_gol_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
         heap->dev, static_cast<const uint8_t*>(alive0_dev), static_cast<dsr_ref*>(cell_ref_dev), W, H, rows);
     return dsr__check_launch("k_gol_init");
+}
+
+// Whether the births of a generation find room before its deaths have given
+// theirs back, whatever the state of the board: a cell holds an Alive object or
+// gets one, never both, so there are at most as many as cells. Of the cells'
+// blocks twice as many as full ones are reckoned, as a chunk's objects beyond
+// its full blocks may lie in blocks of their own (dsr_bulk.cuh). Other types
+// may hold any number of blocks. The default heaps have more than that.
+bool deaths_may_wait(const dsr_heap* h, int W, int Hh) {
+    const dsr_layout& L = h->layout;
+    const dsr_u64 n = (dsr_u64)W * Hh, cc = L.capacity[CELL], ca = L.capacity[ALIVE];
+    return L.n_types == 2 && L.n_blocks >= 2 * ((n + cc - 1) / cc) + (n + ca - 1) / ca;
 }
 
 const int kCellFields[3] = {4, 4, 4};
@@ -269,7 +287,12 @@ static int issue_generation(dsr_gol* g, cudaStream_t s) {
     }
     dsr__list_types(g->heap, CELL, ALIVE, 2, 1, s);
     int rc = dsr__step<DCount<A>>(g->heap, kCells, kCells, g->args, s);
-    if (!rc) rc = dsr__step<DBirth<A>, DDie<A>, true>(g->heap, kCells, kAlive, g->args, s);
+    if (deaths_may_wait(g->heap, g->args.W, g->args.H)) {
+        if (!rc) rc = dsr__step<DBirth<A>, DDie<A>, true>(g->heap, kCells, kAlive, g->args, s);
+        return rc;
+    }
+    if (!rc) rc = dsr__step<DDie<A>>(g->heap, kAlive, kAlive, g->args, s);
+    if (!rc) rc = dsr__step<DBirth<A>, dsr_no_method, true>(g->heap, kCells, kCells, g->args, s);
     return rc;
 }
 
@@ -287,9 +310,10 @@ extern "C" int dsr_gol_step(dsr_gol* g, int n_gen, void* stream) {
     static dsr_per_device fits;
     if (dsr__small_heap(g->heap, kSmallBlocks) && !has_subtypes(g->heap) &&
         dsr__cluster_fits(g->heap, (const void*)k_gol_steps, &fits)) {
+        int apart = deaths_may_wait(g->heap, g->args.W, g->args.H) ? 0 : 1;
         for (int i = 0; i < n_gen;) {
             int n = n_gen - i < DSR_CLUSTER_STEPS ? n_gen - i : DSR_CLUSTER_STEPS;
-            void* args[] = {&g->heap->dev, &g->args, &n};
+            void* args[] = {&g->heap->dev, &g->args, &n, &apart};
             const int rc = dsr__launch_cluster((const void*)k_gol_steps, args, s);
             if (rc) return rc;
             i += n;
@@ -486,7 +510,16 @@ static int ensure_gol_graph(dsr_gol_batch* b) {
     typedef GolBatchArgs A;
     dsr__group_list_types(b->group, CELL, ALIVE, 2, 1, b->capture);
     int rc = dsr__group_step<DCount<A>>(b->group, kCells, kCells, a, b->capture);
-    if (!rc) rc = dsr__group_step<DBirth<A>, DDie<A>, true>(b->group, kCells, kAlive, a, b->capture);
+    bool together = true;
+    for (size_t i = 0; i < b->table_h.size(); ++i)
+        if (b->table_h[i].cell_ref)
+            together = together && deaths_may_wait(b->group->heaps[i], b->table_h[i].W, b->table_h[i].H);
+    if (together) {
+        if (!rc) rc = dsr__group_step<DBirth<A>, DDie<A>, true>(b->group, kCells, kAlive, a, b->capture);
+    } else {
+        if (!rc) rc = dsr__group_step<DDie<A>>(b->group, kAlive, kAlive, a, b->capture);
+        if (!rc) rc = dsr__group_step<DBirth<A>, dsr_no_method, true>(b->group, kCells, kCells, a, b->capture);
+    }
     e = cudaStreamEndCapture(b->capture, &graph);
     if (rc) {
         if (graph) cudaGraphDestroy(graph);
