@@ -251,14 +251,17 @@ extern "C" int dsr_traffic_create(dsr_heap* heap, const dsr_traffic_params* p, c
         return DSR_E_CUDA;
     }
     const dsr_u64 n = (dsr_u64)p->R * p->L;
-    const int rows = dsr__bulk_rows<1>(n, heap->sm_count);
-    k_traffic_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
-        heap->dev, static_cast<const int8_t*>(v0_dev), t->grid[0], *p, rows);
+    // the sources first: their few blocks are then taken before the cars', which
+    // fill whatever is left (after the cars a heap with few blocks to spare,
+    // all of them partly filled with cars, had none left for the sources)
     if (!p->periodic) {
         const int srows = dsr__bulk_rows<1>((dsr_u64)p->R, heap->sm_count);
         k_traffic_sources<<<dsr__bulk_grid((dsr_u64)p->R, srows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
             heap->dev, p->R, srows);
     }
+    const int rows = dsr__bulk_rows<1>(n, heap->sm_count);
+    k_traffic_init<<<dsr__bulk_grid(n, rows, heap->sm_count), DSR_BULK_THREADS, 0, s>>>(
+        heap->dev, static_cast<const int8_t*>(v0_dev), t->grid[0], *p, rows);
     int rc = dsr__check_launch("k_traffic_init");
     if (rc) {
         delete t;

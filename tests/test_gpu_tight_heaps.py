@@ -42,3 +42,24 @@ def test_life_with_room_for_the_births_only_after_the_deaths(tuning, batch):
         assert heap.stats()["error_flags"] == 0
         assert hashes() == o.hash()
     check_invariants(heap, [W * H, o.alive_count()])
+
+
+def test_traffic_sources_find_room_beside_the_cars():
+    # 1838 cars in 29 blocks and 100 sources in two at least: 34 blocks, of
+    # which partly filled blocks of cars may take three more
+    from paper_1809_07444_gb300 import workloads as WL
+    from paper_1809_07444_gb300.apps import TRAFFIC_TYPES, Traffic
+
+    R, L = 100, 90
+    v0 = WL.traffic_initial(R, L, 5, density=0.2, vmax=5)
+    assert (v0 >= 0).sum() == 1838
+    for _ in range(5):
+        g, o = (f(R, L, v0, 9, **kw) for f, kw in (
+            (Traffic, {"heap_bytes": heap_bytes_for_blocks(TRAFFIC_TYPES, 34)}), (O.Traffic, {})))
+        for n in (0, 20):
+            g.step(n)
+            if n:
+                o.step(n)
+            assert g.heap.stats()["error_flags"] == 0
+            for a, b in zip(g.dump(), o.dump()):
+                assert np.array_equal(a, b)
