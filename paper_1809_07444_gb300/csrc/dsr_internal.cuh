@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 
@@ -46,6 +47,21 @@ int dsr__scan_grid(const dsr_heap* h, int type);
 bool dsr__vec4_ok(const dsr_heap* h, int type);
 // exact: list the blocks of `type` only, not those of its subtypes.
 void dsr__launch_scan(const dsr_heap* h, int type, cudaStream_t s, bool exact = false);
+
+// The grid of a kernel that runs with the heap's tuning: dsr__persistent_grid,
+// looked up once per CTA size unless the tuning fixes the CTAs per SM. cache:
+// the kernel's own (several threads may fill it, each with the same value).
+typedef std::atomic<int> dsr_grid_cache[17];
+inline int dsr__tuned_grid(const dsr_heap* h, const void* kernel, dsr_grid_cache& cache) {
+    const int threads = h->tune.threads;
+    if (h->tune.ctas_per_sm > 0) return dsr__persistent_grid(h, kernel, threads);
+    int grid = cache[threads / 64].load(std::memory_order_relaxed);
+    if (!grid) {
+        grid = dsr__persistent_grid(h, kernel, threads);
+        cache[threads / 64].store(grid, std::memory_order_relaxed);
+    }
+    return grid;
+}
 
 // Run a do-all: scan + compaction of allocated[type] into R, then the method
 // kernel over the listed blocks.

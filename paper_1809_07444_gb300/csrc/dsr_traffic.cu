@@ -140,16 +140,31 @@ constexpr dsr_phase kCars{CAR, 0};
 // The Source do-all of an open road's step, with the clearing of the old
 // occupancy, which nothing reads any more: the few CTAs that have sources
 // wait on their chains of accesses while the others write the grid.
-__global__ void __launch_bounds__(256, 5)
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == 256 ? 5 : 1)
     k_traffic_sources_step(const __grid_constant__ dsr_dev_heap H, const __grid_constant__ dsr_phase sources,
                            const __grid_constant__ TrafficArgs a) {
-    __shared__ dsr_later_smem<256> later;
-    dsr_run_list<DSource, dsr_heap_space, 256>(dsr_heap_space{H}, sources, a, H.span_sh[SOURCE] - 5, false, &later);
+    __shared__ dsr_later_smem<MAXT> later;
+    dsr_run_list<DSource, dsr_heap_space, MAXT>(dsr_heap_space{H}, sources, a, H.span_sh[SOURCE] - 5, false, &later);
     uint4* w = reinterpret_cast<uint4*>(a.cur);
     const dsr_u64 n = ((dsr_u64)a.p.R * a.p.L + 255) / 256 * 16;
     for (dsr_u64 i = (dsr_u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (dsr_u64)gridDim.x * blockDim.x)
         w[i] = make_uint4(0, 0, 0, 0);
     if (blockIdx.x == 0 && threadIdx.x == 0) dsr_end_step(H.R_count);
+}
+
+// With the heap's tuning, as the do-alls.
+int launch_sources(const dsr_heap* h, const dsr_phase& sources, const TrafficArgs& a, cudaStream_t s) {
+    static dsr_grid_cache cache;
+    const int threads = h->tune.threads;
+    const bool small = threads <= 256;
+    const int grid = dsr__tuned_grid(
+        h, small ? (const void*)k_traffic_sources_step<256> : (const void*)k_traffic_sources_step<1024>, cache);
+    if (small)
+        k_traffic_sources_step<256><<<grid, threads, 0, s>>>(h->dev, sources, a);
+    else
+        k_traffic_sources_step<1024><<<grid, threads, 0, s>>>(h->dev, sources, a);
+    return dsr__check_launch("k_traffic_sources_step");
 }
 
 // A Car for every cell where v0 >= 0.
@@ -288,12 +303,7 @@ extern "C" int dsr_traffic_step(dsr_traffic* t, int n_steps, void* stream) {
         if (rc) return rc;
         if (open && trees) dsr__list_tree(t->heap, SOURCE, 1, s);
         if (open) {
-            static int per_sm = 0;
-            if (!per_sm && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_traffic_sources_step, 256, 0) !=
-                                cudaSuccess || per_sm < 1))
-                per_sm = 1;
-            k_traffic_sources_step<<<per_sm * t->heap->sm_count, 256, 0, s>>>(t->heap->dev, dsr_phase{SOURCE, trees ? 0 : 1}, a);
-            rc = dsr__check_launch("k_traffic_sources_step");
+            rc = launch_sources(t->heap, dsr_phase{SOURCE, trees ? 0 : 1}, a, s);
             if (rc) return rc;
         } else {
             cudaError_t e = cudaMemsetAsync(t->grid[t->cur], 0, grid_bytes(t->p), s);  // the next step's `next`
