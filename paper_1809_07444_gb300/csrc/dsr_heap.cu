@@ -742,22 +742,22 @@ struct MClone {
 // 32 items of 32 slots (one per warp and item queues up on the counter:
 // 6.7 M cars 160 -> 61 us).
 constexpr int DUMP_ITEMS = 4;   // items of a warp at a time (fewer in a short list)
-constexpr int DUMP_ROW = 2 * DSR_MAX_FIELDS + 2;
-__global__ void __launch_bounds__(256) k_dump(const __grid_constant__ dsr_dev_heap H, int T, uint32_t* out,
-                                              dsr_u64* count, dsr_u64 cap, int row) {
-    __shared__ uint32_t stage[8][32 * DUMP_ROW];
-    __shared__ uint32_t warp_n[8];
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT) k_dump(const __grid_constant__ dsr_dev_heap H, int T, uint32_t* out,
+                                               dsr_u64* count, dsr_u64 cap, int row) {
+    extern __shared__ uint32_t stage[];  // [warps][32 * row]
+    __shared__ uint32_t warp_n[MAXT / 32];
     __shared__ dsr_u64 cta_base;
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const unsigned hsh = H.span_sh[T] - 5;
     const dsr_u64 items = (dsr_u64)(*(volatile uint32_t*)H.R_count) << hsh;
     const uint32_t nf = H.n_fields[T];
     bool words = true;  // every field has 4 bytes
     for (uint32_t f = 0; f < nf; ++f) words = words && H.fsize[T][f] == 4;
-    const dsr_u64 share = items / ((dsr_u64)gridDim.x * 8);
+    const dsr_u64 share = items / ((dsr_u64)gridDim.x * warps);
     const unsigned per = share < 1 ? 1u : (share < DUMP_ITEMS ? (unsigned)share : (unsigned)DUMP_ITEMS);
-    uint32_t* mine = stage[warp];
-    for (dsr_u64 base = (dsr_u64)blockIdx.x * 8 * per; base < items; base += (dsr_u64)gridDim.x * 8 * per) {
+    uint32_t* mine = stage + warp * 32 * row;
+    for (dsr_u64 base = (dsr_u64)blockIdx.x * warps * per; base < items; base += (dsr_u64)gridDim.x * warps * per) {
         // lane k < per holds the warp's k-th item
         const dsr_u64 item = base + warp * per + lane;
         uint32_t bid = 0, live = 0;
@@ -770,7 +770,7 @@ __global__ void __launch_bounds__(256) k_dump(const __grid_constant__ dsr_dev_he
         __syncthreads();
         if (threadIdx.x == 0) {
             uint32_t total = 0;
-            for (int w = 0; w < 8; ++w) {
+            for (unsigned w = 0; w < warps; ++w) {
                 const uint32_t k = warp_n[w];
                 warp_n[w] = total;
                 total += k;
@@ -867,11 +867,21 @@ extern "C" int dsr_heap_dump(dsr_heap* h, int type, void* out_dev, uint64_t cap,
         return DSR_E_CUDA;
     }
     dsr__launch_scan(h, type, s, true);
-    const dsr_u64 most = (h->dev.M * 2 + 8 * DUMP_ITEMS - 1) / (8 * DUMP_ITEMS);
-    const dsr_u64 grid = (dsr_u64)h->sm_count * 5;
-    k_dump<<<(unsigned)(grid < most ? grid : most), 256, 0, s>>>(h->dev, type, static_cast<uint32_t*>(out_dev),
-                                                                 static_cast<dsr_u64*>(count_dev), cap,
-                                                                 dsr_row_words(h, type));
+    // the heap's threads and CTAs per SM; by default 5 CTAs of 256 threads
+    const int threads = h->tune.threads, row = dsr_row_words(h, type);
+    const dsr_u64 items = (dsr_u64)(threads / 32) * DUMP_ITEMS, most = (h->dev.M * 2 + items - 1) / items;
+    dsr_u64 grid = (dsr_u64)h->sm_count * (h->tune.ctas_per_sm > 0 ? h->tune.ctas_per_sm : threads > 256 ? 1 : 5);
+    if (grid > most) grid = most;
+    const size_t smem = (size_t)threads * row * 4;  // up to 136 KB
+    auto run = [&](auto* kernel) {
+        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        kernel<<<(unsigned)grid, threads, smem, s>>>(h->dev, type, static_cast<uint32_t*>(out_dev),
+                                                     static_cast<dsr_u64*>(count_dev), cap, row);
+    };
+    if (threads <= 256)
+        run(k_dump<256>);
+    else
+        run(k_dump<1024>);
     return dsr__check_launch("k_dump");
 }
 
