@@ -276,9 +276,9 @@ __device__ __forceinline__ void dsr_create_pending(const Space& S, const typenam
             if (left && (own_blocks >= DSR_OPEN_SHARE || 2 * left >= cap)) {
                 const dsr_grab g = dsr_init_block(H, T, (int)left, hint ^ 0x5bd1e995u);
                 if (!g.status) {
-                    sm.open = g.bid << 6;  // its lowest slots
-                    sm.n_open = left;
-                    dsr_count(H.ctr, DSR_CTR_ALLOCS, left);
+                    sm.open = g.bid << 6;  // its lowest slots: `left`, or all of a block with fewer
+                    sm.n_open = (uint32_t)__popcll(g.bits);
+                    dsr_count(H.ctr, DSR_CTR_ALLOCS, sm.n_open);
                 }
             }
         }
