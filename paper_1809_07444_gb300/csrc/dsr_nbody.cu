@@ -699,7 +699,7 @@ __device__ __forceinline__ float mass_inv_cubed(float m, float r2) {
 // r^-3 in FP64, r^2 >= FLT_MIN. y: the PTX approximate reciprocal square
 // root, y^2 r^2 = 1 - h. Then r^-3 = y^3 (1 - h)^(-3/2), by the binomial
 // series 1 + 3/2 h + 15/8 h^2 + 35/16 h^3: what follows is 315/128 h^4, below
-// 2^-60 for any |h| < 2^-15.
+// 2^-58 for any |h| < 2^-15.
 __device__ __forceinline__ double inv_cubed(double r2) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
