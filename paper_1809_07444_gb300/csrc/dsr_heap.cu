@@ -742,13 +742,14 @@ struct MClone {
 // 32 items of 32 slots (one per warp and item queues up on the counter:
 // 6.7 M cars 160 -> 61 us).
 constexpr int DUMP_ITEMS = 4;   // items of a warp at a time (fewer in a short list)
-template <int MAXT>
+// WARPS: the CTA's, if known (the default's 8), else 0.
+template <int MAXT, int WARPS>
 __global__ void __launch_bounds__(MAXT) k_dump(const __grid_constant__ dsr_dev_heap H, int T, uint32_t* out,
                                                dsr_u64* count, dsr_u64 cap, int row) {
     extern __shared__ uint32_t stage[];  // [warps][32 * row]
     __shared__ uint32_t warp_n[MAXT / 32];
     __shared__ dsr_u64 cta_base;
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = WARPS ? WARPS : blockDim.x >> 5;
     const unsigned hsh = H.span_sh[T] - 5;
     const dsr_u64 items = (dsr_u64)(*(volatile uint32_t*)H.R_count) << hsh;
     const uint32_t nf = H.n_fields[T];
@@ -878,10 +879,12 @@ extern "C" int dsr_heap_dump(dsr_heap* h, int type, void* out_dev, uint64_t cap,
         kernel<<<(unsigned)grid, threads, smem, s>>>(h->dev, type, static_cast<uint32_t*>(out_dev),
                                                      static_cast<dsr_u64*>(count_dev), cap, row);
     };
-    if (threads <= 256)
-        run(k_dump<256>);
+    if (threads == 256)
+        run(k_dump<256, 8>);
+    else if (threads < 256)
+        run(k_dump<256, 0>);
     else
-        run(k_dump<1024>);
+        run(k_dump<1024, 0>);
     return dsr__check_launch("k_dump");
 }
 
