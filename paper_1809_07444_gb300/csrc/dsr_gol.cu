@@ -115,15 +115,10 @@ struct DDie : GolMethod<A> {
 template <class A>
 struct DBirth : GolMethod<A> {
     enum { kDefers = ALIVE, kDeferBack = 1 };
-    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const GolArgs& a, NoCtx, dsr_ref self,
+    static __device__ __forceinline__ unsigned run(const dsr_dev_heap& H, int, const GolArgs&, NoCtx, dsr_ref self,
                                                    dsr_later& later, dsr_no_acc&) {
         int idx;
-        if (birth(H, self, &idx)) {
-            if (later.on)
-                later.push((dsr_u64)idx);
-            else
-                gol_born(H, a, idx, dsr_new(H, ALIVE));
-        }
+        if (birth(H, self, &idx)) later.push((dsr_u64)idx);
         return 0;
     }
     static __device__ __forceinline__ void born(const dsr_dev_heap& H, const GolArgs& a, dsr_u64 idx, dsr_ref r) {
@@ -296,9 +291,9 @@ static int issue_generation(dsr_gol* g, cudaStream_t s) {
     return rc;
 }
 
-// A generation's three launches take a few microseconds each on a 64 x 64
-// board, so the generation is captured once into a CUDA graph (its kernel
-// arguments never change) and replayed: one launch per generation.
+// A generation's launches take a few microseconds each on a board of some
+// hundred cells a side, so the generation is captured once into a CUDA graph
+// (its kernel arguments never change) and replayed: one launch per generation.
 // Heaps up to this many blocks (a board of about 80 x 80 with the default heap)
 // run their generations in one cluster: 10 against 17 us a generation at 278
 // blocks, 13 and 18 at 580, 23 and 20 at 984.

@@ -825,8 +825,7 @@ __global__ void __launch_bounds__(F::THREADS, F::CTAS) k_force_sym(const __grid_
     Vec* part = sym_part(a.ws, Real(0));
     const Real eps2 = (Real)(a.p.eps * a.p.eps);
     const Real rn2 = (Real)(a.p.r_near * a.p.r_near);
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    (void)lane;
+    const unsigned warp = threadIdx.x >> 5;
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) next = atomicAdd(a.ws.work, 1u);

@@ -12,9 +12,9 @@
 //
 // A warp takes every W-th (block, 32 slots) item of the list, so that at any
 // time the grid works on neighbouring entries; a CTA of a group do-all that
-// creates takes one stretch, which lies in one or two heaps. A warp's 32 lanes load the entries of its next 32
-// items at once and hand them out by shuffle, so the list costs one round
-// trip per 32 items and warp, not one per item.
+// creates takes one stretch, which lies in one or two heaps. A warp's 32 lanes
+// load the entries of its next 32 items at once and hand them out by shuffle,
+// so the list costs one round trip per 32 items and warp, not one per item.
 //
 // Deferred work. A method may put off an object's creation: it pushes a
 // word, and the CTA later creates all pending objects together and calls
@@ -102,7 +102,6 @@ struct dsr_later {
     uint32_t* np;
     dsr_u64* pending;
     dsr_u64 tag;  // groups: heap index << 32
-    bool on;      // work is deferred
     __device__ __forceinline__ void push(dsr_u64 word) {
         const unsigned act = __activemask();
         const unsigned lane = dsr_lane();
@@ -374,7 +373,7 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
     const uint32_t end = kStretch ? (uint32_t)(cta < ctas ? items * (cta + 1) / ctas : 0) : (uint32_t)items;
     const uint32_t stride = kStretch ? warps : ctas * warps;
     const uint32_t cta0 = cta >= ctas ? end : kStretch ? (uint32_t)(items * cta / ctas) : cta * warps;
-    dsr_later later{nullptr, nullptr, 0, M::kDefers != DSR_NOTHING};
+    dsr_later later{nullptr, nullptr, 0};
     if constexpr (M::kDefers != DSR_NOTHING) {
         later.np = &sm->np;
         later.pending = sm->pending;
@@ -430,7 +429,8 @@ __device__ __forceinline__ void dsr_run_list(const Space& S, const dsr_phase& ph
                 }
             }
             if constexpr (M::kDefers != DSR_NOTHING) {
-                // the last thread to arrive sees every push: all decide alike
+                // the last to push reads the count after its own push, so a
+                // count above the half is seen by one at least: all decide alike
                 if (__syncthreads_or(*(volatile uint32_t*)&sm->np > kHalf)) {
                     if constexpr (M::kDefers >= 0)
                         dsr_create_pending<M, Space, MAXT>(S, a, cta, ctas, *sm, dsr_hash32(cta + k0 * 0x85EBCA77u));
@@ -627,15 +627,8 @@ int dsr__step(dsr_heap* h, const dsr_phase& p1, const dsr_phase& p2, const typen
     const bool small = threads <= 256;
     const void* k = small ? (const void*)dsr_step_kernel<M1, M2, END, F, 256>
                           : (const void*)dsr_step_kernel<M1, M2, END, F, 1024>;
-    static int grid_cache[17] = {0};  // as in dsr__doall
-    int grid;
-    if (h->tune.ctas_per_sm > 0) {
-        grid = dsr__persistent_grid(h, k, threads);
-    } else {
-        int& cached = grid_cache[threads / 64];
-        if (cached == 0) cached = dsr__persistent_grid(h, k, threads);
-        grid = cached;
-    }
+    static dsr_grid_cache cache;
+    int grid = dsr__tuned_grid(h, k, cache);
     const dsr_u64 most = (h->dev.M * 64 + threads - 1) / threads;
     if ((dsr_u64)grid > most) grid = (int)most;
     if (grid < 1) grid = 1;

@@ -18,7 +18,7 @@ constexpr uint32_t NO_CLAIM = 0xFFFFFFFFu;  // a claim word no mover holds (cell
 struct WatorInst {
     uint32_t* grid;    // 0 = empty, else (compact handle << 2) | kind (grid_word)
     uint32_t* claim;   // the lowest mover cell that claimed the cell this phase, or NO_CLAIM
-    uint32_t* intent;  // per object slot (intent_index): its chosen target, or NO_MOVE
+    uint32_t* intent;  // per object slot (intent_index): the direction it chose, or NO_MOVE
     dsr_u64 n_slots;   // entries of intent
     dsr_u64* step;     // device step counter (nullptr: unused batch slot)
     dsr_wator_params p;
@@ -92,7 +92,7 @@ __device__ __forceinline__ dsr_u64 step_key(const WatorInst& I, dsr_u64 stream) 
     return dsr_rand_key(I.p.seed, stream, *(volatile dsr_u64*)I.step);
 }
 
-// Births at once, where no do-all defers them (dsr_direct.cuh).
+// Births at once, in the list do-alls of dsr_parallel_do and of BitmapAlloc.
 struct NoDefer {
     template <class HP>
     __device__ __forceinline__ void moved(const HP& H) const {
@@ -105,8 +105,8 @@ struct Defer {
     unsigned& moves;
     __device__ __forceinline__ void moved(const dsr_dev_heap&) const { ++moves; }
     __device__ __forceinline__ bool defer(uint32_t c) const {
-        if (later.on) later.push(c);
-        return later.on;
+        later.push(c);
+        return true;
     }
 };
 
