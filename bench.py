@@ -799,13 +799,13 @@ SUGAR_SIDE = 4096
 def bench_sugarscape(steps=30, warmup=3):
     """Sugarscape (Fig. 6f) on a 4096 x 4096 torus, 10% of the cells holding
     an agent (1.68 M agents), L2 flushed before every step, CUDA events per
-    step. Object-updates: four do-alls visit every agent each step.
+    step. Object-updates: A1 and A2 run on every agent, A3 and A4 on the dead.
     Algorithmic bytes per agent per step: A1 reads x, y, vision (12) and the
     cells in sight (occupancy, capacity, harvest step: 6 bytes a cell, 4 x
     vision cells, vision 3.5 on average) and writes the intent (4); A2 reads
     six fields and the intent (28), writes sugar, age, dead (12) and its
-    cell's harvest step (capacity and step read, step written: 9); A3 and A4
-    read the dead flag (4 each)."""
+    cell's harvest step (capacity and step read, step written: 9). Per death:
+    A3 and A4 read x and y (8 each)."""
     import torch
     from paper_1809_07444_gb300 import workloads as WL
     from paper_1809_07444_gb300.apps import Sugarscape
@@ -826,16 +826,17 @@ def bench_sugarscape(steps=30, warmup=3):
     t = sum(a.elapsed_time(b) for a, b in evs) / 1e3
     ev1 = g.events()
     n = len(agents)
-    per_agent = (12 + 6 * 4 * 3.5 + 4) + (28 + 12 + 9) + 4 + 4
-    alg = n * per_agent * steps
+    d = [b - a for a, b in zip(ev0, ev1)]
+    deaths = d[1] + d[2]
+    per_agent = (12 + 6 * 4 * 3.5 + 4) + (28 + 12 + 9)
+    alg = n * per_agent * steps + 16 * deaths
     peak, peak_kind = _peaks()
     del g, flush
     torch.cuda.empty_cache()
-    d = [b - a for a, b in zip(ev0, ev1)]
     return {"workload": "sugarscape %dx%d, %d agents, steps %d-%d, L2 flushed before every step"
                         % (SUGAR_SIDE, SUGAR_SIDE, n, warmup + 1, warmup + steps),
             "ms_per_step": t * 1e3 / steps, "agent_steps_per_s": n * steps / t,
-            "object_updates_per_s": 4 * n * steps / t, "moves": d[0], "deaths": d[1] + d[2],
+            "object_updates_per_s": (2 * n * steps + 2 * deaths) / t, "moves": d[0], "deaths": deaths,
             "algorithmic_gbs": alg / t / 1e9, "hbm_frac": alg / t / 1e9 / peak, "peak_gbs": peak,
             "peak_kind": peak_kind, "launches_per_step": 5}
 

@@ -51,7 +51,8 @@ enum {
 };
 
 /* Event counters (dsr_heap_counters), cumulative since create or reset. */
-#define DSR_CTR_VISITS 0u  /* objects visited by do-all method kernels */
+#define DSR_CTR_VISITS 0u  /* objects visited by do-alls (sugarscape's A3 and A4: every agent, though their
+                              kernels see only the dead) */
 #define DSR_CTR_ALLOCS 1u  /* objects created by dsr_new */
 #define DSR_CTR_FREES 2u   /* objects deleted by dsr_delete */
 #define DSR_CTR_BLOCKS 3u  /* blocks taken from the free bitmap (slow path) */

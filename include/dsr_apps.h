@@ -42,8 +42,9 @@ int dsr_gol_workspace_bytes(int W, int H, size_t* out);
  * initial Alive objects inside the heap. */
 int dsr_gol_create(dsr_heap* heap, int W, int H, const void* alive0_dev, void* workspace_dev, void* stream,
                    dsr_gol** out);
-/* A small heap (up to 768 blocks, default threads and CTAs per SM) runs all
- * its generations in one launch of a thread-block cluster. Otherwise the
+/* A small heap (up to 768 blocks, default threads and CTAs per SM, no
+ * subtypes) runs all its generations in one launch of a thread-block cluster,
+ * where the device allows one of 16 CTAs. Otherwise the
  * first call captures one generation (its launches) into a CUDA graph on a
  * stream of its own; every generation is then one graph launch on `stream`.
  * Make the first call outside any stream capture. */
@@ -123,7 +124,8 @@ int dsr_wator_create(dsr_heap* heap, const dsr_wator_params* p, const void* kind
                      void* stream, dsr_wator** out);
 /* Advances n_steps steps on `stream` (each step: F1, F2, S0, S1, S2 as
  * do-alls). A small heap (up to 1024 blocks, default threads and CTAs per SM,
- * no phase timing) runs all n_steps in one launch of a thread-block cluster.
+ * no subtypes, no phase timing) runs all n_steps in one launch of a
+ * thread-block cluster, where the device allows one of 16 CTAs.
  * Otherwise a step is replayed from a CUDA graph of its launches that the
  * handle captures on first use on a private stream (one for untimed steps,
  * one for the current dsr_wator_phase_timing / _phase_select setting, which
@@ -267,7 +269,8 @@ int dsr_wator_batch_destroy(dsr_wator_batch* b);
  * the cube fall in the border cells), so that tiles of the all-pairs sum are
  * spatially compact: tiles far from a row skip the near test, and the near
  * field and the merge-partner search look only at the 27 cells around a
- * body. Every sum has a fixed order: a step is deterministic.
+ * body. Every sum has a fixed order: a step is deterministic. A step takes
+ * all bodies in the heap, which may be more than its handle placed there.
  * Workspace (dsr_nbody_workspace_bytes): the cell counts and offsets, the
  * sorted per-body arrays for all M * 64 slots of the heap (rounded up to
  * 1024), the partial sums of the all-pairs kernels (for up to 163,840
