@@ -285,13 +285,16 @@ static void cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, c
 
 bool dsr__cluster_fits(const dsr_heap* h, const void* kernel, dsr_per_device* known) {
     return known->get(h->device, [&] {
-        int n = 0;
+        int n = 0, current = h->device;
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
         cluster_config(&cfg, &attr, nullptr);
+        cudaGetDevice(&current);  // the question is about the heap's device
         const bool ok =
+            cudaSetDevice(h->device) == cudaSuccess &&
             cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+        cudaSetDevice(current);
         cudaGetLastError();
         return ok;
     });
